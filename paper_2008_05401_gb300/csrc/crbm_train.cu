@@ -4,17 +4,34 @@
 //   d loss/d theta = (2/M) sum_i (diff_i - C) [ sum_ij sigma(a^f_ij) v_(i+a)(j+b),
 //                                               sum_ij v_ij,  sum_ij sigma(a^f_ij) ]
 // (the W, v_bias, h_bias components; sum_i (diff_i - C) = 0 removes C's own
-// dependence on theta), then ADAM (Kingma & Ba 2014).  Everything is FP64.
+// dependence on theta), then ADAM (Kingma & Ba 2014).  Everything is FP64; the
+// sums of sigma run in 64-bit fixed point with FP64's spacing below 2.
 //
-// One CTA per training problem (the paper trains one CRBM per temperature):
-// minibatch steps depend on each other through the parameters, so a problem
-// runs its steps in order inside one CTA, with parameters, ADAM moments and
-// the row-sum tables of the current filters in shared memory; independent
-// problems fill the GPU side by side.  Per step: (1) row-sum tables of W,
-// (2) one warp per sample: F (warp reductions) and the hidden probabilities
-// sigma(a^f) kept in shared memory, then C and the loss, (3) one warp per
-// parameter, lanes over (sample, site): the gradient, (4) ADAM.
+// One cluster of CTAs per training problem (the paper trains one CRBM per
+// temperature): minibatch steps depend on each other through the parameters,
+// so a problem runs its steps in order, the samples of a minibatch divided
+// over the cluster's CTAs; independent problems fill the GPU side by side.
+// Every CTA keeps the parameters, ADAM moments and row-sum tables of the
+// current filters in its own shared memory and updates them alike (the same
+// additions in the same order), so that a step needs two cluster barriers:
+// after F of every sample (read from the owners' shared memory) and after the
+// CTAs' gradient sums.
+//
+// What bounds it: the FP64 pipe (a warp instruction holds its sub-partition's
+// pipe for about 64 cycles on GB300) and the serial chain of a step.  Hence:
+//   - the sum of log(1 + e^-|x|) of a warp's units is the log of their product
+//     (each factor in (1, 2]): one multiplication per unit instead of a log1p;
+//   - sigma goes to shared memory as round(2^52 sigma), and the gradient's
+//     sums over sites are exact integer additions off the FP64 pipe;
+//   - the bias corrections 1 / (1 - b^t) are taken for 32 steps at a time, one
+//     step per lane (a pow per thread and step was a third of the epoch);
+//   - the next minibatch's samples and targets are fetched during a step.
+// K = 2 5x5, L = 8, 10^4 samples, batch 20: 24 problems 9.0 ms per epoch
+// (one 512-thread CTA per problem, log1p and pow per unit and thread, FP64
+// gradient sums: 69.3 ms).
 #include <algorithm>
+
+#include <cooperative_groups.h>
 
 #include "crbm.h"
 #include "crbm_device.cuh"
@@ -24,21 +41,19 @@ namespace crbm {
 
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kTrainThreads = 512;
 constexpr int kTrainWarps = kTrainThreads / 32;
+constexpr int kMaxCluster = 8;             // portable cluster size
+constexpr int kMaxBatch = 64;
 constexpr size_t kSigBudget = 96 * 1024;   // shared memory for hidden probabilities
 
 struct TrainParams {
-  int n, batch;
+  int batch, per;                          // samples of a minibatch, of a CTA
   double lr, b1, b2, eps;
   crbm_train_problem pr[CRBM_TRAIN_MAX_PROBLEMS];
 };
-
-__device__ __forceinline__ double warp_sum64(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
 
 // Samples whose hidden probabilities fit the shared buffer at once.
 __host__ __device__ inline int sig_capacity(int K, int N) {
@@ -47,89 +62,183 @@ __host__ __device__ inline int sig_capacity(int K, int N) {
   return c < 1 ? 1 : (int)c;
 }
 
-// Hidden pre-activation of filter f at site (si, sj) of lattice v: h_bias^f
-// plus one row-sum table entry per kernel row (window of k bits, periodic).
-__device__ __forceinline__ double preact(const double* tab, double hb, int f, int k, int T, const int* codes) {
-  double x = hb;
-  for (int a = 0; a < k; ++a) x += tab[(f * k + a) * T + codes[a]];
-  return x;
+// Shared memory of a CTA that takes `per` samples of each minibatch of M
+// (offsets in bytes; 8-byte arrays first).
+struct TrainLayout {
+  int th, am, av, gr, tab, F, cw, tgt, spos, sprod, rbc, part, sig, ord, bits, total;
+};
+__host__ __device__ inline TrainLayout train_layout(int K, int k, int L, int M, int per) {
+  const int N = L * L, P = K * k * k + 1 + K, Wd = (N + 31) / 32, cap = sig_capacity(K, N);
+  TrainLayout y;
+  int o = 0;
+  auto take = [&](int bytes) {
+    const int at = o;
+    o += (bytes + 7) & ~7;
+    return at;
+  };
+  y.th = take(P * 8);
+  y.am = take(P * 8);
+  y.av = take(P * 8);
+  y.gr = take(P * 8);                                // this CTA's gradient sum
+  y.tab = take(K * k * (1 << k) * 8);
+  y.F = take(per * 8);
+  y.cw = take(per * 8);                              // (2/M)(diff_i - C)
+  y.tgt = take(2 * M * 8);                           // targets, this minibatch's and the next
+  y.spos = take((kMaxBatch > kTrainWarps ? kMaxBatch : kTrainWarps) * 8);
+  y.sprod = take((kMaxBatch > kTrainWarps ? kMaxBatch : kTrainWarps) * 8);
+  y.rbc = take(2 * 32 * 8);                          // 1 / (1 - b^t) of 32 steps
+  y.part = take(kTrainThreads * 8);                  // gradient partials
+  y.sig = take((per < cap ? per : cap) * K * N * 8);
+  y.ord = take(3 * M * 4);                           // visiting order of three minibatches
+  y.bits = take(2 * (per * Wd + 1) * 4);             // lattices (one word of padding each)
+  y.total = o;
+  return y;
 }
 
-__device__ __forceinline__ void window_codes(const uint32_t* v, const int* wrap, int L, int k, int si, int sj,
-                                             int (&codes)[kMaxk]) {
+__device__ __forceinline__ double warp_sum64(double v) {
 #pragma unroll
-  for (int a = 0; a < kMaxk; ++a) {
-    if (a >= k) break;
-    const int r = wrap[si + a] * L;
-    int c = 0;
-    for (int b = 0; b < k; ++b) c |= (int)site_bit(v, r + wrap[sj + b]) << b;
-    codes[a] = c;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
 }
 
-// Hidden probabilities sigma(a^f) of samples [i0, min(i1, i0 + cap)) into
-// sig[(i - i0)][f][s] (the buffer holds cap samples); with F != nullptr also
-// F(x_i) = -v_bias sum v - sum softplus(a^f) of every sample of [i0, i1).
-// One warp per sample.
-__device__ void hidden_pass(const uint32_t* vb, int Wd, const double* tab, const double* hbias, double vbias,
-                            int K, int k, int T, int L, const int* wrap, int i0, int i1, int cap, double* sig,
-                            double* F) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = L * L;
-  for (int i = i0 + warp; i < i1; i += kTrainWarps) {
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "n"(BYTES)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// Warps per sample of unit_pass for ns samples, and the hidden units (a
+// multiple of 32) each takes of the sample's K N.
+__device__ __forceinline__ int segments(int ns) { return ns >= kTrainWarps ? 1 : kTrainWarps / ns; }
+
+// Hidden units of samples [i0, i1): SEG warps per sample, lanes over its
+// units (f, site).  sig[(i - i0) K N + unit] = round(2^52 sigma(a)) of the
+// samples below i0 + cap; with WANT_F also, per (sample, segment), the sum of
+// max(a, 0) in spos and the product of 1 + e^-|a| in sprod (softplus a =
+// max(a, 0) + log(1 + e^-|a|)).  A product of up to 960 factors of at most 2
+// cannot overflow; longer segments take their lanes' logs first.
+template <bool WANT_F>
+__device__ void unit_pass(const uint32_t* vb, int Wd, const double* tab, const double* hbias, int K, int k, int T,
+                          int L, int i0, int i1, int cap, unsigned long long* sig, double* spos, double* sprod) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = L * L, U = K * N;
+  const int SEG = segments(i1 - i0), span = ((U + SEG - 1) / SEG + 31) & ~31;
+  for (int task = warp; task < (i1 - i0) * SEG; task += kTrainWarps) {
+    const int i = i0 + task / SEG, u0 = (task % SEG) * span, u1 = min(U, u0 + span);
     const uint32_t* v = vb + i * Wd;
     const bool keep = i - i0 < cap;
-    double sp = 0.0, ones = 0.0;
-    for (int s = lane; s < N; s += 32) {
-      const int si = s / L, sj = s - si * L;
-      int codes[kMaxk];
-      window_codes(v, wrap, L, k, si, sj, codes);
-      for (int f = 0; f < K; ++f) {
-        const double x = preact(tab, hbias[f], f, k, T, codes);
-        const double e = exp(-fabs(x));
-        sp += fmax(x, 0.0) + log1p(e);                           // softplus x
-        if (keep) sig[((size_t)(i - i0) * K + f) * N + s] = (x >= 0.0 ? 1.0 : e) / (1.0 + e);   // sigma(x)
+    double pos = 0.0, prod = 1.0;
+    for (int u = u0 + lane; u < u1; u += 32) {
+      const int f = u / N, s = u - f * N, si = s / L, sj = s - si * L;
+      double x = hbias[f];
+      for (int a = 0; a < k; ++a) {
+        const int r = si + a < L ? si + a : si + a - L;
+        x += tab[(f * k + a) * T + (int)row_window(v, L, r, sj, k)];
       }
-      ones += (double)site_bit(v, s);
+      const double e = exp(-fabs(x)), d = 1.0 + e;
+      if (keep) {
+        // 1 + sigma in [1, 2]: the FP64 addition rounds sigma to a multiple of 2^-52
+        const double y = 1.0 + (x >= 0.0 ? 1.0 : e) / d;
+        sig[(size_t)(i - i0) * U + u] = (unsigned long long)(__double_as_longlong(y) - __double_as_longlong(1.0));
+      }
+      if (WANT_F) {
+        pos += fmax(x, 0.0);
+        prod *= d;
+      }
     }
-    if (F) {
-      sp = warp_sum64(sp);
-      ones = warp_sum64(ones);
-      if (lane == 0) F[i] = -vbias * ones - sp;
+    if (WANT_F) {
+      if (span > 960) {
+        pos += log(prod);
+        prod = 1.0;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        pos += __shfl_xor_sync(kFull, pos, o);
+        prod *= __shfl_xor_sync(kFull, prod, o);
+      }
+      if (lane == 0) {
+        spos[task] = pos;
+        sprod[task] = prod;
+      }
     }
   }
+}
+
+__device__ __forceinline__ int count_ones(const uint32_t* v, int Wd) {
+  int c = 0;
+  for (int w = 0; w < Wd; ++w) c += __popc(v[w]);
+  return c;
 }
 
 __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __grid_constant__ TrainParams p) {
-  const crbm_train_problem& q = p.pr[blockIdx.x];
+  cg::cluster_group cl = cg::this_cluster();
+  const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const crbm_train_problem& q = p.pr[blockIdx.x / CL];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = q.K, k = q.k, L = q.L, N = L * L, T = 1 << k, Wd = (N + 31) / 32;
-  const int nW = K * k * k, P = nW + 1 + K, nlut = K * k * T;
-  const int M = p.batch, cap = sig_capacity(K, N);
+  const int nW = K * k * k, P = nW + 1 + K, nlut = K * k * T, U = K * N;
+  const int M = p.batch, per = p.per, cap = sig_capacity(K, N);
 
   extern __shared__ __align__(16) unsigned char smem[];
-  double* th = (double*)smem;              // P
-  double* am = th + P;                      // P
-  double* av = am + P;                      // P
-  double* gr = av + P;                      // P: gradient of the minibatch
-  double* tab = gr + P;                     // nlut
-  double* Fs = tab + nlut;                  // M
-  double* cw = Fs + M;                      // M: (2/M)(diff_i - C)
-  double* sig = cw + M;                     // min(M, cap) * K * N
-  uint32_t* vb = (uint32_t*)(sig + (size_t)min(M, cap) * K * N);   // M * Wd
-  int* wrap = (int*)(vb + M * Wd);          // 2L: x -> x mod L
+  const TrainLayout y = train_layout(K, k, L, M, per);
+  double* th = (double*)(smem + y.th);
+  double* am = (double*)(smem + y.am);
+  double* av = (double*)(smem + y.av);
+  double* gr = (double*)(smem + y.gr);
+  double* tab = (double*)(smem + y.tab);
+  double* Fs = (double*)(smem + y.F);
+  double* cw = (double*)(smem + y.cw);
+  double* tgt = (double*)(smem + y.tgt);
+  double* spos = (double*)(smem + y.spos);
+  double* sprod = (double*)(smem + y.sprod);
+  double* rbc = (double*)(smem + y.rbc);
+  double* part = (double*)(smem + y.part);
+  unsigned long long* sig = (unsigned long long*)(smem + y.sig);
+  int* ord = (int*)(smem + y.ord);
+  uint32_t* bits = (uint32_t*)(smem + y.bits);
+
+  const int nb = (q.n_samples + M - 1) / M;
+  const int mine = rank * per;                        // this CTA's samples of a minibatch start here
+  auto size_of = [&](int b) { return min(M, q.n_samples - b * M); };
+  // lattices of this CTA's samples and every sample's target of minibatch b,
+  // whose visiting order is in shared memory
+  auto fetch = [&](int b) {
+    const int Mb = size_of(b), ns = max(min(Mb, mine + per) - mine, 0), buf = b & 1;
+    const int* o = ord + (b % 3) * M;
+    uint32_t* dst = bits + buf * (per * Wd + 1);
+    for (int e = tid; e < ns * Wd; e += kTrainThreads) {
+      const int i = e / Wd, w = e - i * Wd;
+      cp_async<4>(dst + e, q.samples + (size_t)o[mine + i] * Wd + w);
+    }
+    for (int i = tid; i < Mb; i += kTrainThreads) cp_async<8>(tgt + buf * M + i, q.targets + o[i]);
+  };
+  auto fetch_order = [&](int b) {
+    for (int i = tid; i < size_of(b); i += kTrainThreads) cp_async<4>(ord + (b % 3) * M + i, q.order + (size_t)b * M + i);
+  };
 
   for (int i = tid; i < P; i += kTrainThreads) {
     th[i] = q.theta[i];
     am[i] = q.adam_m[i];
     av[i] = q.adam_v[i];
   }
-  for (int x = tid; x < 2 * L; x += kTrainThreads) wrap[x] = x < L ? x : x - L;
-  long long t = *q.adam_t;
+  if (tid < 2) bits[tid * (per * Wd + 1) + per * Wd] = 0u;
+  const long long t0 = *q.adam_t;
+  if (nb > 0) fetch_order(0);
+  if (nb > 1) fetch_order(1);
+  cp_async_wait();
   __syncthreads();
-  const int nb = (q.n_samples + M - 1) / M;
+  if (nb > 0) fetch(0);
+  cp_async_wait();
+  __syncthreads();
   for (int b = 0; b < nb; ++b) {
-    const int b0 = b * M, Mb = min(M, q.n_samples - b0);
-    // (1) row-sum tables of the current filters (bits summed in increasing b), samples
+    const int Mb = size_of(b), ns = max(min(Mb, mine + per) - mine, 0);
+    const uint32_t* vb = bits + (b & 1) * (per * Wd + 1);
+    const double* tg = tgt + (b & 1) * M;
+    // the next minibatch's data and the order of the one after it (waited for at the step's end)
+    if (b + 1 < nb) fetch(b + 1);
+    if (b + 2 < nb) fetch_order(b + 2);
+    // (1) row-sum tables of the current filters (bits summed in increasing b)
     for (int e = tid; e < nlut; e += kTrainThreads) {
       const int code = e % T, fa = e / T;
       double acc = 0.0;
@@ -137,110 +246,159 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __g
         if ((code >> bb) & 1) acc += th[fa * k + bb];
       tab[e] = acc;
     }
-    for (int e = tid; e < Mb * Wd; e += kTrainThreads) {
-      const int i = e / Wd, w = e - i * Wd;
-      vb[e] = q.samples[(size_t)q.order[b0 + i] * Wd + w];
+    if ((b & 31) == 0 && warp >= kTrainWarps - 2) {
+      // bias corrections of steps t0 + b + 1 .. t0 + b + 32, one per lane
+      const int which = warp - (kTrainWarps - 2);
+      rbc[which * 32 + lane] = 1.0 / (1.0 - pow(which == 0 ? p.b1 : p.b2, (double)(t0 + b + 1 + lane)));
     }
-    for (int i = tid; i < P; i += kTrainThreads) gr[i] = 0.0;
     __syncthreads();
     const double vbias = th[nW];
     const double* hbias = th + nW + 1;
-    // (2) F of every sample (and the hidden probabilities of the first chunk)
-    hidden_pass(vb, Wd, tab, hbias, vbias, K, k, T, L, wrap, 0, Mb, cap, sig, Fs);
+    // (2) F of this CTA's samples (and the hidden probabilities of the first chunk)
+    if (ns > 0) unit_pass<true>(vb, Wd, tab, hbias, K, k, T, L, 0, ns, cap, sig, spos, sprod);
     __syncthreads();
-    if (tid == 0) {
-      double C = 0.0;
-      for (int i = 0; i < Mb; ++i) C += q.targets[q.order[b0 + i]] - Fs[i];
-      C /= (double)Mb;
-      double loss = 0.0;
-      for (int i = 0; i < Mb; ++i) {
-        const double d = q.targets[q.order[b0 + i]] - Fs[i] - C;
-        loss += d * d;
-        cw[i] = (2.0 / (double)Mb) * d;
+    if (warp == 0) {
+      const int SEG = ns > 0 ? segments(ns) : 1;
+      for (int e = lane; e < ns * SEG; e += 32) spos[e] += log(sprod[e]);
+      __syncwarp();
+      for (int i = lane; i < ns; i += 32) {
+        double sp = 0.0;
+        for (int g = 0; g < SEG; ++g) sp += spos[i * SEG + g];
+        Fs[i] = -vbias * (double)count_ones(vb + i * Wd, Wd) - sp;
       }
-      if (q.losses) q.losses[b] = loss / (double)Mb;
+    }
+    cl.sync();
+    if (warp == 0) {
+      // C and the loss from every sample's F (from the owner's shared memory)
+      double diff[kMaxBatch / 32], sum = 0.0;
+#pragma unroll
+      for (int h = 0; h < kMaxBatch / 32; ++h) {
+        const int i = lane + 32 * h;
+        diff[h] = 0.0;
+        if (i < Mb) {
+          diff[h] = tg[i] - cl.map_shared_rank(Fs, i / per)[i % per];
+          sum += diff[h];
+        }
+      }
+      const double C = warp_sum64(sum) / (double)Mb;
+      double loss = 0.0;
+#pragma unroll
+      for (int h = 0; h < kMaxBatch / 32; ++h) {
+        const int i = lane + 32 * h;
+        const double d = diff[h] - C;
+        if (i < Mb) {
+          loss = fma(d, d, loss);
+          if (i >= mine && i < mine + ns) cw[i - mine] = (2.0 / (double)Mb) * d;
+        }
+      }
+      if (rank == 0 && q.losses) {
+        loss = warp_sum64(loss);
+        if (lane == 0) q.losses[b] = loss / (double)Mb;
+      }
     }
     __syncthreads();
-    // (3) gradient: chunks of samples whose probabilities are in shared memory;
-    // one warp per parameter, lanes over (sample, site), fixed reduction order
-    for (int i0 = 0; i0 < Mb; i0 += cap) {
-      const int i1 = min(Mb, i0 + cap);
+    // (3) this CTA's gradient sums, chunks of samples whose probabilities are
+    // in shared memory: thread (parameter, sample group), sites as integers,
+    // then cw_i times the sum in FP64; the groups' partials added in order
+    const int SG = max(1, min(ns, kTrainThreads / P));
+    const int pp = tid % P, sg = tid / P;
+    double acc = 0.0;
+    for (int i0 = 0; i0 < ns; i0 += cap) {
+      const int i1 = min(ns, i0 + cap);
       if (i0 > 0) {
         // the first pass kept the probabilities of the first chunk only: recompute this one
         __syncthreads();
-        hidden_pass(vb, Wd, tab, hbias, vbias, K, k, T, L, wrap, i0, i1, cap, sig, nullptr);
+        unit_pass<false>(vb, Wd, tab, hbias, K, k, T, L, i0, i1, cap, sig, nullptr, nullptr);
         __syncthreads();
       }
-      for (int pp = warp; pp < P; pp += kTrainWarps) {
-        double acc = 0.0;
-        if (pp < nW) {
-          const int f = pp / (k * k), ab = pp - f * k * k, a = ab / k, bb = ab - a * k;
-          for (int i = i0; i < i1; ++i) {
-            const uint32_t* v = vb + i * Wd;
-            const double* sg = sig + ((size_t)(i - i0) * K + f) * N;
-            double part = 0.0;
-            for (int s = lane; s < N; s += 32) {
-              const int si = s / L, sj = s - si * L;
-              if (site_bit(v, wrap[si + a] * L + wrap[sj + bb])) part += sg[s];
+      if (sg < SG) {
+        for (int i = i0 + sg; i < i1; i += SG) {
+          const uint32_t* v = vb + i * Wd;
+          const unsigned long long* sp = sig + (size_t)(i - i0) * U;
+          unsigned long long sum = 0ull;
+          if (pp < nW) {
+            const int f = pp / (k * k), ab = pp - f * k * k, a = ab / k, bb = ab - a * k;
+            sp += f * N;
+            for (int si = 0; si < L; ++si) {
+              // bit j of the window: v at (si + a, j + bb), periodic
+              const int r = si + a < L ? si + a : si + a - L;
+              const uint32_t lo = row_window(v, L, r, bb, L < 16 ? L : 16);
+              const uint32_t hi = L > 16 ? row_window(v, L, r, bb + 16 < L ? bb + 16 : bb + 16 - L, L - 16) : 0u;
+              const uint32_t win = lo | (hi << 16);
+#pragma unroll 8
+              for (int j = 0; j < L; ++j)
+                if ((win >> j) & 1u) sum += sp[si * L + j];
             }
-            acc = fma(cw[i], part, acc);
+          } else if (pp == nW) {
+            sum = (unsigned long long)count_ones(v, Wd) << 52;
+          } else {
+            sp += (pp - nW - 1) * N;
+            for (int s = 0; s < N; ++s) sum += sp[s];
           }
-        } else if (pp == nW) {
-          for (int i = i0; i < i1; ++i) {
-            const uint32_t* v = vb + i * Wd;
-            double part = 0.0;
-            for (int s = lane; s < N; s += 32) part += (double)site_bit(v, s);
-            acc = fma(cw[i], part, acc);
-          }
-        } else {
-          const int f = pp - nW - 1;
-          for (int i = i0; i < i1; ++i) {
-            const double* sg = sig + ((size_t)(i - i0) * K + f) * N;
-            double part = 0.0;
-            for (int s = lane; s < N; s += 32) part += sg[s];
-            acc = fma(cw[i], part, acc);
-          }
+          acc = fma(cw[i], (double)sum, acc);           // sum in units of 2^-52
         }
-        acc = warp_sum64(acc);
-        if (lane == 0) gr[pp] += acc;
       }
     }
+    if (sg < SG) part[sg * P + pp] = acc * 0x1p-52;
     __syncthreads();
-    // (4) ADAM
-    t += 1;
-    const double bc1 = 1.0 - pow(p.b1, (double)t), bc2 = 1.0 - pow(p.b2, (double)t);
-    for (int pp = tid; pp < P; pp += kTrainThreads) {
-      const double g = gr[pp];
-      const double m = p.b1 * am[pp] + (1.0 - p.b1) * g;
-      const double w = p.b2 * av[pp] + (1.0 - p.b2) * g * g;
-      am[pp] = m;
-      av[pp] = w;
-      th[pp] = th[pp] - p.lr * (m / bc1) / (sqrt(w / bc2) + p.eps);
+    for (int i = tid; i < P; i += kTrainThreads) {
+      double s = 0.0;
+      for (int g = 0; g < SG; ++g) s += part[g * P + i];
+      gr[i] = s;
     }
+    cl.sync();
+    // (4) the whole gradient (the CTAs' sums in rank order) and ADAM, alike in every CTA
+    const double rb1 = rbc[b & 31], rb2 = rbc[32 + (b & 31)];
+    for (int i = tid; i < P; i += kTrainThreads) {
+      double g = 0.0;
+      for (int r = 0; r < CL; ++r) g += cl.map_shared_rank(gr, r)[i];
+      const double m = p.b1 * am[i] + (1.0 - p.b1) * g;
+      const double w = p.b2 * av[i] + (1.0 - p.b2) * g * g;
+      am[i] = m;
+      av[i] = w;
+      th[i] = th[i] - p.lr * (m * rb1) / (sqrt(w * rb2) + p.eps);
+    }
+    cp_async_wait();
     __syncthreads();
   }
-  for (int i = tid; i < P; i += kTrainThreads) {
-    q.theta[i] = th[i];
-    q.adam_m[i] = am[i];
-    q.adam_v[i] = av[i];
+  if (rank == 0) {
+    for (int i = tid; i < P; i += kTrainThreads) {
+      q.theta[i] = th[i];
+      q.adam_m[i] = am[i];
+      q.adam_v[i] = av[i];
+    }
+    if (tid == 0) *q.adam_t = t0 + nb;
   }
-  if (tid == 0) *q.adam_t = t;
+  cl.sync();        // no CTA leaves while another may read its shared memory
+}
+
+// CTAs per problem: as many as the SMs allow side by side (the FP64 pipe of an
+// SM is what a step waits for, so two CTAs on one SM gain nothing), at most
+// the portable cluster size, and no more than leave the largest share of a
+// minibatch unchanged.
+int cluster_size(int n, int batch) {
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int most = std::max(1, std::min({kMaxCluster, sms / n, batch}));
+  const int per = (batch + most - 1) / most;
+  return (batch + per - 1) / per;
 }
 
 }  // namespace
 
+// Shared memory of a CTA that takes a whole minibatch (the most any launch needs).
 size_t train_smem_bytes(const crbm_train_problem& q, int batch) {
-  const size_t N = (size_t)q.L * q.L, P = (size_t)q.K * q.k * q.k + 1 + q.K;
-  const size_t nlut = (size_t)q.K * q.k * ((size_t)1 << q.k), Wd = (N + 31) / 32;
-  const size_t chunk = (size_t)std::min(batch, sig_capacity(q.K, (int)N));
-  return (4 * P + nlut + 2 * (size_t)batch + chunk * q.K * N) * 8 + (size_t)batch * Wd * 4 + 2 * (size_t)q.L * 4;
+  return (size_t)train_layout(q.K, q.k, q.L, batch, batch).total;
 }
 
 cudaError_t launch_train(const crbm_train_problem* pr, int n, int batch, double lr, double b1, double b2,
                          double eps, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
   TrainParams p;
-  p.n = n;
+  const int CL = cluster_size(n, batch);
   p.batch = batch;
+  p.per = (batch + CL - 1) / CL;
   p.lr = lr;
   p.b1 = b1;
   p.b2 = b2;
@@ -248,13 +406,22 @@ cudaError_t launch_train(const crbm_train_problem* pr, int n, int batch, double 
   size_t smem = 0;
   for (int i = 0; i < n; ++i) {
     p.pr[i] = pr[i];
-    const size_t b = train_smem_bytes(pr[i], batch);
-    if (b > smem) smem = b;
+    smem = std::max(smem, (size_t)train_layout(pr[i].K, pr[i].k, pr[i].L, batch, p.per).total);
   }
   cudaError_t e = cudaFuncSetAttribute(train_epoch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  train_epoch_kernel<<<n, kTrainThreads, smem, st>>>(p);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n * CL));
+  cfg.blockDim = dim3(kTrainThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)CL;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, train_epoch_kernel, p);
 }
 
 }  // namespace crbm

@@ -127,6 +127,45 @@ def test_algorithm1_with_pretraining_matches_oracle(ctx):
         np.testing.assert_allclose(hist[:, i], losses, rtol=1e-8, atol=1e-11)
 
 
+@pytest.mark.parametrize("n_problems,K,k,L,n,batch", [
+    (1, 2, 5, 8, 41, 20),      # cluster of 7 CTAs, a last minibatch of one sample
+    (1, 1, 2, 2, 9, 1),        # one sample per minibatch, the smallest lattice
+    (3, 2, 3, 17, 70, 64),     # the largest minibatch, windows wider than 16 columns
+    (2, 4, 3, 31, 9, 5),       # odd side, three chunks of probabilities for a CTA's sample at most
+    (80, 2, 3, 32, 20, 20),    # more problems than half the SMs: one CTA each, chunked, segments of 2048 units
+    (40, 8, 2, 12, 25, 10),    # K = 8, two or three CTAs per problem
+])
+def test_cluster_split_matches_oracle(ctx, n_problems, K, k, L, n, batch):
+    """The division of minibatches over a cluster's CTAs (samples per CTA,
+    warps per sample, chunks of probabilities) leaves the epoch's results.
+    Both sides round F (|F| below about N K) to a few units of 2^-52 |F|; a
+    gradient component is (2/M) sum_i (diff_i - C) S_i with 0 <= S_i <= N, so it
+    is off by eg = 2 N (4 2^-52 N K) whatever it cancels to, a moment m by the
+    same, v by 2 |g| eg, and an ADAM step by at most lr times m's relative error."""
+    import torch
+    from oracle import train
+    from paper_2008_05401_gb300 import trainer
+    v = wl.random_lattices(n, L, seed=L + n)
+    rng = np.random.default_rng(batch)
+    ts = [rng.normal(0.0, 3.0, n) for _ in range(n_problems)]
+    orders = [wl.epoch_order(n, 5, i) for i in range(n_problems)]
+    probs = [trainer.Problem.new(ctx, K, k, L, wl.init_train_params(K, k, seed=i)) for i in range(n_problems)]
+    x = torch.tensor(wl.pack_bits(v).view(np.int32), device="cuda:0")
+    losses = trainer.train_epochs(ctx, probs, [x] * n_problems, [torch.tensor(t, device="cuda:0") for t in ts],
+                                  [torch.tensor(o, device="cuda:0") for o in orders], batch)
+    N, steps = L * L, -(-n // batch)
+    eg = 2.0 * N * (4.0 * 2.0 ** -52 * N * K)
+    for i in {0, n_problems // 2, n_problems - 1}:
+        st = train.Adam.zeros(K * k * k + 1 + K)
+        th, ls = train.epoch(wl.init_train_params(K, k, seed=i), st, v, ts[i], orders[i], K, k, M=batch)
+        np.testing.assert_allclose(losses[i].cpu().numpy(), ls, rtol=1e-9, atol=1e-12)
+        assert np.all(np.abs(probs[i].m.cpu().numpy() - st.m) <= eg + 1e-9 * np.abs(st.m))
+        assert np.all(np.abs(probs[i].v.cpu().numpy() - st.v) <= 2.0 * np.sqrt(st.v / 0.001) * eg + 1e-9 * st.v)
+        step = 1e-3 * steps * np.minimum(2.0, 2.0 * eg / np.maximum(np.abs(st.m), 1e-300))
+        assert np.all(np.abs(probs[i].theta.cpu().numpy() - th) <= step + 1e-12)
+        assert int(probs[i].t.item()) == st.t == steps
+
+
 def test_train_rejects_bad_shapes(ctx):
     import torch
     from paper_2008_05401_gb300 import CrbmError, trainer
