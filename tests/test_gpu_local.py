@@ -155,3 +155,22 @@ def test_local_rejects_odd_ising_lattice(ctx):
     with pytest.raises(CrbmError):
         job.local_run(1)
     job.release()
+
+
+@pytest.mark.parametrize("n,cols,rho", [(1, 2, 0.5), (2, 3, 0.0), (17, 2, 0.6), (33, 3, 0.9), (34, 1, 0.99),
+                                        (130, 7, 0.8), (1500, 4, 0.97), (30000, 2, 0.9)])
+def test_autocorr_rounds_match_oracle(ctx, n, cols, rho):
+    """Lengths around the kernel's rounds of 32 lags and tiles of 16, windows
+    that close within the first round, in a later one or never, and a series
+    too long for shared memory.  Every G(t) is a sum of at most n FP64 products
+    (n 2^-53 of G(0) at most), added over at most W lags: below 1e-9 of tau."""
+    import torch
+    from oracle import autocorr
+    rng = np.random.default_rng(n)
+    x = rng.normal(size=(n, cols))
+    for t in range(1, n):
+        x[t] += rho * x[t - 1]
+    tau, win = ctx.autocorr(torch.tensor(x, device="cuda:0"))
+    t_ref, w_ref = autocorr.tau_int_columns(x)
+    np.testing.assert_array_equal(win, w_ref)
+    np.testing.assert_allclose(tau, t_ref, rtol=1e-9)
