@@ -18,6 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libcrbm.so")
 SOURCES = ["crbm_kernels.cu", "crbm_api.cu", "crbm_tempering.cu", "crbm_analysis.cu", "crbm_train.cu",
+           "crbm_sweep.cu",
            "crbm_step_ising_fp64_t256.cu",
            "crbm_step_ising_mixed_t256.cu",
            "crbm_step_tc.cu",

@@ -1097,20 +1097,28 @@ int crbm_local_run(crbm_ctx* ctx, int job_id, int64_t sweeps, int exchange, int 
   // with the exchange the Kitaev spectra must come from the FP64 stage
   const int prec = (j->kind == kIsing || exchange) ? (int)kFP64 : precision;
   cudaStream_t st = (cudaStream_t)cuda_stream;
+  const bool ising = j->kind == kIsing;
+  const JobDev xd = make_jobdev(ctx, *j);
+  auto launch = [&](int S, bool add) {
+    if (!ising) return launch_jobs(ctx, {job_id}, S, 1, add ? 1 : 0, prec, 3, st);
+    CK(launch_ising_sweeps(xd, S, add, st), "sweep launch");
+    return (int)CRBM_OK;
+  };
   if (!exchange) {
     int64_t left = sweeps;
     while (left > 0) {
       const int chunk = (int)(left < (1 << 20) ? left : (1 << 20));
-      if ((rc = launch_jobs(ctx, {job_id}, chunk, 1, 1, prec, 3, st))) return rc;
+      if ((rc = launch(chunk, true))) return rc;
       left -= chunk;
     }
   } else {
-    const JobDev xd = make_jobdev(ctx, *j);
     for (int64_t c = 0; c < sweeps; ++c) {
-      if ((rc = launch_jobs(ctx, {job_id}, 1, 1, 0, prec, 3, st))) return rc;
+      if ((rc = launch(1, false))) return rc;
       CK(launch_pt_exchange(xd, -1, false, st), "exchange launch");
     }
   }
+  // F of the final lattices (the Kitaev kernel ends with it)
+  if (ising && (rc = launch_jobs(ctx, {job_id}, 0, 1, 1, kFP64, 1, st))) return rc;
   j->step += (uint64_t)sweeps;
   j->stream = st;
   j->exact = (prec == kFP64);

@@ -48,6 +48,11 @@ cudaError_t launch_random_init(uint32_t* bits, int n_chains, int N, int Wd, uint
 // the cycle counter is x's step counter + step_offset; `advance` then adds
 // one to x's step counter.
 cudaError_t launch_pt_exchange(const JobDev& x, int step_offset, bool advance, cudaStream_t st);
+// S checkerboard Metropolis sweeps of the Ising job j (even L; crbm_sweep.cu),
+// then its step counter += S.  Leaves the lattices, accept counts, E, log pi
+// and observables of the last sweep; add: every sweep's observables join the
+// sums and the trace.  F is left to an evaluation of the final lattices.
+cudaError_t launch_ising_sweeps(const JobDev& j, int S, bool add, cudaStream_t st);
 // Integrated autocorrelation time of every column of a time-major
 // [n][n_series] device array (crbm_analysis.cu); tau and w are device arrays.
 cudaError_t launch_tau(const double* x, int n_series, long long n, double c, double* tau, long long* w,

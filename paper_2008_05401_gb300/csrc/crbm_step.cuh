@@ -26,7 +26,6 @@ struct ChainSm {
   double lpb, lppb;      // bounds on |log pi - FP64 path's log pi| (current, proposed)
   double otp[kNobs];
   double beta;
-  double thr[5];         // local Ising sweeps: e^{-beta dE} 2^32 for 0..4 unequal neighbours
   double logu;           // tensor-core kernel: log u of the current proposal's MH draw
   double cst, mgs;       // tensor-core kernel: the tile's constant margin terms, the
                          // current state's margin terms (both off the MH thread's path)
@@ -401,116 +400,91 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     return;
   }
 
-  if (AUX && prm.mode == 3) {
-    // local-update Metropolis sweeps (Sec. III, Sec. IV baselines)
+  if (AUX && KIND == kKitaev && prm.mode == 3) {
+    // local-update Metropolis sweeps (Sec. IV baseline; the Ising kind's are crbm_sweep.cu's)
     const unsigned long long step0 = *(volatile unsigned long long*)jb.step;
-    if (KIND == kIsing && g.active && g.r == 0) {
-      for (int u = 0; u < 5; ++u) {
-        const double dE = (2.0 * jb.J[0]) * (double)(4 - 2 * u);
-        ch.thr[u] = exp(-ch.beta * dE) * 0x1p32;
-      }
-    }
-    __syncthreads();
-    unsigned nacc = 0;
     for (int s = 0; s < prm.S; ++s) {
       const uint32_t step = (uint32_t)(step0 + (uint64_t)s);
-      if (KIND == kIsing) {
-        uint32_t* v = my + ch.cur * P;
-        nacc += ising_colour(jb, g, v, step, 0, ch.thr);
-        __syncthreads();
-        nacc += ising_colour(jb, g, v, step, 1, ch.thr);
-        __syncthreads();
-      } else {
-        // per chain group: every branch below is uniform in the group, and only
-        // the group synchronises (a short last tile has groups without a chain)
-        for (int n = 0; n < N; ++n) {
-          const uint32_t* v = my + ch.cur * P;
-          uint32_t* vp = my + (ch.cur ^ 1) * P;
-          for (int w = g.r; w < jb.Wd; w += g.tpc) vp[w] = v[w] ^ ((w == (n >> 5)) ? (1u << (n & 31)) : 0u);
-          grp_sync<MULTI>(g);
-          double kr[4] = {0.0, 0.0, 0.0, 0.0};
-          if (PREC == kMixed) {
-            kitaev_logpi_df<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, kr, jb.lc_edge > 0);
+      // per chain group: every branch below is uniform in the group, and only
+      // the group synchronises (a short last tile has groups without a chain)
+      for (int n = 0; n < N; ++n) {
+        const uint32_t* v = my + ch.cur * P;
+        uint32_t* vp = my + (ch.cur ^ 1) * P;
+        for (int w = g.r; w < jb.Wd; w += g.tpc) vp[w] = v[w] ^ ((w == (n >> 5)) ? (1u << (n & 31)) : 0u);
+        grp_sync<MULTI>(g);
+        double kr[4] = {0.0, 0.0, 0.0, 0.0};
+        if (PREC == kMixed) {
+          kitaev_logpi_df<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, kr, jb.lc_edge > 0);
+        } else {
+          double k3[3];
+          kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, k3, eps_st, jb.lc_edge > 0);
+          kr[0] = k3[0];
+          kr[1] = k3[1];
+          kr[2] = k3[2];
+        }
+        if (g.r == 0) {
+          const uint4 w = philox4x32_10_rk(make_uint4((uint32_t)(n >> 2), kTagLocal, step, g.cid), jb.rk);
+          const double logu = log(((double)pick(w, n & 3) + 0.5) * 0x1p-32);
+          const double logr = kr[0] - ch.lp;
+          ch.lpp = kr[0];
+          ch.lppb = kr[3];
+          ch.Ep = kr[1];
+          ch.otp[0] = kr[1]; ch.otp[1] = kr[1] * kr[1]; ch.otp[2] = kr[2];
+          ch.flag_rec = 0;
+          if (PREC == kFP64) {
+            ch.flag_acc = logu < logr;
           } else {
-            double k3[3];
-            kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, k3, eps_st, jb.lc_edge > 0);
-            kr[0] = k3[0];
-            kr[1] = k3[1];
-            kr[2] = k3[2];
+            const double M = ch.lppb + ch.lpb + 1e-12 * (fabs(ch.lpp) + fabs(ch.lp)) + 1e-300;
+            if (logr - logu > M) ch.flag_acc = 1;
+            else if (logu - logr > M) ch.flag_acc = 0;
+            else ch.flag_rec = 1;
           }
+        }
+        grp_sync<MULTI>(g);
+        if (PREC == kMixed && ch.flag_rec) {
+          // the FP64 eigen-stage of the proposal (and of the current lattice
+          // when its log-weight came from the df64 stage)
+          double k1v[3], k0v[3] = {0.0, 0.0, 0.0};
+          const bool redo_v = ch.lpb != 0.0;
+          kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, k1v, eps_st, jb.lc_edge > 0);
+          if (redo_v) kitaev_logpi64<MULTI>(g, v, jb.L, jb.J, ch.beta, wk, k0v, nullptr, jb.lc_edge > 0);
           if (g.r == 0) {
+            ch.lpp = k1v[0];
+            ch.lppb = 0.0;
+            ch.Ep = k1v[1];
+            ch.otp[0] = k1v[1]; ch.otp[1] = k1v[1] * k1v[1]; ch.otp[2] = k1v[2];
+            if (redo_v) {
+              ch.lp = k0v[0];
+              ch.lpb = 0.0;
+            }
             const uint4 w = philox4x32_10_rk(make_uint4((uint32_t)(n >> 2), kTagLocal, step, g.cid), jb.rk);
             const double logu = log(((double)pick(w, n & 3) + 0.5) * 0x1p-32);
-            const double logr = kr[0] - ch.lp;
-            ch.lpp = kr[0];
-            ch.lppb = kr[3];
-            ch.Ep = kr[1];
-            ch.otp[0] = kr[1]; ch.otp[1] = kr[1] * kr[1]; ch.otp[2] = kr[2];
-            ch.flag_rec = 0;
-            if (PREC == kFP64) {
-              ch.flag_acc = logu < logr;
-            } else {
-              const double M = ch.lppb + ch.lpb + 1e-12 * (fabs(ch.lpp) + fabs(ch.lp)) + 1e-300;
-              if (logr - logu > M) ch.flag_acc = 1;
-              else if (logu - logr > M) ch.flag_acc = 0;
-              else ch.flag_rec = 1;
-            }
-          }
-          grp_sync<MULTI>(g);
-          if (PREC == kMixed && ch.flag_rec) {
-            // the FP64 eigen-stage of the proposal (and of the current lattice
-            // when its log-weight came from the df64 stage)
-            double k1v[3], k0v[3] = {0.0, 0.0, 0.0};
-            const bool redo_v = ch.lpb != 0.0;
-            kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, k1v, eps_st, jb.lc_edge > 0);
-            if (redo_v) kitaev_logpi64<MULTI>(g, v, jb.L, jb.J, ch.beta, wk, k0v, nullptr, jb.lc_edge > 0);
-            if (g.r == 0) {
-              ch.lpp = k1v[0];
-              ch.lppb = 0.0;
-              ch.Ep = k1v[1];
-              ch.otp[0] = k1v[1]; ch.otp[1] = k1v[1] * k1v[1]; ch.otp[2] = k1v[2];
-              if (redo_v) {
-                ch.lp = k0v[0];
-                ch.lpb = 0.0;
-              }
-              const uint4 w = philox4x32_10_rk(make_uint4((uint32_t)(n >> 2), kTagLocal, step, g.cid), jb.rk);
-              const double logu = log(((double)pick(w, n & 3) + 0.5) * 0x1p-32);
-              ch.flag_acc = logu < ch.lpp - ch.lp;
-              ch.rec_mh += 1ull;
-            }
-            grp_sync<MULTI>(g);
-          }
-          if (ch.flag_acc) {
-            // the spectrum cache follows the lattice when the proposal's came from the FP64 stage
-            if (g.active && (PREC == kFP64 || ch.flag_rec))
-              for (int l = g.r; l < N; l += g.tpc) jb.eps[(size_t)g.c * N + l] = eps_st[l];
-            grp_sync<MULTI>(g);
-            if (g.r == 0) {
-              ch.cur ^= 1;
-              ch.lp = ch.lpp;
-              ch.lpb = ch.lppb;
-              ch.E = ch.Ep;
-              for (int o = 0; o < 3; ++o) ch.ot[o] = ch.otp[o];
-              ch.acc += 1ull;
-            }
+            ch.flag_acc = logu < ch.lpp - ch.lp;
+            ch.rec_mh += 1ull;
           }
           grp_sync<MULTI>(g);
         }
+        if (ch.flag_acc) {
+          // the spectrum cache follows the lattice when the proposal's came from the FP64 stage
+          if (g.active && (PREC == kFP64 || ch.flag_rec))
+            for (int l = g.r; l < N; l += g.tpc) jb.eps[(size_t)g.c * N + l] = eps_st[l];
+          grp_sync<MULTI>(g);
+          if (g.r == 0) {
+            ch.cur ^= 1;
+            ch.lp = ch.lpp;
+            ch.lpb = ch.lppb;
+            ch.E = ch.Ep;
+            for (int o = 0; o < 3; ++o) ch.ot[o] = ch.otp[o];
+            ch.acc += 1ull;
+          }
+        }
+        grp_sync<MULTI>(g);
       }
       // observables of the lattice after the sweep
-      double cn[2];
-      lattice_counts(jb, g, my + ch.cur * P, cn);
-      grp_reduce<2>(cn, g, scratch);
+      double cn[1] = {flux_count(jb, g, my + ch.cur * P)};
+      grp_reduce<1>(cn, g, scratch);
       if (g.active && g.r == 0) {
-        if (KIND == kIsing) {
-          const double E = -jb.J[0] * (double)(2 * N - 2 * (int)cn[1]);
-          const double M = 2.0 * cn[0] - (double)N;
-          ch.E = E;
-          ch.lp = -ch.beta * E;
-          ch.ot[0] = E; ch.ot[1] = E * E; ch.ot[2] = fabs(M); ch.ot[3] = M * M;
-        } else {
-          ch.ot[3] = cn[1] / (double)jb.nhex;
-        }
+        ch.ot[3] = cn[0] / (double)jb.nhex;
         if (prm.correct) {
           for (int o = 0; o < kNobs; ++o) ch.os[o] += ch.ot[o];
           trace_store(jb, g.c, step0 + (uint64_t)s, ch.E);
@@ -518,8 +492,6 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
       }
       __syncthreads();
     }
-    if (nacc) atomicAdd(&ch.acc, (unsigned long long)nacc);
-    __syncthreads();
     // FP64 free energy of the final lattices, then everything back to the job
     Tabs tb64 = tb;
     tb64.f64 = jb.f64;

@@ -75,6 +75,30 @@ def test_ising_local_matches_oracle(ctx, L, n, sweeps, exchange):
     job.release()
 
 
+@pytest.mark.parametrize("L,n,sweeps,exchange,J", [(6, 5, 3, False, 1.0), (10, 33, 2, True, -0.7), (12, 9, 3, False, -1.0),
+                                                   (14, 3, 3, False, 0.0), (18, 2, 2, True, 1.3), (24, 7, 2, False, 1.0),
+                                                   (30, 5, 2, False, 1.0), (96, 2, 2, False, 1.0), (160, 1, 2, False, -1.0),
+                                                   (256, 2, 2, True, 1.0)])
+def test_ising_sweep_words_match_oracle(ctx, L, n, sweeps, exchange, J):
+    """Sides whose rows straddle the packed words, several words per thread,
+    chains that share a warp, both signs of J and J = 0: lattices, flips, energies
+    and traces as the oracle's (its thresholds' margins checked by _compare)."""
+    from paper_2008_05401_gb300 import FP64, ISING
+    W, hb, vb = wl.gaussian_crbm(1, 2, 0.2, seed=L)
+    T = wl.ising_ladder(n, n, 0.3, 3.2)
+    bits0 = wl.pack_bits(wl.random_lattices(n, L, seed=L + 4))
+    ref = oracle_chains("ising", W, hb, vb, L, T, (J,), SEED, n, bits0)
+    tr = []
+    worst = _run_oracle(ref, sweeps, exchange, trace=tr)
+    mid = ctx.load_model(ISING, W, vb, hb)
+    job = ctx.new_job(mid, ISING, L, T, (J,), SEED, 0, bits0, FP64)
+    buf = job.set_trace(sweeps)
+    job.local_run(sweeps, exchange=exchange)
+    _compare(job, ref, worst)
+    np.testing.assert_array_equal(buf.cpu().numpy(), np.array(tr))
+    job.release()
+
+
 @pytest.mark.parametrize("L,n,sweeps,exchange,J", [(2, 6, 3, False, (1.0, 1.0, 1.0)),
                                                    (3, 5, 2, True, (0.8, 1.1, 1.3)),
                                                    (4, 4, 2, False, (1.0, 1.0, 1.0)),
