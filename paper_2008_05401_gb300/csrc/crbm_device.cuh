@@ -218,11 +218,11 @@ __device__ __forceinline__ void fwd_codes(const uint32_t* bits, int L, int N, in
 }
 
 // ------------------------------------------------ Bernoulli decisions
-// FP64: h = [u < sigma(x)], u = (w + 1/2) 2^-32 exactly (App. B.1 sampling).
+// FP64: h = [u < sigma(x)], u = (w + 1/2) 2^-32 exactly (App. B.1 sampling),
+// as u (1 + e^-x) < 1: no division on the FP64 pipe.
 __device__ __forceinline__ uint32_t decide64(double x, uint32_t w) {
-  const double p = 1.0 / (1.0 + exp(-x));
   const double u = ((double)w + 0.5) * 0x1p-32;
-  return u < p ? 1u : 0u;
+  return u * (1.0 + exp(-x)) < 1.0 ? 1u : 0u;
 }
 
 // Special-function-unit approximations (PTX ex2/rcp/lg2, flush-to-zero).
@@ -338,12 +338,6 @@ __device__ __forceinline__ void grp_reduce(double (&x)[NV], const Grp& g, double
   }
 }
 
-// grp_reduce for a warp-aligned group with scratch of its own (NV * tpc / 32
-// doubles), synchronising only the group: the same order of additions, the
-// result valid in the leader (r == 0).
-template <int NV, bool MULTI>
-__device__ __forceinline__ void grp_reduce_local(double (&x)[NV], const Grp& g, double* scratch);
-
 // Barrier of one chain's thread group (warp-aligned groups of 32 .. blockDim
 // threads): the CTA barrier when the group is the whole CTA, the warp's when it
 // is one warp, else a named barrier of its own (id 1 + group index; a CTA holds
@@ -381,29 +375,63 @@ __device__ __forceinline__ double grp_sum(double x, const Grp& g, double* scratc
   return s;
 }
 
-template <int NV, bool MULTI>
-__device__ __forceinline__ void grp_reduce_local(double (&x)[NV], const Grp& g, double* scratch) {
-  for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) x[v] += __shfl_xor_sync(kFull, x[v], o);
+// Sums of a free-energy pass: F's softplus sum -- FP64 (s), or for the FP32
+// pass the thread's sum as an integer in units of 2^-32 (fx: exact additions
+// off the FP64 pipe, each thread's conversion within 2^-33) with the data part
+// of its error bound (b) -- and the lattice counts.
+struct FreeSum {
+  double s;
+  long long fx;
+  float b;
+  int ones, pairs;
+};
+
+// Deterministic sum over a chain's group, valid in its leader (r == 0).
+// scratch: 3 doubles per warp of the CTA (MULTI: of the group, whose threads
+// alone synchronise; else every thread of the CTA calls).
+template <int PREC, bool MULTI>
+__device__ __forceinline__ void reduce_free(FreeSum& x, const Grp& g, double* scratch) {
+  const int span = g.tpc < 32 ? g.tpc : 32;
+  for (int o = 1; o < span; o <<= 1) {
+    if (PREC == kFP64) {
+      x.s += __shfl_xor_sync(kFull, x.s, o);
+    } else {
+      x.fx += __shfl_xor_sync(kFull, x.fx, o);
+      x.b += __shfl_xor_sync(kFull, x.b, o);
+    }
+    x.ones += __shfl_xor_sync(kFull, x.ones, o);
+    x.pairs += __shfl_xor_sync(kFull, x.pairs, o);
   }
   if (g.tpc > 32) {
-    const int warp = g.r >> 5;
-    if ((g.r & 31) == 0) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) scratch[warp * NV + v] = x[v];
+    const int warp = (MULTI ? g.r : (int)threadIdx.x) >> 5;
+    double* mine = scratch + 3 * warp;
+    if ((threadIdx.x & 31) == 0) {
+      if (PREC == kFP64) mine[0] = x.s;
+      else mine[0] = __longlong_as_double(x.fx);
+      ((float*)mine)[2] = x.b;
+      ((int*)mine)[3] = x.ones;
+      ((int*)mine)[4] = x.pairs;
     }
     grp_sync<MULTI>(g);
     if (g.r == 0) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        double s = 0.0;
-        for (int w = 0; w < g.tpc / 32; ++w) s += scratch[w * NV + v];
-        x[v] = s;
+      for (int w = 1; w < g.tpc / 32; ++w) {
+        const double* o = mine + 3 * w;
+        if (PREC == kFP64) x.s += o[0];
+        else x.fx += __double_as_longlong(o[0]);
+        x.b += ((const float*)o)[2];
+        x.ones += ((const int*)o)[3];
+        x.pairs += ((const int*)o)[4];
       }
     }
     grp_sync<MULTI>(g);
   }
+}
+
+// F (Eq. 13) from the group's sums.
+template <int PREC>
+__device__ __forceinline__ double free_value(double vb, const FreeSum& x) {
+  if (PREC == kFP64) return -vb * (double)x.ones - x.s;
+  return fma((double)x.fx, -0x1p-32, -vb * (double)x.ones);
 }
 
 // Deterministic block-wide sum, result returned to every thread.
@@ -487,22 +515,18 @@ __device__ __forceinline__ int lc_class(int j, int L, int e) {
   return j < e ? j : (j >= L - e ? e + (j - (L - e)) : 2 * e);
 }
 
-// FP64 pre-activation of filter f of an LCRBM at site n from the forward
-// codes m (computed with wrap): the window is cut at the open column edge
-// (bits b >= L - j dropped) and the table of the column's class is used.
-template <int kU>
-__device__ __forceinline__ double lc_preact64(const JobDev& jb, const double* f64, int f, const uint32_t (&m)[kU],
-                                              int n, int k, int T) {
-  const int L = jb.L, j = n % L;
+// FP64 pre-activation of filter f of an LCRBM at site n: the window is cut at
+// the open column edge (bits b >= L - j dropped) and the table of the column's
+// class is used.
+__device__ __forceinline__ double lc_preact64(const JobDev& jb, const double* f64, int f, const uint32_t* v, int n,
+                                              int k, int T) {
+  const int L = jb.L, i = n / L, j = n - i * L;
   const int base = (lc_class(j, L, jb.lc_edge) * jb.K + f) * k * T;
   const uint32_t keep = (j + k > L) ? ((1u << (L - j)) - 1u) : 0xFFFFFFFFu;
   double x = jb.hb[f];
-#pragma unroll
-  for (int a = 0; a < kU; ++a) {
-    if (a < k) {
-      const uint32_t code = (m[a] - (uint32_t)(a * T)) & keep;
-      x += f64[base + a * T + (int)code];
-    }
+  for (int a = 0; a < k; ++a) {
+    const int r = i + a < L ? i + a : i + a - L;
+    x += f64[base + a * T + (int)(row_window(v, L, r, j, k) & keep)];
   }
   return x;
 }
@@ -531,21 +555,50 @@ __device__ inline double lc_visible64(const JobDev& jb, const double* f64, const
 // ------------------------------------------------- hidden half-step
 // h^f_ij = [u < sigma(h_bias^f + sum_ab W^f_ab v_(i+a)(j+b))]  (Eq. B2, Eq. 12)
 // FP64 order (shared with the mixed path's recompute): h_bias, then kernel
-// rows a = 0..k-1.  KC, kC > 0 fix K and k at compile time (0: runtime).
-template <int PREC, int KC, int kC>
+// rows a = 0..k-1.
+// FP64 form: thread (filter, site), so that a warp's FP64 instructions (each
+// holds the sub-partition's pipe for about 64 cycles whatever its active
+// lanes) are full; the Philox block of four sites is drawn by each of them,
+// integer work beside it.  sync: the group's barrier.
+template <class SYNC>
+__device__ void hidden_phase64(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v, uint32_t* h, int P,
+                               uint32_t step, int sub, SYNC sync) {
+  const int L = jb.L, N = jb.N, K = jb.K, k = jb.k, T = tb.T;
+  if (g.active)
+    for (int w = g.r; w < K * P; w += g.tpc) h[w] = 0u;
+  sync();
+  if (!g.active) return;
+  for (int e = g.r; e < K * N; e += g.tpc) {
+    const int f = e / N, n = e - f * N, i = n / L, j = n - i * L;
+    double x = jb.hb[f];
+    if (jb.lc_edge) {
+      x = lc_preact64(jb, tb.f64, f, v, n, k, T);
+    } else {
+      for (int a = 0; a < k; ++a) {
+        const int r = i + a < L ? i + a : i + a - L;
+        x += tb.f64[(f * k + a) * T + row_window(v, L, r, j, k)];
+      }
+    }
+    const uint4 w = philox4x32_10_rk(make_uint4((uint32_t)(n >> 2), (uint32_t)(sub * (K + 1) + f), step, g.cid), jb.rk);
+    if (decide64(x, pick(w, n & 3))) atomicOr(h + f * P + (n >> 5), 1u << (n & 31));
+  }
+}
+
+// Mixed form: thread = unit of 4 sites.  KC, kC > 0 fix K and k at compile
+// time (0: runtime).
+template <int KC, int kC>
 __device__ void hidden_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v,
                              uint32_t* h, int P, uint32_t step, int sub, unsigned& nrec) {
   constexpr int kU = kC ? kC : kMaxk;
   const int L = jb.L, N = jb.N, K = KC ? KC : jb.K, k = kC ? kC : jb.k, T = tb.T;
   const int nblk = (N + 3) >> 2;
   const int iters = (nblk + g.tpc - 1) / g.tpc;
-  const uint32_t k0 = (uint32_t)jb.seed, k1 = (uint32_t)(jb.seed >> 32);
   for (int it = 0; it < iters; ++it) {
     const int q = g.r + it * g.tpc;
     const bool act = g.active && q < nblk;
     uint32_t m[4][kU];
     fwd_codes<kC>(v, L, N, k, T, act ? q : 0, m);
-    if (PREC == kMixed && KC == 4) {
+    if (KC == 4) {
       // all four filters per site from the filter-interleaved table
       uint4 w[4];
 #pragma unroll
@@ -589,28 +642,16 @@ __device__ void hidden_phase(const JobDev& jb, const Tabs& tb, const Grp& g, con
       uint32_t nib = 0;
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        uint32_t bit;
-        if (PREC == kFP64) {
-          double x = jb.hb[f];
-          if (KC == 0 && jb.lc_edge) {
-            x = lc_preact64<kU>(jb, tb.f64, f, m[t], (act && 4 * q + t < N) ? 4 * q + t : 0, k, T);
-          } else {
+        float x = jb.hb32[f];
 #pragma unroll
-            for (int a = 0; a < kU; ++a) if (kC || a < k) x += tb.f64[base + m[t][a]];
-          }
-          bit = decide64(x, pick(w, t));
-        } else {
-          float x = jb.hb32[f];
+        for (int a = 0; a < kU; ++a) if (kC || a < k) x += tb.fd[base + m[t][a]];
+        uint32_t bit = decide32(x, pick(w, t), jb.c0h, jb.c1);
+        if (bit == 2u) {
+          uint32_t mm[kMaxk];
 #pragma unroll
-          for (int a = 0; a < kU; ++a) if (kC || a < k) x += tb.fd[base + m[t][a]];
-          bit = decide32(x, pick(w, t), jb.c0h, jb.c1);
-          if (bit == 2u) {
-            uint32_t mm[kMaxk];
-#pragma unroll
-            for (int a = 0; a < kU; ++a) mm[a] = m[t][a];
-            bit = recompute_hidden(jb, f, mm, k, T, pick(w, t));
-            if (act && 4 * q + t < N) ++nrec;
-          }
+          for (int a = 0; a < kU; ++a) mm[a] = m[t][a];
+          bit = recompute_hidden(jb, f, mm, k, T, pick(w, t));
+          if (act && 4 * q + t < N) ++nrec;
         }
         if (act && 4 * q + t < N) nib |= bit << t;
       }
@@ -624,7 +665,35 @@ __device__ void hidden_phase(const JobDev& jb, const Tabs& tb, const Grp& g, con
 // The window of hidden row i - a starting at column j - (k-1) holds, as bit
 // k-1-b, the unit h_(i-a)(j-b); the backward tables are indexed by that raw
 // window.  Order: v_bias, then kernel rows a, then filters f.
-template <int PREC, int KC, int kC>
+// FP64 form: thread = site (see hidden_phase64).
+template <class SYNC>
+__device__ void visible_phase64(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* h, uint32_t* vp, int P,
+                                uint32_t step, int sub, SYNC sync) {
+  const int L = jb.L, N = jb.N, K = jb.K, k = jb.k, T = tb.T;
+  if (g.active)
+    for (int w = g.r; w < jb.Wd; w += g.tpc) vp[w] = 0u;
+  sync();
+  if (!g.active) return;
+  for (int n = g.r; n < N; n += g.tpc) {
+    double x = jb.vb;
+    if (jb.lc_edge) {
+      x = lc_visible64(jb, tb.f64, h, P, n, k, T);
+    } else {
+      const int i = n / L, j = n - i * L;
+      int c = j - (k - 1);
+      if (c < 0) c += L;
+      for (int a = 0; a < k; ++a) {
+        const int r = bwd_row(i, a, L);
+        for (int f = 0; f < K; ++f) x += tb.b64[(f * k + a) * T + row_window(h + f * P, L, r, c, k)];
+      }
+    }
+    const uint4 w = philox4x32_10_rk(make_uint4((uint32_t)(n >> 2), (uint32_t)(sub * (K + 1) + K), step, g.cid), jb.rk);
+    if (decide64(x, pick(w, n & 3))) atomicOr(vp + (n >> 5), 1u << (n & 31));
+  }
+}
+
+// Mixed form: thread = unit of 4 sites.
+template <int KC, int kC>
 __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* h,
                               uint32_t* vp, int P, uint32_t step, int sub, unsigned& nrec) {
   constexpr int kU = kC ? kC : kMaxk;
@@ -633,19 +702,14 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
   const uint32_t mk = (1u << k) - 1u;
   const int nblk = (N + 3) >> 2;
   const int iters = (nblk + g.tpc - 1) / g.tpc;
-  const uint32_t k0 = (uint32_t)jb.seed, k1 = (uint32_t)(jb.seed >> 32);
   const bool rows4 = (L & 3) == 0;
   for (int it = 0; it < iters; ++it) {
     const int q = g.r + it * g.tpc;
     const bool act = g.active && q < nblk;
     const int qq = act ? q : 0;
-    double x64[4];
     float x32[4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      x64[t] = jb.vb;
-      x32[t] = jb.vb32;
-    }
+    for (int t = 0; t < 4; ++t) x32[t] = jb.vb32;
     if (rows4) {
       const int n0 = 4 * qq, i = n0 / L, j0 = n0 - i * L;
       int c = j0 - (k - 1);
@@ -685,8 +749,7 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
 #pragma unroll
               for (int t = 0; t < 4; ++t) {
                 const uint32_t code = (win >> t) & mk;
-                if (PREC == kFP64) x64[t] += tb.b64[base + code];
-                else x32[t] += tb.bd[base + code];
+                x32[t] += tb.bd[base + code];
               }
             }
           }
@@ -705,17 +768,9 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
           for (int f = 0; f < K; ++f) {
             const uint32_t code = row_window(h + f * P, L, r, c, k);
             const int base = (f * k + a) * T;
-            if (PREC == kFP64) x64[t] += tb.b64[base + code];
-            else x32[t] += tb.bd[base + code];
+            x32[t] += tb.bd[base + code];
           }
         }
-      }
-    }
-    if (PREC == kFP64 && KC == 0 && jb.lc_edge) {
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int n = 4 * qq + t;
-        x64[t] = lc_visible64(jb, tb.f64, h, P, n < N ? n : 0, k, T);
       }
     }
     const uint4 w = philox4x32_10_rk(make_uint4((uint32_t)q, (uint32_t)(sub * (K + 1) + K), step, g.cid), jb.rk);
@@ -723,15 +778,10 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       if (act && 4 * q + t < N) {
-        uint32_t bit;
-        if (PREC == kFP64) {
-          bit = decide64(x64[t], pick(w, t));
-        } else {
-          bit = decide32(x32[t], pick(w, t), jb.c0v, jb.c1);
-          if (bit == 2u) {
-            bit = recompute_visible(jb, h, P, 4 * q + t, pick(w, t));
-            ++nrec;
-          }
+        uint32_t bit = decide32(x32[t], pick(w, t), jb.c0v, jb.c1);
+        if (bit == 2u) {
+          bit = recompute_visible(jb, h, P, 4 * q + t, pick(w, t));
+          ++nrec;
         }
         nib |= bit << t;
       }
@@ -742,18 +792,68 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
 
 // ------------------------------------------------- free energy + lattice sums
 // F(v) = -v_bias sum v - sum_{f,i,j} softplus(h_bias^f + (W^f * v)_ij)   (Eq. 13)
-// Per-thread partial sums: out[0] = sum softplus (FP64 order, or FP32 with
-// Kahan compensation), out[1] = data part of the FP32 error bound (mixed),
-// out[2] = number of ones, out[3] = number of unequal nearest-neighbour pairs
-// (Ising) or of hexagons with flux -1 (Kitaev).
-template <int PREC, int KC, int kC>
-__device__ void free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v,
-                           double (&out)[4]) {
+// Per-thread partial sums: softplus (FreeSum), the number of ones and of
+// unequal nearest-neighbour pairs (Ising) or of hexagons with flux -1 (Kitaev).
+// FP64 form: thread (filter, site); the log(1 + e^-|x|) of a thread's units are
+// the log of their product (factors in (1, 2], the log taken at least every 512).
+__device__ inline FreeSum free_phase64(const JobDev& jb, const double* f64, const Grp& g, const uint32_t* v) {
+  const int L = jb.L, N = jb.N, K = jb.K, k = jb.k, T = 1 << k;
+  FreeSum out = {0.0, 0ll, 0.0f, 0, 0};
+  if (!g.active) return out;
+  double prod = 1.0;
+  int held = 0;
+  for (int e = g.r; e < K * N; e += g.tpc) {
+    const int f = e / N, n = e - f * N, i = n / L, j = n - i * L;
+    double x = jb.hb[f];
+    if (jb.lc_edge) {
+      x = lc_preact64(jb, f64, f, v, n, k, T);
+    } else {
+      for (int a = 0; a < k; ++a) {
+        const int r = i + a < L ? i + a : i + a - L;
+        x += f64[(f * k + a) * T + row_window(v, L, r, j, k)];
+      }
+    }
+    out.s += fmax(x, 0.0);
+    prod *= 1.0 + exp(-fabs(x));
+    if (++held == 512) {
+      out.s += log(prod);
+      prod = 1.0;
+      held = 0;
+    }
+  }
+  if (held) out.s += log(prod);
+  for (int n = g.r; n < N; n += g.tpc) {
+    const int i = n / L, j = n - i * L, jr = j + 1 == L ? 0 : j + 1;
+    const uint32_t b0 = site_bit(v, n);
+    out.ones += (int)b0;
+    if (jb.kind == kIsing) {
+      out.pairs += (int)(b0 ^ site_bit(v, i * L + jr)) + (int)(b0 ^ site_bit(v, (i + 1 == L ? 0 : i + 1) * L + j));
+    } else if (!(jb.lc_edge && j + 1 == L)) {
+      // the hexagon of cell r holds the z-bonds r and r - e1 + e2 (with
+      // open columns the hexagons of column L-1 do not exist)
+      out.pairs += (int)(b0 ^ site_bit(v, (i == 0 ? L - 1 : i - 1) * L + jr));
+    }
+  }
+  return out;
+}
+
+// Bound on |F - F_fp64| of an FP32 free energy beyond the constant cst of
+// free_constant: the summed data terms and F's own rounding.
+__device__ __forceinline__ double free_bound(const FreeSum& x, double cst, double F) {
+  return ((double)x.b * 1.001 + cst) + 1e-12 * fabs(F);
+}
+// Per unit the special-function and table errors, per thread the fixed-point conversion.
+__device__ __forceinline__ double free_constant(const JobDev& jb, int tpc) {
+  return (double)jb.K * (double)jb.N * (1.5 * 0x1p-23 + (double)jb.csp) + (double)tpc * 0x1p-33;
+}
+
+// Mixed form: thread = unit of 4 sites, FP32 with Kahan compensation.
+template <int KC, int kC>
+__device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v) {
   constexpr int kU = kC ? kC : kMaxk;
   const int L = jb.L, N = jb.N, K = KC ? KC : jb.K, k = kC ? kC : jb.k, T = tb.T;
   const int nblk = (N + 3) >> 2;
   const int iters = (nblk + g.tpc - 1) / g.tpc;
-  double s64 = 0.0;
   float s32 = 0.0f, c32 = 0.0f, sabs = 0.0f, ssp = 0.0f;
   int ones = 0, pairs = 0;
   for (int it = 0; it < iters; ++it) {
@@ -762,7 +862,7 @@ __device__ void free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const
     if (!act) continue;
     uint32_t m[4][kU];
     fwd_codes<kC>(v, L, N, k, T, q, m);
-    if (PREC == kMixed && KC == 4) {
+    if (KC == 4) {
       float sp[4][4];
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
@@ -796,46 +896,30 @@ __device__ void free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const
     } else {
       for (int f = 0; f < K; ++f) {
         const int base = f * k * T;
-        if (PREC == kFP64) {
+        float sp[4];
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            if (4 * q + t < N) {
-              double x = jb.hb[f];
-              if (KC == 0 && jb.lc_edge) {
-                x = lc_preact64<kU>(jb, tb.f64, f, m[t], 4 * q + t, k, T);
-              } else {
+        for (int t = 0; t < 4; ++t) {
+          sp[t] = 0.0f;
+          if (4 * q + t < N) {
+            float xh = jb.hb_hi[f], xl = jb.hb_lo[f];
 #pragma unroll
-                for (int a = 0; a < kU; ++a) if (kC || a < k) x += tb.f64[base + m[t][a]];
+            for (int a = 0; a < kU; ++a) {
+              if (kC || a < k) {
+                xh += tb.fh[base + m[t][a]];
+                xl += tb.fl[base + m[t][a]];
               }
-              s64 += softplus64(x);
             }
+            const float x = xh + xl;
+            sp[t] = softplus32(x);
+            sabs += fabsf(x);
           }
-        } else {
-          float sp[4];
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            sp[t] = 0.0f;
-            if (4 * q + t < N) {
-              float xh = jb.hb_hi[f], xl = jb.hb_lo[f];
-#pragma unroll
-              for (int a = 0; a < kU; ++a) {
-                if (kC || a < k) {
-                  xh += tb.fh[base + m[t][a]];
-                  xl += tb.fl[base + m[t][a]];
-                }
-              }
-              const float x = xh + xl;
-              sp[t] = softplus32(x);
-              sabs += fabsf(x);
-            }
-          }
-          const float us = (sp[0] + sp[1]) + (sp[2] + sp[3]);
-          ssp += us;
-          const float y = us - c32;
-          const float tt = s32 + y;
-          c32 = (tt - s32) - y;
-          s32 = tt;
         }
+        const float us = (sp[0] + sp[1]) + (sp[2] + sp[3]);
+        ssp += us;
+        const float y = us - c32;
+        const float tt = s32 + y;
+        c32 = (tt - s32) - y;
+        s32 = tt;
       }
     }
 #pragma unroll
@@ -859,17 +943,15 @@ __device__ void free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const
       }
     }
   }
-  if (PREC == kFP64) {
-    out[0] = s64;
-    out[1] = 0.0;
-  } else {
-    out[0] = (double)s32;
-    // x rounding + ex2 argument: 2^-23 |x|; pairwise, Kahan and final add: 6 2^-24 sp;
-    // 1.001 covers the FP32 accumulation of these two sums themselves
-    out[1] = ((double)sabs * 0x1p-23 + (double)ssp * (6.0 * 0x1p-24)) * 1.001;
-  }
-  out[2] = (double)ones;
-  out[3] = (double)pairs;
+  FreeSum out;
+  out.s = 0.0;
+  out.fx = __float2ll_rn(s32 * 0x1p32f);
+  // x rounding + ex2 argument: 2^-23 |x|; pairwise, Kahan and final add: 6 2^-24 sp
+  // (free_bound's factor covers the FP32 accumulation of these two sums themselves)
+  out.b = sabs * 0x1p-23f + ssp * (6.0f * 0x1p-24f);
+  out.ones = ones;
+  out.pairs = pairs;
+  return out;
 }
 
 // --------------------------------------------------- Kitaev log-weight

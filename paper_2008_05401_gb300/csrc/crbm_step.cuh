@@ -16,6 +16,8 @@
 #include "crbm_local.cuh"
 #include "crbm_kernels.h"
 
+#include <type_traits>
+
 namespace crbm {
 
 struct ChainSm {
@@ -24,13 +26,14 @@ struct ChainSm {
   double os[kNobs];      // running sums
   double Fp, Bp, lpp, Ep;
   double lpb, lppb;      // bounds on |log pi - FP64 path's log pi| (current, proposed)
-  double otp[kNobs];
+  double cfp;            // Kitaev: c_f of the proposal
   double beta;
-  double logu;           // tensor-core kernel: log u of the current proposal's MH draw
-  double cst, mgs;       // tensor-core kernel: the tile's constant margin terms, the
-                         // current state's margin terms (both off the MH thread's path)
+  double logu;           // log u of the current proposal's MH draw
+  double cst, mgs;       // constant margin terms; tensor-core kernel: the current
+                         // state's margin terms (both off the MH thread's path)
   unsigned long long acc, rec, rec_mh;
-  int cur, flag_rec, flag_acc, onesp;   // onesp: set units of the proposal (tensor-core kernel)
+  int cur, flag_rec, flag_acc;
+  int onesp, pairsp;     // lattice counts of the proposal
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -45,39 +48,29 @@ __host__ __device__ inline size_t kitaev_work_bytes(int N) {
 }
 
 // The mixed path's FP64 free energy (rare), out of line to spare registers.
-static __device__ __noinline__ void free_energy64(const JobDev& jb, const Tabs& tb, const Grp& g,
-                                                  const uint32_t* v, double* out) {
-  double o[4];
-  free_phase<kFP64, 0, 0>(jb, tb, g, v, o);
-  for (int i = 0; i < 4; ++i) out[i] = o[i];
+static __device__ __noinline__ void free_energy64(const JobDev& jb, const Grp& g, const uint32_t* v, FreeSum* out) {
+  *out = free_phase64(jb, jb.f64, g, v);
 }
 
-// FP64 free energy, log pi, E and observables of chain c's lattice from the
-// group sums fo (Eq. 13 sums, magnetisation count, bond/vison count) and, for
-// the Kitaev kind, kr = (log pi, e, c_f) of its spectrum.
+// Observables of a lattice: Ising from E and the number of ones; Kitaev from
+// (e, c_f) of its spectrum and its count of hexagons with flux -1.
 template <int KIND>
-// Fb: bound on |F - F_fp64| of an FP32 free energy (0 for an FP64 one).
-__device__ inline void store_evaluation(const JobDev& jb, int c, double beta, const double* fo, const double* kr,
-                                        double Fb = 0.0) {
-  const int N = jb.N;
-  const double Fv = -jb.vb * fo[2] - fo[0];
-  double lp, E, ot[kNobs];
+__device__ __forceinline__ void observables(const JobDev& jb, double E, double cf, int ones, int flux,
+                                            double (&ot)[kNobs]) {
+  ot[0] = E;
+  ot[1] = E * E;
   if (KIND == kIsing) {
-    E = -jb.J[0] * (double)(2 * N - 2 * (int)fo[3]);
-    const double M = 2.0 * fo[2] - (double)N;
-    lp = -beta * E;
-    ot[0] = E; ot[1] = E * E; ot[2] = fabs(M); ot[3] = M * M;
+    const double M = (double)(2 * ones - jb.N);
+    ot[2] = fabs(M);
+    ot[3] = M * M;
   } else {
-    lp = kr[0];
-    E = kr[1];
-    ot[0] = kr[1]; ot[1] = kr[1] * kr[1]; ot[2] = kr[2]; ot[3] = fo[3] / (double)jb.nhex;
+    ot[2] = cf;
+    ot[3] = (double)flux / (double)jb.nhex;
   }
-  jb.F[c] = Fv;
-  jb.Fb[c] = Fb;
-  jb.Lb[c] = 0.0;
-  jb.logpi[c] = lp;
-  jb.Ephys[c] = E;
-  for (int o = 0; o < kNobs; ++o) jb.obs_t[(size_t)c * kNobs + o] = ot[o];
+}
+// Ising energy from the number of unequal nearest-neighbour pairs (2 N bonds).
+__device__ __forceinline__ double ising_energy(const JobDev& jb, int pairs) {
+  return -jb.J[0] * (double)(2 * jb.N - 2 * pairs);
 }
 
 // AUX = 0: the proposal loop (mode 0) only; AUX = 1: modes 1-3.  Two kernels,
@@ -233,21 +226,25 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     // evaluate F (FP64, or in the mixed path FP32 with its certified bound,
     // as after a mixed proposal), log pi and the observables (FP64) of the
     // current lattices
-    double fo[4];
-    if (PREC == kMixed) free_phase<PREC, KC, kC>(jb, tb, g, my, fo);
-    else free_energy64(jb, tb, g, my, fo);
-    grp_reduce<4>(fo, g, scratch);
+    FreeSum fs;
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, my);
+    else fs = free_phase64(jb, tb.f64, g, my);
+    reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
     if (KIND == kKitaev)
       kitaev_logpi64<MULTI>(g, my, jb.L, jb.J, g.active ? ch.beta : 1.0, wk, kr,
                      g.active ? jb.eps + (size_t)g.c * N : nullptr, jb.lc_edge > 0);
     if (g.active && g.r == 0) {
-      double Fb = 0.0;
-      if (PREC == kMixed) {
-        const double Fv = -jb.vb * fo[2] - fo[0];
-        Fb = fo[1] + (double)K * (double)N * (1.5 * 0x1p-23 + (double)jb.csp) + 1e-12 * fabs(Fv);
-      }
-      store_evaluation<KIND>(jb, g.c, ch.beta, fo, kr, Fb);
+      const double F = free_value<PREC>(jb.vb, fs);
+      const double E = KIND == kIsing ? ising_energy(jb, fs.pairs) : kr[1];
+      double ot[kNobs];
+      observables<KIND>(jb, E, kr[2], fs.ones, fs.pairs, ot);
+      jb.F[g.c] = F;
+      jb.Fb[g.c] = PREC == kMixed ? free_bound(fs, free_constant(jb, g.tpc), F) : 0.0;
+      jb.Lb[g.c] = 0.0;
+      jb.logpi[g.c] = KIND == kIsing ? -ch.beta * E : kr[0];
+      jb.Ephys[g.c] = E;
+      for (int o = 0; o < kNobs; ++o) jb.obs_t[(size_t)g.c * kNobs + o] = ot[o];
     }
     return;
   }
@@ -266,15 +263,18 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     uint32_t* h = my + 2 * P;
     const uint32_t* src = my;
     for (int sub = 0; sub < prm.g; ++sub) {
-      hidden_phase<PREC, KC, kC>(jb, tb, g, src, h, P, step, sub, nrec);
+      if constexpr (PREC == kMixed) hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec);
+      else hidden_phase64(jb, tb, g, src, h, P, step, sub, []() { __syncthreads(); });
       __syncthreads();
-      visible_phase<PREC, KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec);
+      if constexpr (PREC == kMixed) visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec);
+      else visible_phase64(jb, tb, g, h, vp, P, step, sub, []() { __syncthreads(); });
       __syncthreads();
       src = vp;
     }
-    double fo[4];
-    free_phase<PREC, KC, kC>(jb, tb, g, vp, fo);
-    grp_reduce<4>(fo, g, scratch);
+    FreeSum fs;
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp);
+    else fs = free_phase64(jb, tb.f64, g, vp);
+    reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
     if (KIND == kKitaev)
       kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, g.active ? ch.beta : 1.0, wk, kr,
@@ -283,21 +283,13 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     if (g.active)
       for (int w = g.r; w < jb.Wd; w += g.tpc) h[w] = xj.bits[(size_t)g.c * jb.Wd + w];
     if (g.active && g.r == 0) {
-      ch.Fp = -jb.vb * fo[2] - fo[0];
-      ch.Bp = (PREC == kMixed)
-                  ? fo[1] + (double)K * (double)N * (1.5 * 0x1p-23 + (double)jb.csp) + 1e-12 * fabs(ch.Fp)
-                  : 0.0;
-      if (KIND == kIsing) {
-        const double E = -jb.J[0] * (double)(2 * N - 2 * (int)fo[3]);
-        const double M = 2.0 * fo[2] - (double)N;
-        ch.Ep = E;
-        ch.lpp = -ch.beta * E;
-        ch.otp[0] = E; ch.otp[1] = E * E; ch.otp[2] = fabs(M); ch.otp[3] = M * M;
-      } else {
-        ch.Ep = kr[1];
-        ch.lpp = kr[0];
-        ch.otp[0] = kr[1]; ch.otp[1] = kr[1] * kr[1]; ch.otp[2] = kr[2]; ch.otp[3] = fo[3] / (double)jb.nhex;
-      }
+      ch.Fp = free_value<PREC>(jb.vb, fs);
+      ch.Bp = PREC == kMixed ? free_bound(fs, free_constant(jb, g.tpc), ch.Fp) : 0.0;
+      ch.Ep = KIND == kIsing ? ising_energy(jb, fs.pairs) : kr[1];
+      ch.lpp = KIND == kIsing ? -ch.beta * ch.Ep : kr[0];
+      ch.cfp = kr[2];
+      ch.onesp = fs.ones;
+      ch.pairsp = fs.pairs;
       ch.F = xj.F[g.c];
       ch.Fb = xj.Fb[g.c];
       ch.lp = xj.logpi[g.c];
@@ -319,24 +311,21 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
       const int need = __syncthreads_or(g.active && g.r == 0 && ch.flag_rec);
       if (need) {
         // FP64 free energies of y' and (when only its FP32 value is known) of x
-        Tabs tb64g = tb;
-        tb64g.f64 = jb.f64;
-        tb64g.b64 = jb.b64;
         Grp g2 = g;
         g2.active = g.active && ch.flag_rec;
-        double f1[4];
-        free_energy64(jb, tb64g, g2, vp, f1);
-        grp_reduce<4>(f1, g2, scratch);
+        FreeSum f1;
+        free_energy64(jb, g2, vp, &f1);
+        reduce_free<kFP64, false>(f1, g2, scratch);
         Grp g3 = g2;
         g3.active = g2.active && ch.Fb != 0.0;
-        double f2[4];
-        free_energy64(jb, tb64g, g3, h, f2);
-        grp_reduce<4>(f2, g3, scratch);
+        FreeSum f2;
+        free_energy64(jb, g3, h, &f2);
+        reduce_free<kFP64, false>(f2, g3, scratch);
         if (g2.active && g.r == 0) {
-          ch.Fp = -jb.vb * f1[2] - f1[0];
+          ch.Fp = free_value<kFP64>(jb.vb, f1);
           ch.Bp = 0.0;
           if (g3.active) {
-            ch.F = -jb.vb * f2[2] - f2[0];
+            ch.F = free_value<kFP64>(jb.vb, f2);
             ch.Fb = 0.0;
           }
           const double loga = (ch.lpp - ch.lp) + (ch.Fp - ch.F);
@@ -370,6 +359,8 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         }
       }
       if (g.r == 0) {
+        double otp[kNobs];
+        observables<KIND>(jb, ch.Ep, ch.cfp, ch.onesp, ch.pairsp, otp);
         if (sw) {
           // the RBM slot takes x (read before the physical slot is overwritten)
           jb.F[c] = ch.F;
@@ -383,7 +374,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
           xj.Lb[c] = 0.0;
           xj.logpi[c] = ch.lpp;
           xj.Ephys[c] = ch.Ep;
-          for (int o = 0; o < kNobs; ++o) xj.obs_t[c * kNobs + o] = ch.otp[o];
+          for (int o = 0; o < kNobs; ++o) xj.obs_t[c * kNobs + o] = otp[o];
           xj.acc[c] += 1ull;
         } else {
           jb.F[c] = ch.Fp;
@@ -391,7 +382,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
           jb.Lb[c] = 0.0;
           jb.logpi[c] = ch.lpp;
           jb.Ephys[c] = ch.Ep;
-          for (int o = 0; o < kNobs; ++o) jb.obs_t[c * kNobs + o] = ch.otp[o];
+          for (int o = 0; o < kNobs; ++o) jb.obs_t[c * kNobs + o] = otp[o];
         }
         jb.rec[2 * c] += ch.rec;
         jb.rec[2 * c + 1] += ch.rec_mh;
@@ -429,7 +420,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
           ch.lpp = kr[0];
           ch.lppb = kr[3];
           ch.Ep = kr[1];
-          ch.otp[0] = kr[1]; ch.otp[1] = kr[1] * kr[1]; ch.otp[2] = kr[2];
+          ch.cfp = kr[2];
           ch.flag_rec = 0;
           if (PREC == kFP64) {
             ch.flag_acc = logu < logr;
@@ -452,7 +443,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
             ch.lpp = k1v[0];
             ch.lppb = 0.0;
             ch.Ep = k1v[1];
-            ch.otp[0] = k1v[1]; ch.otp[1] = k1v[1] * k1v[1]; ch.otp[2] = k1v[2];
+            ch.cfp = k1v[2];
             if (redo_v) {
               ch.lp = k0v[0];
               ch.lpb = 0.0;
@@ -474,7 +465,9 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
             ch.lp = ch.lpp;
             ch.lpb = ch.lppb;
             ch.E = ch.Ep;
-            for (int o = 0; o < 3; ++o) ch.ot[o] = ch.otp[o];
+            ch.ot[0] = ch.Ep;
+            ch.ot[1] = ch.Ep * ch.Ep;
+            ch.ot[2] = ch.cfp;
             ch.acc += 1ull;
           }
         }
@@ -493,17 +486,14 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
       __syncthreads();
     }
     // FP64 free energy of the final lattices, then everything back to the job
-    Tabs tb64 = tb;
-    tb64.f64 = jb.f64;
-    tb64.b64 = jb.b64;
-    double fo[4];
-    free_energy64(jb, tb64, g, my + ch.cur * P, fo);
-    grp_reduce<4>(fo, g, scratch);
+    FreeSum fs;
+    free_energy64(jb, g, my + ch.cur * P, &fs);
+    reduce_free<kFP64, false>(fs, g, scratch);
     if (g.active) {
       const uint32_t* v = my + ch.cur * P;
       for (int w = g.r; w < jb.Wd; w += g.tpc) jb.bits[(size_t)g.c * jb.Wd + w] = v[w];
       if (g.r == 0) {
-        jb.F[g.c] = -jb.vb * fo[2] - fo[0];
+        jb.F[g.c] = free_value<kFP64>(jb.vb, fs);
         jb.Fb[g.c] = 0.0;
         jb.Lb[g.c] = ch.lpb;
         jb.logpi[g.c] = ch.lp;
@@ -528,14 +518,36 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     if (KIND == kKitaev && MULTI) grp_sync<MULTI>(g);
     else __syncthreads();
   };
-  auto loop_reduce4 = [&](double (&x)[4], const Grp& gg) {
-    if (KIND == kKitaev && MULTI) grp_reduce_local<4, MULTI>(x, gg, wk.sc);
-    else grp_reduce<4>(x, gg, scratch);
+  auto loop_reduce = [&](FreeSum& x, const Grp& gg, auto prec) {
+    reduce_free<decltype(prec)::value, KIND == kKitaev && MULTI>(x, gg, KIND == kKitaev && MULTI ? wk.sc : scratch);
   };
-  const uint32_t k0 = (uint32_t)jb.seed, k1 = (uint32_t)(jb.seed >> 32);
   // the step counter lives in device memory (advanced by advance_steps after
   // the launch), so a captured CUDA graph can be replayed
   const unsigned long long step0 = *(volatile unsigned long long*)jb.step;
+  // What follows a decision (the accepted state's values, the running sums)
+  // and the next proposal's log u are left to the group's last thread, which
+  // takes them beside the hidden half-step: a single thread's FP64 instructions
+  // hold their sub-partition's pipe as long as a full warp's, and the leader's
+  // would hold up the whole group.
+  const bool clerk = g.active && g.r == g.tpc - 1;
+  auto settle = [&](unsigned long long t) {
+    if (ch.flag_acc) {
+      ch.F = ch.Fp;
+      ch.Fb = ch.Bp;
+      ch.lp = ch.lpp;
+      ch.lpb = ch.lppb;
+      ch.E = ch.Ep;
+      observables<KIND>(jb, ch.Ep, ch.cfp, ch.onesp, ch.pairsp, ch.ot);
+      ch.acc += 1ull;
+    }
+    for (int o = 0; o < kNobs; ++o) ch.os[o] += ch.ot[o];
+    trace_store(jb, g.c, t, ch.E);
+  };
+  auto accept_word = [&](uint32_t step) {
+    return philox4x32_10_rk(make_uint4(0u, kTagAcc, step, g.cid), jb.rk).x;
+  };
+  auto log_u64 = [&](uint32_t step) { return log(((double)accept_word(step) + 0.5) * 0x1p-32); };
+  if (PREC == kMixed && g.active && g.r == 0) ch.cst = free_constant(jb, g.tpc);
   for (int s = 0; s < prm.S; ++s) {
     const uint32_t step = (uint32_t)(step0 + (uint64_t)s);
     const int cur = ch.cur;
@@ -543,16 +555,24 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     uint32_t* vp = my + (cur ^ 1) * P;
     uint32_t* h = my + 2 * P;
     const uint32_t* src = v;
+    if (clerk) {
+      if (s > 0) settle(step0 + (uint64_t)(s - 1));
+      // mixed: in FP32, within 2^-20 (1 + |log u|), a term of the decision's margin
+      if (prm.correct) ch.logu = PREC == kFP64 ? log_u64(step) : (double)log_u32(accept_word(step));
+    }
     for (int sub = 0; sub < prm.g; ++sub) {
-      hidden_phase<PREC, KC, kC>(jb, tb, g, src, h, P, step, sub, nrec);
+      if constexpr (PREC == kMixed) hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec);
+      else hidden_phase64(jb, tb, g, src, h, P, step, sub, loop_sync);
       loop_sync();
-      visible_phase<PREC, KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec);
+      if constexpr (PREC == kMixed) visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec);
+      else visible_phase64(jb, tb, g, h, vp, P, step, sub, loop_sync);
       loop_sync();
       src = vp;
     }
-    double fo[4];
-    free_phase<PREC, KC, kC>(jb, tb, g, vp, fo);
-    loop_reduce4(fo, g);
+    FreeSum fs;
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp);
+    else fs = free_phase64(jb, tb.f64, g, vp);
+    loop_reduce(fs, g, std::integral_constant<int, PREC>());
     double kr[4] = {0.0, 0.0, 0.0, 0.0};
     if (KIND == kKitaev) {
       if (PREC == kMixed) {
@@ -565,49 +585,53 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         kr[2] = k3[2];
       }
     }
-    double logu = 0.0;
     if (g.active && g.r == 0) {
-      if (KIND == kIsing) {
-        const double E = -jb.J[0] * (double)(2 * N - 2 * (int)fo[3]);
-        const double M = 2.0 * fo[2] - (double)N;
-        ch.Ep = E;
-        ch.lpp = -ch.beta * E;
-        ch.otp[0] = E; ch.otp[1] = E * E; ch.otp[2] = fabs(M); ch.otp[3] = M * M;
-      } else {
-        ch.Ep = kr[1];
-        ch.lpp = kr[0];
-        ch.otp[0] = kr[1]; ch.otp[1] = kr[1] * kr[1]; ch.otp[2] = kr[2]; ch.otp[3] = fo[3] / (double)jb.nhex;
-      }
+      const double E = KIND == kIsing ? ising_energy(jb, fs.pairs) : kr[1];
+      const double lpp = KIND == kIsing ? -ch.beta * E : kr[0];
+      const double Fp = free_value<PREC>(jb.vb, fs);
+      ch.Ep = E;
+      ch.lpp = lpp;
+      ch.cfp = kr[2];
+      ch.onesp = fs.ones;
+      ch.pairsp = fs.pairs;
       ch.lppb = kr[3];
-      ch.Fp = -jb.vb * fo[2] - fo[0];
-      ch.Bp = (PREC == kMixed)
-                  ? fo[1] + (double)K * (double)N * (1.5 * 0x1p-23 + (double)jb.csp) + 1e-12 * fabs(ch.Fp)
-                  : 0.0;
+      ch.Fp = Fp;
+      ch.Bp = PREC == kMixed ? free_bound(fs, ch.cst, Fp) : 0.0;
       ch.flag_rec = 0;
       if (!prm.correct) {
         ch.flag_acc = 1;
       } else {
-        const double logr = (ch.lpp - ch.lp) + (ch.Fp - ch.F);
-        const uint4 w = philox4x32_10_rk(make_uint4(0u, kTagAcc, step, g.cid), jb.rk);
-        logu = log(((double)w.x + 0.5) * 0x1p-32);
+        const double logu = ch.logu, logr = (lpp - ch.lp) + (Fp - ch.F);
         if (PREC == kFP64) {
           ch.flag_acc = logu < logr;
         } else {
           const double M = ch.Bp + ch.Fb + ch.lppb + ch.lpb +
-                           1e-12 * (fabs(ch.lpp) + fabs(ch.lp) + fabs(ch.Fp) + fabs(ch.F)) + 1e-300;
+                           1e-12 * (fabs(lpp) + fabs(ch.lp) + fabs(Fp) + fabs(ch.F)) +
+                           0x1p-20 * (1.0 + fabs(logu)) + 1e-300;
           if (logr - logu > M) ch.flag_acc = 1;
           else if (logu - logr > M) ch.flag_acc = 0;
           else ch.flag_rec = 1;
         }
       }
+      if (!ch.flag_rec && ch.flag_acc) ch.cur ^= 1;
     }
-    if (PREC == kMixed && KIND == kIsing) {
-      // second level: F of v' (and of v when only an FP32 value of it is
-      // known) with df64 softplus (bound ~1e-7); flag_rec = 2 sends a decision
-      // that still straddles the threshold on to the FP64 path's code below
-      if (__syncthreads_or(g.active && g.r == 0 && ch.flag_rec)) {
-        Grp g2 = g;
-        g2.active = g.active && ch.flag_rec;
+    int need = 0;
+    if (PREC == kMixed && !(KIND == kKitaev && MULTI)) {
+      need = __syncthreads_or(g.active && g.r == 0 && ch.flag_rec);
+    } else {
+      loop_sync();                 // the leader's decision, read by its whole group
+      if (PREC == kMixed) need = g.active && ch.flag_rec;
+    }
+    if (PREC == kMixed && need) {
+      // the chains (several per CTA: some of them) whose margin straddled the threshold
+      Grp g2 = g;
+      g2.active = g.active && ch.flag_rec != 0;
+      loop_sync();
+      const bool mine = g2.active && g.r == 0;
+      if (KIND == kIsing) {
+        // second level: F of v' (and of v when only an FP32 value of it is
+        // known) with df64 softplus (bound ~1e-7); flag_rec = 2 sends a decision
+        // that still straddles the threshold on to the FP64 path's code below
         Grp g3 = g2;
         g3.active = g2.active && ch.Fb != 0.0;
         double f1[3], f2[3];
@@ -615,7 +639,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         grp_reduce<3>(f1, g2, scratch);
         free_sum_df<KC ? KC : kMaxK>(jb, g3, v, f2);
         grp_reduce<3>(f2, g3, scratch);
-        if (g2.active && g.r == 0) {
+        if (mine) {
           ch.Fp = -jb.vb * f1[2] - f1[0];
           ch.Bp = f1[1] + 1e-15 * fabs(ch.Fp);
           if (g3.active) {
@@ -623,41 +647,29 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
             ch.Fb = f2[1] + 1e-15 * fabs(ch.F);
           }
           const double logr = (ch.lpp - ch.lp) + (ch.Fp - ch.F);
-          const uint4 w = philox4x32_10_rk(make_uint4(0u, kTagAcc, step, g.cid), jb.rk);
-          const double lu = log(((double)w.x + 0.5) * 0x1p-32);
+          const double lu = log_u64(step);
           const double Mg = ch.Bp + ch.Fb + 1e-12 * (fabs(ch.lpp) + fabs(ch.lp) + fabs(ch.Fp) + fabs(ch.F)) + 1e-300;
-          if (logr - lu > Mg) ch.flag_acc = 1, ch.flag_rec = 0;
-          else if (lu - logr > Mg) ch.flag_acc = 0, ch.flag_rec = 0;
+          if (logr - lu > Mg) ch.flag_acc = 1;
+          else if (lu - logr > Mg) ch.flag_acc = 0;
           else ch.flag_rec = 2;
           ch.rec_mh += 1ull;
         }
-      }
-    }
-    if (PREC == kMixed) {
-      int need;
-      if (KIND == kKitaev && MULTI) {
-        loop_sync();                 // the leader's flag_rec, read by its whole group
-        need = g.active && ch.flag_rec;
-      } else {
-        need = __syncthreads_or(g.active && g.r == 0 && ch.flag_rec);
+        need = __syncthreads_or(mine && ch.flag_rec == 2);
       }
       if (need) {
         // the FP64 path's free energies of v' (and of v when only its FP32
         // value is known), computed by the same code and reduction order
-        // FP64 tables from global memory (the mixed kernel keeps only FP32 ones)
-        Tabs tb64g = tb;
-        tb64g.f64 = jb.f64;
-        tb64g.b64 = jb.b64;
-        Grp g2 = g;
-        g2.active = g.active && ch.flag_rec;
-        double f1[4];
-        free_energy64(jb, tb64g, g2, vp, f1);
-        loop_reduce4(f1, g2);
-        Grp g3 = g2;
-        g3.active = g2.active && ch.Fb != 0.0;
-        double f2[4];
-        free_energy64(jb, tb64g, g3, v, f2);
-        loop_reduce4(f2, g3);
+        // (tables from global memory: the mixed kernel keeps only FP32 ones)
+        Grp g4 = g2;
+        g4.active = g2.active && (KIND == kKitaev || ch.flag_rec == 2);
+        FreeSum f1;
+        free_energy64(jb, g4, vp, &f1);
+        loop_reduce(f1, g4, std::integral_constant<int, kFP64>());
+        Grp g3 = g4;
+        g3.active = g4.active && ch.Fb != 0.0;
+        FreeSum f2;
+        free_energy64(jb, g3, v, &f2);
+        loop_reduce(f2, g3, std::integral_constant<int, kFP64>());
         // Kitaev: the FP64 eigen-stage of v' (and of v when its log-weight
         // came from the df64 stage), by the group that needs it
         double k1v[3] = {0.0, 0.0, 0.0}, k0v[3] = {0.0, 0.0, 0.0};
@@ -666,47 +678,32 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
           kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, k1v, nullptr, jb.lc_edge > 0);
           if (redo_v) kitaev_logpi64<MULTI>(g, v, jb.L, jb.J, ch.beta, wk, k0v, nullptr, jb.lc_edge > 0);
         }
-        if (g2.active && g.r == 0) {
-          ch.Fp = -jb.vb * f1[2] - f1[0];
+        if (g4.active && g.r == 0) {
+          ch.Fp = free_value<kFP64>(jb.vb, f1);
           ch.Bp = 0.0;
           if (g3.active) {
-            ch.F = -jb.vb * f2[2] - f2[0];
+            ch.F = free_value<kFP64>(jb.vb, f2);
             ch.Fb = 0.0;
           }
           if (KIND == kKitaev) {
             ch.lpp = k1v[0];
             ch.lppb = 0.0;
             ch.Ep = k1v[1];
-            ch.otp[0] = k1v[1]; ch.otp[1] = k1v[1] * k1v[1]; ch.otp[2] = k1v[2];
+            ch.cfp = k1v[2];
             if (redo_v) {
               ch.lp = k0v[0];
               ch.lpb = 0.0;
             }
           }
-          const double logr = (ch.lpp - ch.lp) + (ch.Fp - ch.F);
-          const uint4 w = philox4x32_10_rk(make_uint4(0u, kTagAcc, step, g.cid), jb.rk);
-          const double lu = log(((double)w.x + 0.5) * 0x1p-32);
-          ch.flag_acc = lu < logr;
+          ch.flag_acc = log_u64(step) < (ch.lpp - ch.lp) + (ch.Fp - ch.F);
           if (KIND == kKitaev) ch.rec_mh += 1ull;   // Ising: counted at the df64 level
         }
       }
+      if (mine && ch.flag_acc) ch.cur ^= 1;
+      loop_sync();
     }
-    if (g.active && g.r == 0) {
-      if (ch.flag_acc) {
-        ch.cur ^= 1;
-        ch.F = ch.Fp;
-        ch.Fb = ch.Bp;
-        ch.lp = ch.lpp;
-        ch.lpb = ch.lppb;
-        ch.E = ch.Ep;
-        for (int o = 0; o < kNobs; ++o) ch.ot[o] = ch.otp[o];
-        ch.acc += 1ull;
-      }
-      for (int o = 0; o < kNobs; ++o) ch.os[o] += ch.ot[o];
-      trace_store(jb, g.c, step0 + (uint64_t)s, ch.E);
-    }
-    loop_sync();
   }
+  if (clerk && prm.S > 0) settle(step0 + (uint64_t)(prm.S - 1));
 
   if (nrec) atomicAdd(&ch.rec, (unsigned long long)nrec);
   __syncthreads();
@@ -767,38 +764,49 @@ cudaError_t limit_inst(size_t bytes) {
 
 template <int KIND, int PREC, int NT>
 cudaError_t launch_nt(int KC, int kC, const LaunchParams& p, int grid, size_t smem, cudaStream_t st) {
-  if (KC == 4 && kC == 5) return launch_inst<KIND, PREC, 4, 5, NT>(p, grid, smem, st);
-  if (KC == 4 && kC == 3) return launch_inst<KIND, PREC, 4, 3, NT>(p, grid, smem, st);
+  if constexpr (PREC == kMixed) {
+    if (KC == 4 && kC == 5) return launch_inst<KIND, PREC, 4, 5, NT>(p, grid, smem, st);
+    if (KC == 4 && kC == 3) return launch_inst<KIND, PREC, 4, 3, NT>(p, grid, smem, st);
+  }
   return launch_inst<KIND, PREC, 0, 0, NT>(p, grid, smem, st);
 }
 
 template <int KIND, int PREC, int NT>
 cudaError_t limit_nt(size_t bytes) {
-  cudaError_t e = limit_inst<KIND, PREC, 4, 5, NT>(bytes);
-  if (e == cudaSuccess) e = limit_inst<KIND, PREC, 4, 3, NT>(bytes);
-  if (e == cudaSuccess) e = limit_inst<KIND, PREC, 0, 0, NT>(bytes);
+  cudaError_t e = limit_inst<KIND, PREC, 0, 0, NT>(bytes);
+  if constexpr (PREC == kMixed) {
+    if (e == cudaSuccess) e = limit_inst<KIND, PREC, 4, 5, NT>(bytes);
+    if (e == cudaSuccess) e = limit_inst<KIND, PREC, 4, 3, NT>(bytes);
+  }
   return e;
 }
 
 // The several-chains-per-CTA proposal kernel (mixed-size Kitaev batches).
 template <int KIND, int PREC, int NT>
 cudaError_t launch_multi(int KC, int kC, const LaunchParams& p, int grid, size_t smem, cudaStream_t st) {
-  if (KC == 4 && kC == 5) return launch_inst<KIND, PREC, 4, 5, NT, true>(p, grid, smem, st);
-  if (KC == 4 && kC == 3) return launch_inst<KIND, PREC, 4, 3, NT, true>(p, grid, smem, st);
+  if constexpr (PREC == kMixed) {
+    if (KC == 4 && kC == 5) return launch_inst<KIND, PREC, 4, 5, NT, true>(p, grid, smem, st);
+    if (KC == 4 && kC == 3) return launch_inst<KIND, PREC, 4, 3, NT, true>(p, grid, smem, st);
+  }
   return launch_inst<KIND, PREC, 0, 0, NT, true>(p, grid, smem, st);
 }
 
 template <int KIND, int PREC, int NT>
 cudaError_t limit_multi(size_t bytes) {
-  cudaError_t e = cudaSuccess;
-  for (auto f : {crbm_step_kernel<KIND, PREC, 4, 5, NT, 0, true>, crbm_step_kernel<KIND, PREC, 4, 3, NT, 0, true>,
-                 crbm_step_kernel<KIND, PREC, 0, 0, NT, 0, true>})
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  auto limit = [&](auto f) {
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  cudaError_t e = limit(crbm_step_kernel<KIND, PREC, 0, 0, NT, 0, true>);
+  if constexpr (PREC == kMixed) {
+    if (e == cudaSuccess) e = limit(crbm_step_kernel<KIND, PREC, 4, 5, NT, 0, true>);
+    if (e == cudaSuccess) e = limit(crbm_step_kernel<KIND, PREC, 4, 3, NT, 0, true>);
+  }
   return e;
 }
 
 // One translation unit per (kind, precision, CTA size) instantiates the
-// (K, k) variants (4, 5), (4, 3) and runtime: CTAs of 256 threads, plus 128,
+// (K, k) variants (mixed: (4, 5), (4, 3) and runtime; FP64, whose phases wait
+// on the FP64 pipe and not on their integer work: runtime alone): CTAs of 256 threads, plus 128,
 // 64 and 32 threads for the Kitaev kind (small matrices); every CTA size gets
 // the same 128-register budget.  Separate units compile in parallel.
 #define CRBM_VARIANTS_NT(KIND, PREC, NT)                                                       \

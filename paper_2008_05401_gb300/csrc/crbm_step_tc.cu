@@ -477,7 +477,7 @@ template <int LT>
 static __device__ __noinline__ void mh_redo(const JobDev& jb, ChainSm* chs, double* scratch, const uint32_t* pv,
                                             const uint32_t* vbits, uint32_t step, int c0) {
   using G = Geo<LT>;
-  const int tid = threadIdx.x, k = jb.k;
+  const int tid = threadIdx.x;
   Grp g2;
   g2.tpc = kEpi / G::CH;
   g2.gl = tid / g2.tpc;
@@ -529,24 +529,19 @@ static __device__ __noinline__ void mh_redo(const JobDev& jb, ChainSm* chs, doub
   if (__syncthreads_or(g2.active && g2.r == 0 && ch.flag_rec == 2)) {
     Grp g4 = g2;
     g4.active = g2.active && ch.flag_rec == 2;
-    Tabs tb64;
-    memset(&tb64, 0, sizeof tb64);
-    tb64.T = 1 << k;
-    tb64.f64 = jb.f64;
-    tb64.b64 = jb.b64;
-    double f1[4];
-    free_energy64(jb, tb64, g4, pv + c * G::WPC, f1);
-    grp_reduce<4>(f1, g4, scratch);
+    FreeSum f1;
+    free_energy64(jb, g4, pv + c * G::WPC, &f1);
+    reduce_free<kFP64, false>(f1, g4, scratch);
     Grp g3 = g4;
     g3.active = g4.active && ch.Fb != 0.0;
-    double f2[4];
-    free_energy64(jb, tb64, g3, vbits + c * G::WPC, f2);
-    grp_reduce<4>(f2, g3, scratch);
+    FreeSum f2;
+    free_energy64(jb, g3, vbits + c * G::WPC, &f2);
+    reduce_free<kFP64, false>(f2, g3, scratch);
     if (g4.active && g4.r == 0) {
-      ch.Fp = -jb.vb * f1[2] - f1[0];
+      ch.Fp = free_value<kFP64>(jb.vb, f1);
       ch.Bp = 0.0;
       if (g3.active) {
-        ch.F = -jb.vb * f2[2] - f2[0];
+        ch.F = free_value<kFP64>(jb.vb, f2);
         ch.Fb = 0.0;
       }
       const double logr = (ch.lpp - ch.lp) + (ch.Fp - ch.F);

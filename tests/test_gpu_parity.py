@@ -90,6 +90,27 @@ def test_ising_matches_oracle(ctx, L, K, k, n, g, correct, std):
     jm.release()
 
 
+@pytest.mark.parametrize("L,K,k,n,g", [(2, 1, 2, 5003, 1), (4, 2, 3, 4999, 2), (6, 2, 3, 2501, 1), (8, 2, 3, 1301, 1),
+                                       (12, 4, 3, 310, 1), (24, 2, 5, 307, 1)])
+def test_many_ising_chains_match_oracle(ctx, L, K, k, n, g):
+    """Enough chains for several to share a CTA, a warp or a word's lanes (the
+    few chains of the cases above take a CTA each), a partly empty last CTA:
+    both precisions against the oracle."""
+    from paper_2008_05401_gb300 import FP64, ISING, MIXED
+    W, hb, vb = wl.gaussian_crbm(K, k, 0.3, seed=L * 10 + K)
+    T = wl.ising_ladder(n, 8)
+    bits0 = wl.pack_bits(wl.random_lattices(n, L, seed=L))
+    S = 3
+    ref = oracle_chains("ising", W, hb, vb, L, T, (1.0,), SEED, n, bits0)
+    worst = run_oracle(ref, S, g=g)
+    mid = ctx.load_model(ISING, W, vb, hb)
+    for prec in (FP64, MIXED):
+        job = ctx.new_job(mid, ISING, L, T, (1.0,), SEED, 0, bits0, prec)
+        job.run(S, g=g, precision=prec)
+        _compare(job, ref, worst, S)
+        job.release()
+
+
 KITAEV_CASES = [
     # L, K, k, n, correct
     (2, 2, 2, 6, True),
