@@ -1214,10 +1214,10 @@ __device__ __forceinline__ double eigen_idx(const KitaevWork& wk, const EigGrid&
 // log 2cosh x, -(eps/2) tanh x and x^2 sech^2 x with x = beta eps / 2.
 __device__ __forceinline__ void thermal_add(double eps, double beta, double& lp, double& en, double& cf) {
   const double x = 0.5 * beta * eps;
-  const double qx = exp(-2.0 * x);
+  const double qx = exp(-2.0 * x), r = 1.0 / (1.0 + qx), t = x * r;
   lp += x + log1p(qx);
-  en += -0.5 * eps * (1.0 - qx) / (1.0 + qx);
-  cf += x * x * 4.0 * qx / ((1.0 + qx) * (1.0 + qx));
+  en += -0.5 * eps * ((1.0 - qx) * r);
+  cf += 4.0 * qx * (t * t);
 }
 
 // eps_out (optional, device memory): the N energies eps, ascending.

@@ -175,3 +175,34 @@ def test_f32_rounding_matches_numpy():
     for _ in range(2000):
         x = rng.uniform(-1e3, 1e3)
         assert f32(Fr(x)) == Fr(float(np.float32(x)))
+
+
+def df_mul(a, b):
+    ph, pl = two_prod(a[0], b[0])
+    return fast_two_sum(ph, fma(a[0], b[1], fma(a[1], b[0], pl)))
+
+
+def test_df_sqrt_and_reciprocal_bound():
+    """The square root and reciprocal from approximations within 2^-22 of the
+    exact value (any such value, here the worst and random ones): relative
+    errors below 2^-44."""
+    rng = random.Random(71)
+    for n in range(N_CASES):
+        a = rand_df(rng, scale=2.0)
+        if val(a) <= 0:
+            a = (-a[0], -a[1])
+        if a[0] == 0:
+            continue
+        off = 1 + Fr(1, 2 ** 22) * Fr(1 if n % 3 == 0 else -1 if n % 3 == 1 else rng.uniform(-1.0, 1.0))
+        root = Fr(float(a[0])) ** 1
+        y = f32(Fr(float(root) ** -0.5) * off)
+        h = mul(a[0], y)
+        h = fma(fma(-h, h, a[0]), mul(Fr(1, 2), y), h)
+        r = add(fma(-h, h, a[0]), a[1])
+        q = fast_two_sum(h, mul(r, mul(Fr(1, 2), y)))
+        assert abs(val(q) ** 2 - val(a)) <= Fr(1, 2 ** 43) * val(a)
+        y = f32(1 / a[0] * off)
+        y = fma(y, fma(-a[0], y, Fr(1)), y)
+        e = fma(-a[1], y, fma(-a[0], y, Fr(1)))
+        q = fast_two_sum(y, mul(y, e))
+        assert abs(val(q) * val(a) - 1) <= Fr(1, 2 ** 44)
