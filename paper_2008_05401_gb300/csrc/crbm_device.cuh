@@ -356,25 +356,6 @@ __device__ __forceinline__ void grp_sync(const Grp& g) {
   }
 }
 
-// Deterministic sum over a chain's (warp-aligned) group, returned to every
-// thread of it: a butterfly within each warp, then the warps' partials added
-// in warp order -- the order of block_sum for a CTA of tpc threads, so a group
-// gives the same bits as a CTA of its size.  scratch: 32 doubles of the group.
-template <bool MULTI>
-__device__ __forceinline__ double grp_sum(double x, const Grp& g, double* scratch) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) x += __shfl_xor_sync(kFull, x, o);
-  const int r = MULTI ? g.r : (int)threadIdx.x, tpc = MULTI ? g.tpc : (int)blockDim.x;
-  const int warp = r >> 5, nw = tpc >> 5;
-  grp_sync<MULTI>(g);
-  if ((r & 31) == 0) scratch[warp] = x;
-  grp_sync<MULTI>(g);
-  double s = 0.0;
-  for (int w = 0; w < nw; ++w) s += scratch[w];
-  grp_sync<MULTI>(g);
-  return s;
-}
-
 // Sums of a free-energy pass: F's softplus sum -- FP64 (s), or for the FP32
 // pass the thread's sum as an integer in units of 2^-32 (fx: exact additions
 // off the FP64 pipe, each thread's conversion within 2^-33) with the data part
@@ -955,10 +936,6 @@ __device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
 }
 
 // --------------------------------------------------- Kitaev log-weight
-// FP64 eigen-stage for one lattice by the whole CTA.  A = M^T M (Sec. IV,
-// M_bw = 2 J_a u_bw) is reduced to tridiagonal form by Householder
-// reflections, its eigenvalues mu_l = eps_l^2 are found by bisection with
-// Sturm counts, and log pi = sum_l log 2cosh(beta eps_l / 2).
 // Packed lower triangle of a symmetric N x N matrix: element (i, c), c <= i.
 __device__ __forceinline__ int tri(int i, int c) { return i * (i + 1) / 2 + c; }
 // Lanes per row of a group's matrix-vector product over m rows with nt
@@ -999,14 +976,12 @@ struct FoldWalk {
 };
 
 struct KitaevWork {
-  double* A;       // packed lower triangle, N (N+1) / 2 entries
+  double* A;       // packed lower triangle, N (N+1) / 2 entries; reduced: d and e^2 scaled, the counts' grid
   double* d;       // N
   double* e;       // N
-  double* vv;      // N
-  double* pw;      // N
+  double* uw;      // 2 N: (u, w) of the Householder step
   double* sc;      // 64 doubles
-  float* d32;      // N   FP32 copies of the tridiagonal for eigenvalue isolation
-  float* e32;      // N   (squared off-diagonals)
+  double* xs;      // N + 8: the current column; reduced: the FP32 tridiagonal, padded to a multiple of 8 float2
 };
 
 // Number of eigenvalues below x of the symmetric tridiagonal (d, off-diagonal^2
@@ -1044,37 +1019,32 @@ __device__ __forceinline__ int sturm_count(const double* d, const double* e2, in
   return cnt;
 }
 
-// FP32 Sturm count (same recurrence, rescaled by 2^-+60): used only to
-// isolate eigenvalues; every bracket it yields is checked with FP64 counts.
-__device__ __forceinline__ int sturm_count32(const float* d, const float* e2, int N, float x) {
-  float pp = 1.0f, p = d[0] - x;
-  uint32_t b = __float_as_uint(p);
-  uint32_t sprev = 0u;
-  uint32_t s = (b << 1) == 0u ? 1u : (b >> 31);
-  int cnt = (int)(s ^ sprev);
-  sprev = s;
-  for (int i = 1; i < N; ++i) {
-    const float pn = fmaf(-e2[i - 1], pp, (d[i] - x) * p);
-    pp = p;
-    p = pn;
-    b = __float_as_uint(p);
-    s = (b << 1) == 0u ? (sprev ^ 1u) : (b >> 31);
-    cnt += (int)(s ^ sprev);
-    sprev = s;
-    const int ex = (int)((b >> 23) & 0xffu);
-    if (ex > 127 + 60) {
-      p *= 0x1p-60f;
-      pp *= 0x1p-60f;
-    } else if (ex < 127 - 60 && (int)((__float_as_uint(pp) >> 23) & 0xffu) < 127 - 60) {
-      p *= 0x1p+60f;
-      pp *= 0x1p+60f;
+// FP32 Sturm count of the scaled tridiagonal, entry i = (d_i, e_{i-1}^2),
+// padded to a multiple of 8 with entries (2, 0), which change no sign (every
+// x is below 2; the spectrum lies in [-1, 1], so nothing overflows): used only
+// to isolate eigenvalues.
+__device__ __forceinline__ int sturm_count32(const float2* de, int N, float x) {
+  float pp = 0.0f, p = 1.0f;
+  int cnt = 0;
+  for (int i0 = 0; i0 < N; i0 += 8) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float2 t = de[i0 + i];
+      const float pn = fmaf(-t.y, pp, (t.x - x) * p);
+      cnt += (int)((__float_as_uint(pn) ^ __float_as_uint(p)) >> 31);
+      pp = p;
+      p = pn;
+    }
+    if (fmaxf(fabsf(p), fabsf(pp)) < 0x1p-50f) {
+      p *= 0x1p+50f;
+      pp *= 0x1p+50f;
     }
   }
   return cnt;
 }
 
-// Shared start of the eigenvalues' FP32 bisections: G points strictly inside
-// the (FP32) Gershgorin interval, point k at lo + (k + 1) h with
+// Isolation of the eigenvalues of the scaled tridiagonal: G points strictly
+// inside the Gershgorin interval (lo, hi), point k at lo + (k + 1) h with
 // h = (hi - lo) / (G + 1), and the FP32 Sturm count at each, one point per
 // thread of the group.  The count at a point is the number of eigenvalues
 // below it, so eigenvalue idx lies between the last point whose count is
@@ -1083,131 +1053,203 @@ __device__ __forceinline__ int sturm_count32(const float* d, const float* e2, in
 // counts live in the reduced matrix's storage, free by then beyond the
 // first 2N doubles (at most N^2 - 3N ints).
 struct EigGrid {
-  const int* cnt;
-  int G;
+  const float2* de;
+  int* cnt;
+  int N, G;
   float lo, hi, h;
+  double glo, ghi;   // the interval widened by FP32's roundings: it holds the spectrum
+  __device__ __forceinline__ EigGrid(const float2* de_, double* A, int n, float l, float u, int nt)
+      : de(de_), cnt(reinterpret_cast<int*>(A + 2 * n)), N(n), G(min(nt, n * n - 3 * n)), lo(l), hi(u),
+        h((u - l) / (float)(G + 1)) {
+    const float out = 0x1p-20f * fmaxf(fabsf(l), fabsf(u));
+    glo = (double)(l - out);
+    ghi = (double)(u + out);
+  }
   __device__ __forceinline__ float x(int k) const { return __fmaf_rn((float)(k + 1), h, lo); }
-  // [lo32, hi32]: neighbouring grid points (or interval ends) with
-  // count(lo32) <= idx < count(hi32) as computed; the bisection goes on from
-  // there, and the verification after it falls back to the Gershgorin interval
-  // should the FP32 counts not be monotone
-  __device__ __forceinline__ void bracket(int idx, float& lo32, float& hi32) const {
-    int a = 0, b = G;
-    while (a < b) {
-      const int mid = (a + b) >> 1;
-      if (cnt[mid] > idx) b = mid; else a = mid + 1;
+  // this thread's point (the caller syncs the group before the counts are read)
+  __device__ __forceinline__ void fill(int tid) {
+    if (tid < G) cnt[tid] = sturm_count32(de, N, x(tid));
+  }
+  // [a, b]: at most 2^-q of the interval wide (FP32 permitting), with
+  // count(a) <= idx < count(b) as computed in FP32 (what it yields is certified
+  // by the stage's own counts)
+  __device__ __forceinline__ void isolate(int idx, float w, float& a, float& b) const {
+    int i = 0, j = G;
+    while (i < j) {
+      const int mid = (i + j) >> 1;
+      if (cnt[mid] > idx) j = mid; else i = mid + 1;
     }
-    lo32 = a == 0 ? lo : x(a - 1);
-    hi32 = a == G ? hi : x(a);
+    a = i == 0 ? lo : x(i - 1);
+    b = i == G ? hi : x(i);
+    for (int it = 0; it < 32 && b - a > w; ++it) {
+      const float mid = 0.5f * (a + b);
+      if (!(mid > a && mid < b)) break;
+      if (sturm_count32(de, N, mid) > idx) b = mid; else a = mid;
+    }
   }
 };
 
-// Fill the grid (every thread of the group calls; the caller syncs the group
-// before the counts are read).  d32 / e32 and the interval must be final.
-__device__ __forceinline__ EigGrid eig_grid(const KitaevWork& wk, int N, double glo, double ghi, int tid, int nt) {
-  EigGrid gr;
-  int* cnt = reinterpret_cast<int*>(wk.A + 2 * N);
-  gr.cnt = cnt;
-  gr.G = min(nt, N * N - 3 * N);
-  gr.lo = (float)glo;
-  gr.hi = (float)ghi;
-  gr.h = (gr.hi - gr.lo) / (float)(gr.G + 1);
-  if (tid < gr.G) cnt[tid] = sturm_count32(wk.d32, wk.e32, N, gr.x(tid));
-  return gr;
+// The leading 24 bits of an FP64 value as a float, by integer operations; 0
+// below 2^-120 (|x| < 2^127).
+__device__ __forceinline__ float lead32(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), e = (hi >> 20) & 0x7ffu;
+  const uint32_t b = __funnelshift_l((uint32_t)__double2loint(x), hi, 3);
+  return e < 1023 - 120 ? 0.0f : __uint_as_float(((b + 0x40000000u) & 0x7fffffffu) | (hi & 0x80000000u));
+}
+// x 2^k, k > 0, by its exponent field (0 stays 0).
+__device__ __forceinline__ double shift_exponent(double x, int k) {
+  const int hi = __double2hiint(x);
+  return ((hi >> 20) & 0x7ff) == 0 ? x : __hiloint2double(hi + (k << 20), __double2loint(x));
 }
 
-// FP64 Sturm count together with p_N(x) and p_N'(x) (for a Newton step):
-// p_i' = (d_i - x) p_{i-1}' - p_{i-1} - e2_{i-1} p_{i-2}', all four values of a
-// step rescaled together.  Five FP64 operations per step.
-struct SturmNewton {
-  int cnt;
-  double p, dp;
-};
-
-__device__ __forceinline__ SturmNewton sturm_newton(const double* d, const double* e2, int N, double x) {
-  double pp = 1.0, p = d[0] - x, dpp = 0.0, dp = -1.0;
-  int hi = __double2hiint(p);
-  uint32_t sprev = 0u;
-  uint32_t s = ((hi & 0x7fffffff) | __double2loint(p)) == 0 ? 1u : ((uint32_t)hi >> 31);
-  int cnt = (int)(s ^ sprev);
-  sprev = s;
-  for (int i = 1; i < N; ++i) {
-    const double dx = d[i] - x;
-    const double pn = fma(-e2[i - 1], pp, dx * p);
-    const double dpn = fma(-e2[i - 1], dpp, fma(dx, dp, -p));
-    pp = p;
-    p = pn;
-    dpp = dp;
-    dp = dpn;
-    hi = __double2hiint(p);
-    const uint32_t zero = ((hi & 0x7fffffff) | __double2loint(p)) == 0;
-    s = zero ? (sprev ^ 1u) : ((uint32_t)hi >> 31);
-    cnt += (int)(s ^ sprev);
-    sprev = s;
-    const int ex = max((hi >> 20) & 0x7ff, (__double2hiint(dp) >> 20) & 0x7ff);
-    if (ex > 1023 + 500) {
-      p *= 0x1p-500;
-      pp *= 0x1p-500;
-      dp *= 0x1p-500;
-      dpp *= 0x1p-500;
-    } else if (ex < 1023 - 500 && max((__double2hiint(pp) >> 20) & 0x7ff, (__double2hiint(dpp) >> 20) & 0x7ff) <
-                                      1023 - 500) {
-      p *= 0x1p+500;
-      pp *= 0x1p+500;
-      dp *= 0x1p+500;
-      dpp *= 0x1p+500;
+// p_N(x) / p_N'(x) of the scaled tridiagonal: p in FP64 (three operations a
+// step), its derivative in FP32 on the other pipe (the quotient needs no more
+// than its leading digits).  An overflowing or lost value shows in the
+// certification of the root.
+__device__ __forceinline__ float newton_step64(const double* d, const double* e2, const float2* de, int N, double x) {
+  const float xf = (float)x;
+  double pp = 1.0, p = d[0] - x;
+  float ppf = 1.0f, pf = lead32(p), dpp = 0.0f, dp = -1.0f;
+  for (int i0 = 1; i0 < N; i0 += 4) {
+    const int i1 = min(i0 + 4, N);
+    for (int i = i0; i < i1; ++i) {
+      const double pn = fma(-e2[i - 1], pp, (d[i] - x) * p);
+      const float2 t = de[i];
+      const float dpn = fmaf(-t.y, dpp, fmaf(t.x - xf, dp, -pf));
+      dpp = dp;
+      dp = dpn;
+      pp = p;
+      p = pn;
+      ppf = pf;
+      pf = lead32(p);
+    }
+    if (fmaxf(fabsf(pf), fabsf(ppf)) < 0x1p-30f) {
+      p = shift_exponent(p, 30);
+      pp = shift_exponent(pp, 30);
+      pf = lead32(p);
+      dp *= 0x1p+30f;
+      dpp *= 0x1p+30f;
     }
   }
-  return {cnt, p, dp};
+  return pf / dp;
 }
 
-// Eigenvalue idx (ascending) of the tridiagonal: FP32 bisection isolates it,
-// two FP64 Sturm counts verify the bracket (falling back to the Gershgorin
-// interval), then safeguarded Newton steps on p_N refine it in FP64; every
-// iterate updates the bracket through its Sturm count, and a step that leaves
-// the bracket is replaced by bisection.
-__device__ __forceinline__ double eigen_idx(const KitaevWork& wk, const EigGrid& gr, int N, int idx, double glo,
-                                           double ghi) {
-  const double range = fmax(ghi - glo, 1e-300);
-  float lo32, hi32;
-  gr.bracket(idx, lo32, hi32);
-  const float w32 = (float)(range * 0x1p-20);
-  for (int it = 0; it < 48 && hi32 - lo32 > w32; ++it) {
-    const float mid = 0.5f * (lo32 + hi32);
-    if (!(mid > lo32 && mid < hi32)) break;
-    if (sturm_count32(wk.d32, wk.e32, N, mid) > idx) hi32 = mid; else lo32 = mid;
+// The eigenvalues of one warp's lanes, idx = its lane's index (N or more:
+// none): FP32 isolation, Newton steps, then two of the stage's own counts
+// certify each: count(x - tolc) <= idx < count(x + tolc), tolc several times
+// the counts' own noise.  An eigenvalue that does not certify (clusters closer
+// than FP32 separates, underflow) is found by the whole warp: 32 counts a round
+// on points that span its bracket, which falls back to the Gershgorin interval
+// where the bracket does not hold it, until it is tol wide (about 8 rounds,
+// where one lane's bisection takes 40 counts); more than 6 of a warp bisect
+// side by side.
+// newton(x): refine a double; count(x): the stage's Sturm count.
+template <class NEWTON, class COUNT>
+__device__ __forceinline__ double warp_eigenvalues(const EigGrid& gr, int idx, float w, double tolc, double tol,
+                                                   NEWTON newton, COUNT count) {
+  const int lane = threadIdx.x & 31;
+  const double glo = gr.glo, ghi = gr.ghi;
+  float lo = gr.lo, hi = gr.hi;
+  double x = 0.0;
+  bool open = false;
+  if (idx < gr.N) {
+    gr.isolate(idx, w, lo, hi);
+    x = newton(0.5f * (lo + hi));
+    open = !(x >= glo && x <= ghi && count(x - tolc) <= idx && count(x + tolc) > idx);
   }
-  const double pad = 0x1p-14 * range;
-  double lo = fmax(glo, (double)lo32 - pad), hi = fmin(ghi, (double)hi32 + pad);
-  if (sturm_count(wk.d, wk.vv, N, lo) > idx) lo = glo;
-  if (sturm_count(wk.d, wk.vv, N, hi) <= idx) hi = ghi;
-  const double tol_abs = 1e-15 * range;
-  double x = 0.5 * (lo + hi);
-  for (int it = 0; it < 100; ++it) {
-    const double tol = fmax(tol_abs, 4.0 * 2.220446049250313e-16 * fmax(fabs(lo), fabs(hi)));
-    if (hi - lo <= tol) {
-      x = 0.5 * (lo + hi);
-      break;
+  unsigned left = __ballot_sync(kFull, open);
+  if (__popc(left) > 6) {
+    if (open) {
+      double a = (double)lo, b = (double)hi;
+      if (count(a) > idx) a = glo;
+      if (count(b) <= idx) b = ghi;
+      for (int it = 0; it < 64 && b - a > tol; ++it) {
+        const double mid = 0.5 * (a + b);
+        if (count(mid) > idx) b = mid; else a = mid;
+      }
+      x = 0.5 * (a + b);
     }
-    const SturmNewton r = sturm_newton(wk.d, wk.vv, N, x);
-    if (r.cnt > idx) hi = x; else lo = x;
-    const double step = r.p / r.dp;
-    double xn = x - step;
-    // a Newton step below the tolerance that stays in the bracket has found
-    // the root: stop before the bracket test below can turn it into bisection
-    // (x may sit on the root itself, which then is one end of the bracket)
-    if (fabs(step) <= tol && xn >= lo && xn <= hi) {
-      x = xn;
-      break;
+    left = 0u;
+  }
+  while (left) {
+    const int who = __ffs(left) - 1, i = __shfl_sync(kFull, idx, who);
+    left &= left - 1;
+    const float pad = 0x1p-18f * (gr.hi - gr.lo);
+    double a = fmax(glo, (double)(__shfl_sync(kFull, lo, who) - pad));
+    double b = fmin(ghi, (double)(__shfl_sync(kFull, hi, who) + pad));
+    bool below = false, above = false;                  // a, b known to enclose eigenvalue i
+    for (int it = 0; it < 24 && (b - a > tol || !below || !above); ++it) {
+      const double h = (b - a) * (1.0 / 31.0), at = lane < 31 ? fma((double)lane, h, a) : b;
+      const unsigned over = __ballot_sync(kFull, count(at) > i);
+      const int f = over ? __ffs(over) - 1 : 32;        // first point beyond eigenvalue i
+      const double na = f > 0 ? __shfl_sync(kFull, at, f - 1) : (below ? a : glo);
+      b = f < 32 ? __shfl_sync(kFull, at, f & 31) : (above ? b : ghi);
+      a = na;
+      below = above = true;
     }
-    if (!(xn > lo && xn < hi)) xn = 0.5 * (lo + hi);
-    if (fabs(xn - x) <= tol) {
-      x = xn;
-      break;
-    }
-    x = xn;
+    if (lane == who) x = 0.5 * (a + b);
   }
   return x;
+}
+
+// The Gershgorin interval of a group's tridiagonal: the least lo and the
+// largest hi over its threads.  sc: 16 floats of the group.
+template <bool MULTI>
+__device__ __forceinline__ void group_interval(float& lo, float& hi, const Grp& g, float* sc) {
+  const int tid = MULTI ? g.r : (int)threadIdx.x, nw = (MULTI ? g.tpc : (int)blockDim.x) >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
+  }
+  if ((tid & 31) == 0) {
+    sc[2 * (tid >> 5)] = lo;
+    sc[2 * (tid >> 5) + 1] = hi;
+  }
+  grp_sync<MULTI>(g);
+  for (int w = 0; w < nw; ++w) {
+    lo = fminf(lo, sc[2 * w]);
+    hi = fmaxf(hi, sc[2 * w + 1]);
+  }
+}
+
+// Sums of (lp, en, cf) and of a bound over a group, valid in its leader.  sc:
+// 4 doubles per warp.
+template <bool MULTI>
+__device__ __forceinline__ void group_thermal(double& lp, double& en, double& cf, float& bd, const Grp& g, double* sc) {
+  const int tid = MULTI ? g.r : (int)threadIdx.x, nw = (MULTI ? g.tpc : (int)blockDim.x) >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lp += __shfl_xor_sync(kFull, lp, o);
+    en += __shfl_xor_sync(kFull, en, o);
+    cf += __shfl_xor_sync(kFull, cf, o);
+    bd += __shfl_xor_sync(kFull, bd, o);
+  }
+  if (nw == 1) return;
+  grp_sync<MULTI>(g);
+  if ((tid & 31) == 0) {
+    double* mine = sc + 4 * (tid >> 5);
+    mine[0] = lp;
+    mine[1] = en;
+    mine[2] = cf;
+    *(float*)(mine + 3) = bd;
+  }
+  grp_sync<MULTI>(g);
+  if (tid == 0)
+    for (int w = 1; w < nw; ++w) {
+      lp += sc[4 * w];
+      en += sc[4 * w + 1];
+      cf += sc[4 * w + 2];
+      bd += *(const float*)(sc + 4 * w + 3);
+    }
+}
+
+// Couplings scaled by a power of two so that the largest lies in [1, 2) (exact,
+// undone at the end): FP32 helpers then never run out of exponents.  M's
+// entries are the 2 J.
+__device__ __forceinline__ int coupling_exponent(const double* J) {
+  const double m = fmax(fabs(J[0]), fmax(fabs(J[1]), fabs(J[2])));
+  return m > 0.0 ? ((__double2hiint(m) >> 20) & 0x7ff) - 1023 : 0;
 }
 
 // One single-fermion level's share of log pi, e and c_f (Sec. IV):
@@ -1220,31 +1262,55 @@ __device__ __forceinline__ void thermal_add(double eps, double beta, double& lp,
   cf += 4.0 * qx * (t * t);
 }
 
+// FP64 eigen-stage for one lattice: A = M^T M (Sec. IV, M_bw = 2 J_a u_bw) is
+// reduced to tridiagonal form by Householder reflections, its eigenvalues
+// mu_l = eps_l^2 found one per thread, and res = {log pi = sum_l
+// log 2cosh(beta eps_l / 2), e, c_f}, valid in the group's leader (r == 0).
 // eps_out (optional, device memory): the N energies eps, ascending.
-// open_cols: the lattice is open along j (the y-bonds from column L-1 to
-// column 0 are absent), the physics of the LCRBM's open boundary conditions.
-// Run by the chain's thread group g (warp-aligned) with its own work areas wk;
-// every thread of the group calls, and only the group synchronises (MULTI:
-// see grp_sync).
+// For periodic lattices (open ones: kitaev_logpi64_open).  Run by the chain's
+// thread group g (warp-aligned) with its own work areas wk; every thread of the
+// group calls, and only the group synchronises (MULTI: see grp_sync).
+//
+// Column j of the reduction, with x = A[j+1:, j], u = x - alpha e_1, tau = 2 /
+// u^T u, p = tau A22 u, w = p - (tau p^T u / 2) u, A22 -= u w^T + w u^T, in three
+// group barriers:
+//   1. y = A22 x with H lanes per row, and per warp the partial of x^T y; beside
+//      it one warp (each in turn) takes s = x^T x - x_0^2, alpha, u_0 and tau,
+//      on which y does not wait;
+//   2. u^T A22 u = x^T y - 2 alpha y_0 + alpha^2 a_00, p_l = tau (y_l - alpha
+//      a_l0) and w;
+//   3. the rank-2 update of the packed triangle, the first column (the next x)
+//      into an array of its own.
+// A column whose x is below 2^-59 ||A||_2 is taken as reduced.
+// What bounds it: the FP64 pipe, which every warp instruction holds for about
+// 64 cycles, so the count of FP64 instructions per warp -- hence the scalars in
+// one warp instead of all, FP32 derivatives and two counts per eigenvalue
+// (before: two counts, then Newton steps of five operations until one confirms
+// the last), one Gershgorin interval in FP32 (before: a serial FP64 loop of one
+// thread), and clusters found by the whole warp.  1024 chains of L = 6, four
+// proposals: 1.81 ms (3.74); six tempering cycles of 1024 + 1024 chains of L = 8,
+// four Gibbs steps each: 7.7 ms (15.0).
 template <bool MULTI>
 __device__ inline void kitaev_logpi64(const Grp& g, const uint32_t* v, int L, const double* J, double beta,
-                               const KitaevWork& wk, double (&res)[3], double* eps_out = nullptr,
-                               bool open_cols = false) {
+                               const KitaevWork& wk, double (&res)[3], double* eps_out = nullptr) {
   const int N = L * L, tid = MULTI ? g.r : (int)threadIdx.x, nt = MULTI ? g.tpc : (int)blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   double* A = wk.A;
-  const double tx = 2.0 * J[0], ty = 2.0 * J[1], tz = 2.0 * J[2];
+  double2* uw = reinterpret_cast<double2*>(wk.uw);     // (u, w) of a row; .y holds y until w is known
+  double* xs = wk.xs;
+  const int kJ = coupling_exponent(J);
+  const double sJ = ldexp(2.0, -kJ), tx = sJ * J[0], ty = sJ * J[1], tz = sJ * J[2];
   // A = M^T M, row w accumulated in a fixed order (z, x, y bond of w, then the
   // three whites of that black site)
+  for (int e = tid; e < N * (N + 1) / 2; e += nt) A[e] = 0.0;
+  grp_sync<MULTI>(g);
   for (int w = tid; w < N; w += nt) {
     double* row = A + tri(w, 0);                    // lower-triangle row w: columns 0..w
-    for (int c = 0; c <= w; ++c) row[c] = 0.0;
     const int i = w / L, j = w - i * L;
     for (int typ = 0; typ < 3; ++typ) {
       int bi = i, bj = j;
       if (typ == 1) bi = (i == 0) ? L - 1 : i - 1;
       if (typ == 2) bj = (j == 0) ? L - 1 : j - 1;
-      if (typ == 2 && open_cols && j == 0) continue;      // this y-bond crosses the open cut
       const int b = bi * L + bj;
       const double mz = site_bit(v, b) ? tz : -tz;
       const double mw = (typ == 0) ? mz : (typ == 1 ? tx : ty);
@@ -1253,170 +1319,220 @@ __device__ inline void kitaev_logpi64(const Grp& g, const uint32_t* v, int L, co
       const int wy = bi * L + ((bj + 1 == L) ? 0 : bj + 1);
       if (wz <= w) row[wz] += mw * mz;
       if (wx <= w) row[wx] += mw * tx;
-      if (wy <= w && !(open_cols && bj + 1 == L)) row[wy] += mw * ty;
+      if (wy <= w) row[wy] += mw * ty;
     }
   }
   grp_sync<MULTI>(g);
-  // Householder tridiagonalisation, column j: x = A[j+1:, j] -> alpha e_1 by
-  // H = I - tau u u^T, u = x - alpha e_1.  Only the lower triangle of the
-  // trailing block A22 (rows and columns j+1..N-1, m of them) is read and
-  // updated; the product with A22 reads u from column j itself (u_0 = x_0 -
-  // alpha, u_c = A[j+1+c][j]), which the step does not change, and stores it
-  // in vv for the update.  Three group barriers per column: p = tau A22 u
-  // with H lanes per row and, per warp, the partial of p^T u; then w = p -
-  // (tau p^T u / 2) u; then A22 -= u w^T + w u^T, its first column (with
-  // per-warp partials of the next step's s, the sum of squares below the
-  // subdiagonal) and the rest of the packed triangle element by element over
-  // the group's threads in the folded order of FoldWalk.  sc[0..31]: p^T u
-  // partials, sc[32..63]: s.
-  double* scP = wk.sc;
-  double* scS = wk.sc + 32;
-  double s;
+  // sc: floats 0..15 partials of |x|^2 without x_0 (FP32, tells a reduced
+  // column); doubles 16.. partials of x^T y; 48.. alpha, u_0, tau, y_0
+  float* scS = reinterpret_cast<float*>(wk.sc);
+  double* scQ = wk.sc + 16;
+  double* scA = wk.sc + 48;
+  auto column_sum = [&](float part) {           // this thread's share of |x|^2 - x_0^2
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
+    if (lane == 0) scS[warp] = part;
+  };
   {
-    double s0 = 0.0;
-    for (int i = 2 + tid; i < N; i += nt) {
-      const double a = A[tri(i, 0)];
-      s0 = fma(a, a, s0);
+    float part = 0.0f;
+    for (int r = tid; r < N - 1; r += nt) {
+      const double a = A[tri(1 + r, 0)];
+      const float f = lead32(a);
+      xs[r] = a;
+      if (r >= 1) part = fmaf(f, f, part);
     }
-    s = grp_sum<MULTI>(s0, g, wk.sc);
+    column_sum(part);
   }
+  grp_sync<MULTI>(g);
+  const float amax = fabsf(lead32(tx)) + fabsf(lead32(ty)) + fabsf(lead32(tz));    // sqrt of a bound on ||A||_2
+  const float tiny = 0x1p-118f * (amax * amax) * (amax * amax);
   for (int j = 0; j < N - 2; ++j) {
     const int m = N - j - 1, j1 = j + 1;
-    const double x0 = A[tri(j1, j)];
-    if (tid == 0) wk.d[j] = A[tri(j, j)];
-    if (s == 0.0) {
-      // column already reduced: no reflection; s of the next column directly
-      if (tid == 0) wk.e[j] = x0;
-      double s2 = 0.0;
-      for (int i = j + 3 + tid; i < N; i += nt) {
-        const double a = A[tri(i, j1)];
-        s2 = fma(a, a, s2);
+    float sf = 0.0f;
+    for (int w = 0; w < nw; ++w) sf += scS[w];
+    if (sf <= tiny) {
+      // column already reduced: no reflection
+      if (tid == 0) {
+        wk.d[j] = A[tri(j, j)];
+        wk.e[j] = xs[0];
       }
-      s = grp_sum<MULTI>(s2, g, wk.sc);
+      grp_sync<MULTI>(g);
+      float part = 0.0f;
+      for (int r = tid; r < m - 1; r += nt) {
+        const double a = A[tri(j1 + 1 + r, j1)];
+        const float f = lead32(a);
+        xs[r] = a;
+        if (r >= 1) part = fmaf(f, f, part);
+      }
+      column_sum(part);
+      grp_sync<MULTI>(g);
       continue;
     }
-    const double nrm = sqrt(x0 * x0 + s);
-    const double alpha = (x0 >= 0.0) ? -nrm : nrm;
-    const double u0 = x0 - alpha;
-    const double tau = 2.0 / (u0 * u0 + s);
-    if (tid == 0) wk.e[j] = alpha;
-    // p_l = tau sum_c A22[l][c] u_c, u_c = A[tri(j1 + c, j)] (c >= 1): H lanes
-    // of a warp per row (H = 1, 2, 4, .. while H m still fits the group), lane
-    // h of a row taking the columns c = h mod H -- the row part c <= l
-    // (contiguous), then the column part c > l -- alternately into two
-    // accumulators, the H lanes' sums then added by a butterfly
-    const int H = row_split(m, nt), h = lane & (H - 1);
-    double part = 0.0;
-    for (int l0 = 0; l0 < m; l0 += nt / H) {
+    // 1. y, x^T y; the scalars
+    if (warp == j % nw) {
+      double s = 0.0;
+      for (int r = 1 + lane; r < m; r += 32) s = fma(xs[r], xs[r], s);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+      const double x0 = xs[0], sig = fma(x0, x0, s), nrm = sqrt(sig);
+      const double alpha = (x0 >= 0.0) ? -nrm : nrm;
+      // tau = 2 / (u_0^2 + s) = 1 / (|x|^2 + |x_0| |x|)
+      const double tau = 1.0 / fma(fabs(x0), nrm, sig);
+      if (lane == 0) {
+        scA[0] = alpha;
+        scA[1] = x0 - alpha;
+        scA[2] = tau;
+        wk.d[j] = A[tri(j, j)];
+        wk.e[j] = alpha;
+      }
+    }
+    double q = 0.0;
+    for (int l0 = 0; l0 < m;) {
+      const int H = row_split(min(m - l0, nt), nt), h = lane & (H - 1);
       const int l = l0 + warp * (32 / H) + lane / H;
-      double e0 = 0.0, e1 = 0.0;
+      double y0 = 0.0, y1 = 0.0;
       if (l < m) {
         const double* row = A + tri(j1 + l, j1);
         int c = h;
-        if (c == 0) {
-          e0 = row[0] * u0;
-          c = H;
-        }
         for (; c + H <= l; c += 2 * H) {
-          e1 = fma(row[c], A[tri(j1 + c, j)], e1);
-          e0 = fma(row[c + H], A[tri(j1 + c + H, j)], e0);
+          y0 = fma(row[c], xs[c], y0);
+          y1 = fma(row[c + H], xs[c + H], y1);
         }
         if (c <= l) {
-          e1 = fma(row[c], A[tri(j1 + c, j)], e1);
+          y0 = fma(row[c], xs[c], y0);
           c += H;
         }
         for (; c + H < m; c += 2 * H) {
-          const int b1 = tri(j1 + c, 0), b2 = tri(j1 + c + H, 0);
-          e0 = fma(A[b1 + j1 + l], A[b1 + j], e0);
-          e1 = fma(A[b2 + j1 + l], A[b2 + j], e1);
+          y1 = fma(A[tri(j1 + c, j1) + l], xs[c], y1);
+          y0 = fma(A[tri(j1 + c + H, j1) + l], xs[c + H], y0);
         }
-        if (c < m) {
-          const int b1 = tri(j1 + c, 0);
-          e0 = fma(A[b1 + j1 + l], A[b1 + j], e0);
-        }
+        if (c < m) y1 = fma(A[tri(j1 + c, j1) + l], xs[c], y1);
       }
-      double e = e0 + e1;
-      for (int o = 1; o < H; o <<= 1) e += __shfl_xor_sync(kFull, e, o);
+      double y = y0 + y1;
+      for (int o = 1; o < H; o <<= 1) y += __shfl_xor_sync(kFull, y, o);
       if (l < m && h == 0) {
-        const double p = tau * e, ul = l == 0 ? u0 : A[tri(j1 + l, j)];
-        wk.pw[l] = p;
-        wk.vv[l] = ul;
-        part = fma(p, ul, part);
+        uw[l].y = y;
+        if (l == 0) scA[3] = y;
+        q = fma(xs[l], y, q);
+      }
+      l0 += nt / H;
+    }
+    if (warp * 32 < m * row_split(min(m, nt), nt) || m > nt) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(kFull, q, o);
+    }
+    if (lane == 0) scQ[warp] = q;
+    grp_sync<MULTI>(g);
+    // 2. u and w
+    if (warp * 32 < m) {
+      const double alpha = scA[0], u0 = scA[1], tau = scA[2];
+      double xy = scQ[0];
+      for (int w = 1; w < nw; ++w) xy += scQ[w];
+      // K = tau^2 / 2 (x^T y + alpha (alpha a_00 - 2 y_0))
+      const double uAu = fma(alpha, fma(alpha, A[tri(j1, j1)], -2.0 * scA[3]), xy);
+      const double nK = (-0.5 * tau) * (tau * uAu);
+      for (int l = tid; l < m; l += nt) {
+        const double u = l == 0 ? u0 : xs[l];
+        const double p = tau * fma(-alpha, A[tri(j1 + l, j1)], uw[l].y);
+        uw[l] = make_double2(u, fma(nK, u, p));
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
-    if (lane == 0) scP[warp] = part;
     grp_sync<MULTI>(g);
-    double pv = 0.0;
-    for (int w = 0; w < nw; ++w) pv += scP[w];
-    const double Kc = 0.5 * tau * pv;
-    for (int l = tid; l < m; l += nt) wk.pw[l] = fma(-Kc, wk.vv[l], wk.pw[l]);
-    grp_sync<MULTI>(g);
-    // A22 -= u w^T + w u^T (u in vv, w in pw): column 0 of A22 -- the next
-    // step's column -- row r by thread r mod nt, with the partials of s; then
-    // the rest of the packed triangle (rows and columns 1..m-1), in the
-    // folded order of FoldWalk
-    const double* uu = wk.vv;
-    const double* ww = wk.pw;
-    double sp = 0.0;
+    // 3. A22 -= u w^T + w u^T: the first column (the next x), then the rest of
+    // the packed triangle (rows and columns 1..m-1) in the folded order of FoldWalk
+    float part = 0.0f;
+    const double2 c0 = uw[0];
     for (int r = tid; r < m; r += nt) {
       double* a = A + tri(j1 + r, j1);
-      const double x = fma(-uu[r], ww[0], fma(-ww[r], u0, *a));
-      *a = x;
-      if (r >= 2) sp = fma(x, x, sp);
+      const double2 ur = uw[r];
+      const double x = fma(-ur.x, c0.y, fma(-ur.y, c0.x, *a));
+      if (r == 0) *a = x;
+      else xs[r - 1] = x;
+      if (r >= 2) {
+        const float f = lead32(x);
+        part = fmaf(f, f, part);
+      }
     }
     const int ntri = (m - 1) * m / 2;
     FoldWalk fw(m - 1, tid, nt);
-    for (int q = tid; q < ntri; q += nt, fw.next()) {
+    for (int e = tid; e < ntri; e += nt, fw.next()) {
       int r, c;
       fw.rc(r, c);
       double* a = A + tri(j1 + 1 + r, j1 + 1 + c);
-      *a = fma(-uu[r + 1], ww[c + 1], fma(-ww[r + 1], uu[c + 1], *a));
+      const double2 ur = uw[r + 1], uc = uw[c + 1];
+      *a = fma(-ur.x, uc.y, fma(-ur.y, uc.x, *a));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sp += __shfl_xor_sync(kFull, sp, o);
-    if (lane == 0) scS[warp] = sp;
+    column_sum(part);
     grp_sync<MULTI>(g);
-    s = 0.0;
-    for (int w = 0; w < nw; ++w) s += scS[w];
   }
   if (tid == 0) {
     wk.d[N - 2] = A[tri(N - 2, N - 2)];
     wk.d[N - 1] = A[tri(N - 1, N - 1)];
-    wk.e[N - 2] = A[tri(N - 1, N - 2)];
+    wk.e[N - 2] = xs[0];
     wk.e[N - 1] = 0.0;
-    // Gershgorin interval
-    double lo = 1e300, hi = -1e300;
-    for (int i = 0; i < N; ++i) {
-      const double r = fabs(wk.e[i]) + (i > 0 ? fabs(wk.e[i - 1]) : 0.0);
-      lo = fmin(lo, wk.d[i] - r);
-      hi = fmax(hi, wk.d[i] + r);
-    }
-    wk.sc[0] = lo;
-    wk.sc[1] = hi;
   }
   grp_sync<MULTI>(g);
-  // squared off-diagonals for the Sturm recurrence (reuse vv), FP32 copies
+  float lo = 3e38f, hi = -3e38f;
   for (int i = tid; i < N; i += nt) {
-    wk.vv[i] = wk.e[i] * wk.e[i];
-    wk.d32[i] = (float)wk.d[i];
-    wk.e32[i] = (float)(wk.e[i] * wk.e[i]);
+    const double d = wk.d[i], r = fabs(wk.e[i]) + (i > 0 ? fabs(wk.e[i - 1]) : 0.0);
+    lo = fminf(lo, (float)(d - r));
+    hi = fmaxf(hi, (float)(d + r));
   }
-  const double glo = wk.sc[0], ghi = wk.sc[1];
+  group_interval<MULTI>(lo, hi, g, reinterpret_cast<float*>(scQ));
+  // the tridiagonal scaled by 2^-ks to a spectrum inside [-1, 1]: d and e^2 in
+  // the matrix's storage, FP32 copies for isolation
+  const float big = fmaxf(fabsf(lo), fabsf(hi));
+  const int ks = big > 0.0f ? (int)((__float_as_uint(big) >> 23) & 0xffu) - 127 + 2 : 0;
+  const double s1 = ldexp(1.0, -ks);
+  double* ds = A;
+  double* es = A + N;
+  float2* de = reinterpret_cast<float2*>(xs);
+  for (int i = tid; i < ((N + 7) & ~7); i += nt) {
+    float2 t = make_float2(2.0f, 0.0f);
+    if (i < N) {
+      const double d = wk.d[i] * s1, e = wk.e[i] * s1;
+      ds[i] = d;
+      es[i] = e * e;
+      const double em = i > 0 ? wk.e[i - 1] * s1 : 0.0;
+      t = make_float2((float)d, (float)(em * em));
+    }
+    de[i] = t;
+  }
   grp_sync<MULTI>(g);
-  const EigGrid gr = eig_grid(wk, N, glo, ghi, tid, nt);
+  EigGrid gr(de, A, N, lo * (float)s1, hi * (float)s1, nt);
+  gr.fill(tid);
   grp_sync<MULTI>(g);
+  const float range = gr.hi - gr.lo;
+  const double tol = 0x1p-50 * (double)(range + fabsf(gr.lo)), back = ldexp(1.0, ks + 2 * kJ);
+  // each step shrinks the error at least as it did the one before: done when the
+  // next one would be below FP64's spacing
+  auto newton = [&](float x0) {
+    double x = (double)x0;
+    float prev = 0.0f;
+    for (int it = 0; it < 6; ++it) {
+      const float step = newton_step64(ds, es, de, N, x);
+      x -= (double)step;
+      if (!(step * step > 0x1p-54f * range * prev)) break;
+      prev = fabsf(step);
+    }
+    return x;
+  };
   double lp = 0.0, en = 0.0, cf = 0.0;
-  for (int idx = tid; idx < N; idx += nt) {
-    const double mu = fmax(eigen_idx(wk, gr, N, idx, glo, ghi), 0.0);
-    const double eps = sqrt(mu);
-    if (eps_out) eps_out[idx] = eps;
-    thermal_add(eps, beta, lp, en, cf);
+  for (int base = 32 * warp; base < N; base += nt) {
+    const int idx = base + lane;
+    const double x = warp_eigenvalues(gr, idx, range * 0x1p-22f, 4.0 * tol, tol, newton,
+                                      [&](double at) { return sturm_count(ds, es, N, at); });
+    if (idx < N) {
+      const double eps = sqrt(fmax(x, 0.0) * back);
+      if (eps_out) eps_out[idx] = eps;
+      thermal_add(eps, beta, lp, en, cf);
+    }
   }
-  res[0] = grp_sum<MULTI>(lp, g, wk.sc);
-  res[1] = grp_sum<MULTI>(en, g, wk.sc);
-  res[2] = grp_sum<MULTI>(cf, g, wk.sc);
+  float none = 0.0f;
+  group_thermal<MULTI>(lp, en, cf, none, g, wk.sc);
+  res[0] = lp;
+  res[1] = en;
+  res[2] = cf;
 }
 
 }  // namespace crbm

@@ -13,6 +13,7 @@
 #pragma once
 #include "crbm_device.cuh"
 #include "crbm_df64.cuh"
+#include "crbm_open64.cuh"
 #include "crbm_local.cuh"
 #include "crbm_kernels.h"
 
@@ -40,11 +41,13 @@ __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(
 
 // Shared-memory work areas of one Kitaev chain (one per thread group of the
 // CTA): the packed lower triangle of A (N (N+1) / 2 FP64 or double-FP32
-// entries), d, e, vv, pw (N each), 64 doubles of reduction scratch, the FP32
-// tridiagonal copies (N each) and the proposed spectrum of a local sweep (N).
+// entries), d, e, (u, w), 64 doubles of scratch, the current column (or the
+// FP32 tridiagonal padded to a multiple of 8) and the proposed spectrum of a
+// local sweep (N).
 __host__ __device__ inline size_t kitaev_work_bytes(int N) {
   const size_t n = (size_t)N;
-  return align16(n * (n + 1) / 2 * 8) + 4 * align16(n * 8) + align16(64 * 8) + 2 * align16(n * 4) + align16(n * 8);
+  return align16(n * (n + 1) / 2 * 8) + 2 * align16(n * 8) + n * 16 + align16(64 * 8) + align16((n + 8) * 8) +
+         align16(n * 8);
 }
 
 // The mixed path's FP64 free energy (rare), out of line to spare registers.
@@ -73,6 +76,15 @@ __device__ __forceinline__ double ising_energy(const JobDev& jb, int pairs) {
   return -jb.J[0] * (double)(2 * jb.N - 2 * pairs);
 }
 
+// log pi, e and c_f of a Kitaev lattice in FP64, valid in the group's leader
+// (the open lattices' jobs run in FP64 only).
+template <int PREC, bool MULTI>
+__device__ __forceinline__ void fp64_spectrum(const JobDev& jb, const Grp& g, const uint32_t* v, double beta,
+                                              const KitaevWork& wk, double (&res)[3], double* eps_out) {
+  if (PREC == kFP64 && jb.lc_edge) kitaev_logpi64_open<MULTI>(g, v, jb.L, jb.J, beta, wk, res, eps_out);
+  else kitaev_logpi64<MULTI>(g, v, jb.L, jb.J, beta, wk, res, eps_out);
+}
+
 // AUX = 0: the proposal loop (mode 0) only; AUX = 1: modes 1-3.  Two kernels,
 // so that the hot proposal loop carries none of the other modes' code and
 // registers (with them it spilled).  MULTI (Kitaev, mode 0 only): CTAs hold
@@ -95,16 +107,13 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
   tb.fd = tb.bd = tb.fh = tb.fl = nullptr;
   tb.fd4 = tb.fh4 = tb.fl4 = nullptr;
   const int nq = jb.k * T;   // entries of a filter-interleaved table
-  double* t64[2] = {nullptr, nullptr};
   float* t32[4] = {nullptr, nullptr, nullptr, nullptr};
   float4* t4[3] = {nullptr, nullptr, nullptr};
   if (PREC == kFP64) {
-    for (int i = 0; i < 2; ++i) {
-      t64[i] = (double*)sp;
-      sp += align16((size_t)nlut * 8);
-    }
-    tb.f64 = t64[0];
-    tb.b64 = t64[1];
+    // read through L1: the FP64 pipe, not the tables, paces the FP64 phases, and
+    // an LCRBM's 36 KB of them per CTA left half of the chains waiting for an SM
+    tb.f64 = jb.f64;
+    tb.b64 = jb.b64;
   } else if (KC == 4) {
     for (int i = 0; i < 3; ++i) {
       t4[i] = (float4*)sp;
@@ -151,32 +160,27 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     kp += align16((size_t)N * 8);
     wk.e = (double*)kp;
     kp += align16((size_t)N * 8);
-    wk.vv = (double*)kp;
-    kp += align16((size_t)N * 8);
-    wk.pw = (double*)kp;
-    kp += align16((size_t)N * 8);
+    wk.uw = (double*)kp;
+    kp += (size_t)N * 16;
     wk.sc = (double*)kp;
     kp += align16(64 * 8);
-    wk.d32 = (float*)kp;
-    kp += align16((size_t)N * 4);
-    wk.e32 = (float*)kp;
-    kp += align16((size_t)N * 4);
+    wk.xs = (double*)kp;
+    kp += align16((size_t)(N + 8) * 8);
     eps_st = (double*)kp;
   }
   uint32_t* my = planes + (size_t)g.gl * (2 + K) * P;
   ChainSm& ch = cs[g.gl];
 
-  for (int i = tid; i < nlut; i += NT) {
-    if (PREC == kFP64) {
-      t64[0][i] = jb.f64[i];
-      t64[1][i] = jb.b64[i];
-    } else if (KC == 4) {
-      t32[1][i] = jb.bd[i];
-    } else {
-      t32[0][i] = jb.fd[i];
-      t32[1][i] = jb.bd[i];
-      t32[2][i] = jb.fh[i];
-      t32[3][i] = jb.fl[i];
+  if (PREC == kMixed) {
+    for (int i = tid; i < nlut; i += NT) {
+      if (KC == 4) {
+        t32[1][i] = jb.bd[i];
+      } else {
+        t32[0][i] = jb.fd[i];
+        t32[1][i] = jb.bd[i];
+        t32[2][i] = jb.fh[i];
+        t32[3][i] = jb.fl[i];
+      }
     }
   }
   if (PREC == kMixed && KC == 4) {
@@ -232,8 +236,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
     if (KIND == kKitaev)
-      kitaev_logpi64<MULTI>(g, my, jb.L, jb.J, g.active ? ch.beta : 1.0, wk, kr,
-                     g.active ? jb.eps + (size_t)g.c * N : nullptr, jb.lc_edge > 0);
+      fp64_spectrum<PREC, MULTI>(jb, g, my, g.active ? ch.beta : 1.0, wk, kr, g.active ? jb.eps + (size_t)g.c * N : nullptr);
     if (g.active && g.r == 0) {
       const double F = free_value<PREC>(jb.vb, fs);
       const double E = KIND == kIsing ? ising_energy(jb, fs.pairs) : kr[1];
@@ -277,8 +280,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
     if (KIND == kKitaev)
-      kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, g.active ? ch.beta : 1.0, wk, kr,
-                     g.active ? jb.eps + (size_t)g.c * N : nullptr, jb.lc_edge > 0);
+      fp64_spectrum<PREC, MULTI>(jb, g, vp, g.active ? ch.beta : 1.0, wk, kr, g.active ? jb.eps + (size_t)g.c * N : nullptr);
     // the physical chain's lattice into the first hidden plane (free now)
     if (g.active)
       for (int w = g.r; w < jb.Wd; w += g.tpc) h[w] = xj.bits[(size_t)g.c * jb.Wd + w];
@@ -405,10 +407,10 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         grp_sync<MULTI>(g);
         double kr[4] = {0.0, 0.0, 0.0, 0.0};
         if (PREC == kMixed) {
-          kitaev_logpi_df<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, kr, jb.lc_edge > 0);
+          kitaev_logpi_df<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, kr);
         } else {
           double k3[3];
-          kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, k3, eps_st, jb.lc_edge > 0);
+          fp64_spectrum<PREC, MULTI>(jb, g, vp, ch.beta, wk, k3, eps_st);
           kr[0] = k3[0];
           kr[1] = k3[1];
           kr[2] = k3[2];
@@ -437,8 +439,8 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
           // when its log-weight came from the df64 stage)
           double k1v[3], k0v[3] = {0.0, 0.0, 0.0};
           const bool redo_v = ch.lpb != 0.0;
-          kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, k1v, eps_st, jb.lc_edge > 0);
-          if (redo_v) kitaev_logpi64<MULTI>(g, v, jb.L, jb.J, ch.beta, wk, k0v, nullptr, jb.lc_edge > 0);
+          fp64_spectrum<PREC, MULTI>(jb, g, vp, ch.beta, wk, k1v, eps_st);
+          if (redo_v) fp64_spectrum<PREC, MULTI>(jb, g, v, ch.beta, wk, k0v, nullptr);
           if (g.r == 0) {
             ch.lpp = k1v[0];
             ch.lppb = 0.0;
@@ -576,10 +578,10 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     double kr[4] = {0.0, 0.0, 0.0, 0.0};
     if (KIND == kKitaev) {
       if (PREC == kMixed) {
-        kitaev_logpi_df<MULTI>(g, vp, jb.L, jb.J, g.active ? ch.beta : 1.0, wk, kr, jb.lc_edge > 0);
+        kitaev_logpi_df<MULTI>(g, vp, jb.L, jb.J, g.active ? ch.beta : 1.0, wk, kr);
       } else {
         double k3[3];
-        kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, g.active ? ch.beta : 1.0, wk, k3, nullptr, jb.lc_edge > 0);
+        fp64_spectrum<PREC, MULTI>(jb, g, vp, g.active ? ch.beta : 1.0, wk, k3, nullptr);
         kr[0] = k3[0];
         kr[1] = k3[1];
         kr[2] = k3[2];
@@ -675,8 +677,8 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         double k1v[3] = {0.0, 0.0, 0.0}, k0v[3] = {0.0, 0.0, 0.0};
         const bool redo_v = ch.lpb != 0.0;
         if (KIND == kKitaev) {
-          kitaev_logpi64<MULTI>(g, vp, jb.L, jb.J, ch.beta, wk, k1v, nullptr, jb.lc_edge > 0);
-          if (redo_v) kitaev_logpi64<MULTI>(g, v, jb.L, jb.J, ch.beta, wk, k0v, nullptr, jb.lc_edge > 0);
+          fp64_spectrum<PREC, MULTI>(jb, g, vp, ch.beta, wk, k1v, nullptr);
+          if (redo_v) fp64_spectrum<PREC, MULTI>(jb, g, v, ch.beta, wk, k0v, nullptr);
         }
         if (g4.active && g.r == 0) {
           ch.Fp = free_value<kFP64>(jb.vb, f1);
