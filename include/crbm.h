@@ -156,7 +156,10 @@ CRBM_API int crbm_run(crbm_ctx* ctx, int job_id, int64_t S, int g, int correct, 
 
 /* As crbm_run for n_jobs jobs, chains of different L and temperature side
  * by side: the jobs on the tensor-core form (crbm_set_tensor_cores) share ONE
- * persistent launch whatever their sides; the other jobs share one launch
+ * persistent launch whatever their sides; a call of mixed-precision Ising jobs
+ * of other shapes with L a multiple of 32 and no more chains than the device
+ * runs clusters for divides each chain over a cluster of up to 8 CTAs (the same
+ * decisions); the other jobs share one launch
  * (Kitaev: one chain per CTA of its thread-group size when the jobs' group
  * sizes agree, else 256-thread CTAs holding several chain groups); when both
  * kinds of launch are needed they

@@ -21,6 +21,7 @@ SOURCES = ["crbm_kernels.cu", "crbm_api.cu", "crbm_tempering.cu", "crbm_analysis
            "crbm_sweep.cu",
            "crbm_step_ising_fp64_t256.cu",
            "crbm_step_ising_mixed_t256.cu",
+           "crbm_step_slab.cu",
            "crbm_step_tc.cu",
            "crbm_step_kitaev_fp64_t256.cu",
            "crbm_step_kitaev_fp64_t128.cu",

@@ -142,10 +142,13 @@ struct crbm_ctx {
   std::vector<Graph> graphs;
   // chains per CTA chosen by crbm_tune for (kind, L, K, k)
   std::map<std::tuple<int, int, int, int>, int> tuned;
+  // clusters that run side by side, by (K, k, CTAs per cluster, shared memory)
+  std::map<std::tuple<int, int, int, size_t>, int> slab_fits;
   // proposals of eligible jobs (crbm_step_tc.cu) run on the tensor-core form;
   // tc_ok: the device grants its shared memory
   bool use_tc = true, tc_ok = false;
   int sms = 1;                          // SMs of the device: persistent grid size
+  size_t smem_optin = 0;                // shared memory a CTA may have
   long long wait_limit = 1ll << 28;     // cycles before a device-side wait gives up
   // device buffer of crbm_read_energies' FP64 re-evaluation (a copy of one
   // job's memory), grown on demand
@@ -378,21 +381,93 @@ static int launch_tc_group(crbm_ctx* ctx, std::vector<int> ids, int S, int g, in
   return CRBM_OK;
 }
 
+// CTAs per chain of the jobs' proposals (crbm_step_slab.cu): the largest cluster
+// size at which every chain of the call has a cluster running side by side with
+// the others (a GPC holds whole clusters: 15 of eight CTAs, not 19), at most
+// what each job's side allows; 0 for calls with more chains, and with jobs of
+// the tensor-core form, FP64 or other sides, which keep their kernels.  Every
+// kernel takes the same decisions, so the results do not depend on the choice.
+// (L = 256, K = 4 5x5, us per proposal: 15 chains 37 at 8; 16 chains 72 at 8 in
+// two waves, 62 at 4, 49 at the size this picks; 76 chains 116, 152 chains 218;
+// one 256-thread CTA per chain 310 to 319, from 153 chains on 445.  L = 96: 13 for
+// 16 chains, 44 for 152, against 48 and 57.)
+static int slab_size(crbm_ctx* ctx, const std::vector<int>& ids, int prec, int mode) {
+  if (mode != 0 || prec != kMixed) return 0;
+  long long chains = 0;
+  size_t smem = 0;
+  int most = 8, K = 0, k = 0;
+  for (int id : ids) {
+    const Job& j = ctx->jobs[id];
+    const Model& m = ctx->models[j.model];
+    if (j.n == 0) continue;
+    if (j.kind != kIsing || tc_supported(j.kind, prec, j.L, m.K, m.k)) return 0;
+    K = m.K;
+    k = m.k;
+    most = std::min(most, slab_most(j.L, K, k, ctx->smem_optin));
+    smem = std::max(smem, slab_smem_bytes(j.L, K, k));
+    chains += j.n;
+  }
+  if (chains == 0 || chains > ctx->sms) return 0;
+  for (int CL = most; CL >= 1; --CL) {
+    if (chains * CL > ctx->sms) continue;
+    const auto key = std::make_tuple(K, k, CL, smem);
+    auto it = ctx->slab_fits.find(key);
+    if (it == ctx->slab_fits.end()) {
+      int fit = 0;
+      if (slab_fit(K, k, CL, smem, &fit) != cudaSuccess) {
+        cudaGetLastError();
+        fit = 0;
+      }
+      it = ctx->slab_fits.emplace(key, fit).first;
+    }
+    if (chains <= it->second) return CL;
+  }
+  return 0;
+}
+
+// One launch of the jobs' chains in clusters of CL CTAs.
+static int launch_slab_group(crbm_ctx* ctx, const std::vector<int>& ids, int S, int g, int correct, int CL,
+                             cudaStream_t st) {
+  LaunchParams p;
+  memset(&p, 0, sizeof p);
+  p.n_jobs = (int)ids.size();
+  p.S = S;
+  p.g = g;
+  p.correct = correct;
+  p.err = ctx->d_err;
+  int chains = 0;
+  size_t smem = 0;
+  for (size_t i = 0; i < ids.size(); ++i) {
+    const Job& j = ctx->jobs[ids[i]];
+    p.tile_begin[i] = chains;
+    p.job[i] = make_jobdev(ctx, j);
+    chains += j.n;
+    smem = std::max(smem, slab_smem_bytes(j.L, ctx->models[j.model].K, ctx->models[j.model].k));
+  }
+  p.tile_begin[ids.size()] = chains;
+  if (chains == 0 || S == 0) return CRBM_OK;
+  CK(launch_slab(p, chains, CL, smem, st), "kernel launch");
+  return CRBM_OK;
+}
+
 static int launch_jobs(crbm_ctx* ctx, const std::vector<int>& ids, int S, int g, int correct, int prec, int mode,
                        cudaStream_t st, const Job* partner = nullptr) {
-  // parts: (CTA size, jobs); CTA size -1 = the tensor-core form (one persistent launch for every side)
+  // parts: (CTA size, jobs); CTA size -1 = the tensor-core form (one persistent
+  // launch for every side), -2 = every job's chains in clusters
   std::vector<std::pair<int, std::vector<int>>> parts;
-  for (int nt : {-1, 256, 128, 64, 32}) {
+  const int slab = partner ? 0 : slab_size(ctx, ids, prec, mode);
+  auto part_of = [&](const Job& j) {
+    if (slab > 0) return -2;
+    return !partner && on_tc(ctx, j, prec, mode) ? -1 : threads_for(j.kind, j.N);
+  };
+  for (int nt : {-2, -1, 256}) {
     std::vector<int> part;
-    for (int id : ids) {
-      const Job& j = ctx->jobs[id];
-      if (j.n == 0) continue;
-      const bool tc = !partner && on_tc(ctx, j, prec, mode);
-      if (nt < 0 ? tc : (!tc && threads_for(j.kind, j.N) == nt)) part.push_back(id);
-    }
+    for (int id : ids)
+      if (ctx->jobs[id].n > 0 && part_of(ctx->jobs[id]) == nt) part.push_back(id);
     if (!part.empty()) parts.emplace_back(nt, part);
   }
   auto launch_part = [&](const std::pair<int, std::vector<int>>& pt, cudaStream_t s) {
+    if (pt.first == -2) return launch_slab_group(ctx, pt.second, S, g, correct, slab, s);
     return pt.first < 0 ? launch_tc_group(ctx, pt.second, S, g, correct, mode, s)
                         : launch_group(ctx, pt.second, S, g, correct, prec, mode, pt.first, s, partner);
   };
@@ -441,7 +516,9 @@ int crbm_create(crbm_ctx** out, int device, size_t hbm_budget_bytes) {
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, device);
     if (ctx->sms < 1) ctx->sms = 1;
+    ctx->smem_optin = (size_t)optin;
     e = set_smem_limits((size_t)optin);
+    if (e == cudaSuccess) e = slab_set_smem_limit((size_t)optin);
     if (e == cudaSuccess && (size_t)optin >= tc_smem_bytes(128, 4, 5)) {
       e = tc_set_smem_limit();
       ctx->tc_ok = e == cudaSuccess;

@@ -565,18 +565,17 @@ __device__ void hidden_phase64(const JobDev& jb, const Tabs& tb, const Grp& g, c
   }
 }
 
-// Mixed form: thread = unit of 4 sites.  KC, kC > 0 fix K and k at compile
-// time (0: runtime).
+// Mixed form: thread = unit of 4 sites, units q0 .. q1 - 1.  KC, kC > 0 fix K
+// and k at compile time (0: runtime).
 template <int KC, int kC>
 __device__ void hidden_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v,
-                             uint32_t* h, int P, uint32_t step, int sub, unsigned& nrec) {
+                             uint32_t* h, int P, uint32_t step, int sub, unsigned& nrec, int q0, int q1) {
   constexpr int kU = kC ? kC : kMaxk;
   const int L = jb.L, N = jb.N, K = KC ? KC : jb.K, k = kC ? kC : jb.k, T = tb.T;
-  const int nblk = (N + 3) >> 2;
-  const int iters = (nblk + g.tpc - 1) / g.tpc;
+  const int iters = (q1 - q0 + g.tpc - 1) / g.tpc;
   for (int it = 0; it < iters; ++it) {
-    const int q = g.r + it * g.tpc;
-    const bool act = g.active && q < nblk;
+    const int q = q0 + g.r + it * g.tpc;
+    const bool act = g.active && q < q1;
     uint32_t m[4][kU];
     fwd_codes<kC>(v, L, N, k, T, act ? q : 0, m);
     if (KC == 4) {
@@ -673,20 +672,19 @@ __device__ void visible_phase64(const JobDev& jb, const Tabs& tb, const Grp& g, 
   }
 }
 
-// Mixed form: thread = unit of 4 sites.
+// Mixed form: thread = unit of 4 sites, units q0 .. q1 - 1.
 template <int KC, int kC>
 __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* h,
-                              uint32_t* vp, int P, uint32_t step, int sub, unsigned& nrec) {
+                              uint32_t* vp, int P, uint32_t step, int sub, unsigned& nrec, int q0, int q1) {
   constexpr int kU = kC ? kC : kMaxk;
   constexpr int KU = KC ? KC : kMaxK;
   const int L = jb.L, N = jb.N, K = KC ? KC : jb.K, k = kC ? kC : jb.k, T = tb.T;
   const uint32_t mk = (1u << k) - 1u;
-  const int nblk = (N + 3) >> 2;
-  const int iters = (nblk + g.tpc - 1) / g.tpc;
+  const int iters = (q1 - q0 + g.tpc - 1) / g.tpc;
   const bool rows4 = (L & 3) == 0;
   for (int it = 0; it < iters; ++it) {
-    const int q = g.r + it * g.tpc;
-    const bool act = g.active && q < nblk;
+    const int q = q0 + g.r + it * g.tpc;
+    const bool act = g.active && q < q1;
     const int qq = act ? q : 0;
     float x32[4];
 #pragma unroll
@@ -775,16 +773,17 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
 // F(v) = -v_bias sum v - sum_{f,i,j} softplus(h_bias^f + (W^f * v)_ij)   (Eq. 13)
 // Per-thread partial sums: softplus (FreeSum), the number of ones and of
 // unequal nearest-neighbour pairs (Ising) or of hexagons with flux -1 (Kitaev).
-// FP64 form: thread (filter, site); the log(1 + e^-|x|) of a thread's units are
+// FP64 form: thread (filter, site), sites n0 .. n1 - 1; the log(1 + e^-|x|) of a thread's units are
 // the log of their product (factors in (1, 2], the log taken at least every 512).
-__device__ inline FreeSum free_phase64(const JobDev& jb, const double* f64, const Grp& g, const uint32_t* v) {
-  const int L = jb.L, N = jb.N, K = jb.K, k = jb.k, T = 1 << k;
+__device__ inline FreeSum free_phase64(const JobDev& jb, const double* f64, const Grp& g, const uint32_t* v, int n0,
+                                       int n1) {
+  const int L = jb.L, K = jb.K, k = jb.k, T = 1 << k;
   FreeSum out = {0.0, 0ll, 0.0f, 0, 0};
   if (!g.active) return out;
   double prod = 1.0;
   int held = 0;
-  for (int e = g.r; e < K * N; e += g.tpc) {
-    const int f = e / N, n = e - f * N, i = n / L, j = n - i * L;
+  for (int e = g.r; e < K * (n1 - n0); e += g.tpc) {
+    const int f = e / (n1 - n0), n = n0 + e - f * (n1 - n0), i = n / L, j = n - i * L;
     double x = jb.hb[f];
     if (jb.lc_edge) {
       x = lc_preact64(jb, f64, f, v, n, k, T);
@@ -803,7 +802,7 @@ __device__ inline FreeSum free_phase64(const JobDev& jb, const double* f64, cons
     }
   }
   if (held) out.s += log(prod);
-  for (int n = g.r; n < N; n += g.tpc) {
+  for (int n = n0 + g.r; n < n1; n += g.tpc) {
     const int i = n / L, j = n - i * L, jr = j + 1 == L ? 0 : j + 1;
     const uint32_t b0 = site_bit(v, n);
     out.ones += (int)b0;
@@ -828,18 +827,18 @@ __device__ __forceinline__ double free_constant(const JobDev& jb, int tpc) {
   return (double)jb.K * (double)jb.N * (1.5 * 0x1p-23 + (double)jb.csp) + (double)tpc * 0x1p-33;
 }
 
-// Mixed form: thread = unit of 4 sites, FP32 with Kahan compensation.
+// Mixed form: thread = unit of 4 sites, units q0 .. q1 - 1, FP32 with Kahan
+// compensation.
 template <int KC, int kC>
-__device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v) {
+__device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v, int q0, int q1) {
   constexpr int kU = kC ? kC : kMaxk;
   const int L = jb.L, N = jb.N, K = KC ? KC : jb.K, k = kC ? kC : jb.k, T = tb.T;
-  const int nblk = (N + 3) >> 2;
-  const int iters = (nblk + g.tpc - 1) / g.tpc;
+  const int iters = (q1 - q0 + g.tpc - 1) / g.tpc;
   float s32 = 0.0f, c32 = 0.0f, sabs = 0.0f, ssp = 0.0f;
   int ones = 0, pairs = 0;
   for (int it = 0; it < iters; ++it) {
-    const int q = g.r + it * g.tpc;
-    const bool act = g.active && q < nblk;
+    const int q = q0 + g.r + it * g.tpc;
+    const bool act = g.active && q < q1;
     if (!act) continue;
     uint32_t m[4][kU];
     fwd_codes<kC>(v, L, N, k, T, q, m);

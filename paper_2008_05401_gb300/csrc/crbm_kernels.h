@@ -38,6 +38,16 @@ int tc_chains_per_cta(int L);
 size_t tc_smem_bytes(int L, int K, int k);
 cudaError_t launch_tc(const LaunchParams& p, int grid, size_t smem, cudaStream_t st);
 cudaError_t tc_set_smem_limit();
+// Ising proposals (mixed precision, mode 0) with each chain divided over a
+// cluster of CL CTAs (crbm_step_slab.cu): the most CTAs a chain of side L takes
+// (0: not served; smem_limit: shared memory a CTA may have), a CTA's dynamic
+// shared memory, the clusters that the device runs side by side, and the launch
+// of p's jobs (tile_begin counts chains), their step counters after it.
+int slab_most(int L, int K, int k, size_t smem_limit);
+size_t slab_smem_bytes(int L, int K, int k);
+cudaError_t slab_fit(int K, int k, int CL, size_t smem, int* clusters);
+cudaError_t launch_slab(const LaunchParams& p, int chains, int CL, size_t smem, cudaStream_t st);
+cudaError_t slab_set_smem_limit(size_t bytes);
 // One CTA waiting on an mbarrier with the tensor-core pipeline's bounded wait
 // (arrive = 0: nothing arrives; after `limit` cycles *err = timeout).
 cudaError_t launch_wait_probe(long long limit, int arrive, int* err, cudaStream_t st);

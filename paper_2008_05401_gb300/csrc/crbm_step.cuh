@@ -51,8 +51,9 @@ __host__ __device__ inline size_t kitaev_work_bytes(int N) {
 }
 
 // The mixed path's FP64 free energy (rare), out of line to spare registers.
-static __device__ __noinline__ void free_energy64(const JobDev& jb, const Grp& g, const uint32_t* v, FreeSum* out) {
-  *out = free_phase64(jb, jb.f64, g, v);
+static __device__ __noinline__ void free_energy64(const JobDev& jb, const Grp& g, const uint32_t* v, int n0, int n1,
+                                                  FreeSum* out) {
+  *out = free_phase64(jb, jb.f64, g, v, n0, n1);
 }
 
 // Observables of a lattice: Ising from E and the number of ones; Kitaev from
@@ -76,6 +77,48 @@ __device__ __forceinline__ double ising_energy(const JobDev& jb, int pairs) {
   return -jb.J[0] * (double)(2 * jb.N - 2 * pairs);
 }
 
+// The mixed path's FP32 tables at sp (copied by the CTA's nt threads; a barrier
+// before their first use is the caller's), their pointers into tb; returns the
+// end of the area.
+template <int KC>
+__device__ __forceinline__ unsigned char* mixed_tables(const JobDev& jb, unsigned char* sp, Tabs& tb, int tid, int nt) {
+  const int T = 1 << jb.k, nlut = jb.K * jb.k * T, nq = jb.k * T;   // nq: entries of a filter-interleaved table
+  auto take = [&](size_t bytes) {
+    unsigned char* at = sp;
+    sp += align16(bytes);
+    return at;
+  };
+  if (KC == 4) {
+    float4* t4[3];
+    for (int i = 0; i < 3; ++i) t4[i] = (float4*)take((size_t)nq * 16 * 8);      // 8 bank-interleaved copies
+    float* bd = (float*)take((size_t)nlut * 4);
+    for (int i = tid; i < nlut; i += nt) bd[i] = jb.bd[i];
+    for (int i = tid; i < nq * 8; i += nt) {
+      t4[0][i] = jb.fd4[i >> 3];
+      t4[1][i] = jb.fh4[i >> 3];
+      t4[2][i] = jb.fl4[i >> 3];
+    }
+    tb.fd4 = t4[0] + (tid & 7);
+    tb.fh4 = t4[1] + (tid & 7);
+    tb.fl4 = t4[2] + (tid & 7);
+    tb.bd = bd;
+  } else {
+    float* t[4];
+    for (int i = 0; i < 4; ++i) t[i] = (float*)take((size_t)nlut * 4);
+    for (int i = tid; i < nlut; i += nt) {
+      t[0][i] = jb.fd[i];
+      t[1][i] = jb.bd[i];
+      t[2][i] = jb.fh[i];
+      t[3][i] = jb.fl[i];
+    }
+    tb.fd = t[0];
+    tb.bd = t[1];
+    tb.fh = t[2];
+    tb.fl = t[3];
+  }
+  return sp;
+}
+
 // log pi, e and c_f of a Kitaev lattice in FP64, valid in the group's leader
 // (the open lattices' jobs run in FP64 only).
 template <int PREC, bool MULTI>
@@ -97,7 +140,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
   const JobDev& jb = prm.job[jid];
   const int ltile = (int)blockIdx.x - prm.tile_begin[jid];
   const int tid = threadIdx.x;
-  const int N = jb.N, P = jb.P, K = jb.K, T = 1 << jb.k, nlut = jb.ncls * K * jb.k * T;
+  const int N = jb.N, nblk = (N + 3) >> 2, P = jb.P, K = jb.K, T = 1 << jb.k;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* sp = smem_raw;
@@ -106,34 +149,13 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
   tb.f64 = tb.b64 = nullptr;
   tb.fd = tb.bd = tb.fh = tb.fl = nullptr;
   tb.fd4 = tb.fh4 = tb.fl4 = nullptr;
-  const int nq = jb.k * T;   // entries of a filter-interleaved table
-  float* t32[4] = {nullptr, nullptr, nullptr, nullptr};
-  float4* t4[3] = {nullptr, nullptr, nullptr};
-  if (PREC == kFP64) {
+  if constexpr (PREC == kFP64) {
     // read through L1: the FP64 pipe, not the tables, paces the FP64 phases, and
     // an LCRBM's 36 KB of them per CTA left half of the chains waiting for an SM
     tb.f64 = jb.f64;
     tb.b64 = jb.b64;
-  } else if (KC == 4) {
-    for (int i = 0; i < 3; ++i) {
-      t4[i] = (float4*)sp;
-      sp += align16((size_t)nq * 16 * 8);      // 8 bank-interleaved copies
-    }
-    t32[1] = (float*)sp;
-    sp += align16((size_t)nlut * 4);
-    tb.fd4 = t4[0] + (threadIdx.x & 7);
-    tb.fh4 = t4[1] + (threadIdx.x & 7);
-    tb.fl4 = t4[2] + (threadIdx.x & 7);
-    tb.bd = t32[1];
   } else {
-    for (int i = 0; i < 4; ++i) {
-      t32[i] = (float*)sp;
-      sp += align16((size_t)nlut * 4);
-    }
-    tb.fd = t32[0];
-    tb.bd = t32[1];
-    tb.fh = t32[2];
-    tb.fl = t32[3];
+    sp = mixed_tables<KC>(jb, sp, tb, tid, NT);
   }
   ChainSm* cs = (ChainSm*)sp;
   sp += align16(jb.nc * sizeof(ChainSm));
@@ -171,25 +193,6 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
   uint32_t* my = planes + (size_t)g.gl * (2 + K) * P;
   ChainSm& ch = cs[g.gl];
 
-  if (PREC == kMixed) {
-    for (int i = tid; i < nlut; i += NT) {
-      if (KC == 4) {
-        t32[1][i] = jb.bd[i];
-      } else {
-        t32[0][i] = jb.fd[i];
-        t32[1][i] = jb.bd[i];
-        t32[2][i] = jb.fh[i];
-        t32[3][i] = jb.fl[i];
-      }
-    }
-  }
-  if (PREC == kMixed && KC == 4) {
-    for (int i = tid; i < nq * 8; i += NT) {
-      t4[0][i] = jb.fd4[i >> 3];
-      t4[1][i] = jb.fh4[i >> 3];
-      t4[2][i] = jb.fl4[i >> 3];
-    }
-  }
   for (int i = tid; i < jb.nc * (2 + K) * P; i += NT) planes[i] = 0u;
   __syncthreads();
   if (g.r == 0) {
@@ -231,8 +234,8 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     // as after a mixed proposal), log pi and the observables (FP64) of the
     // current lattices
     FreeSum fs;
-    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, my);
-    else fs = free_phase64(jb, tb.f64, g, my);
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, my, 0, nblk);
+    else fs = free_phase64(jb, tb.f64, g, my, 0, N);
     reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
     if (KIND == kKitaev)
@@ -266,17 +269,17 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     uint32_t* h = my + 2 * P;
     const uint32_t* src = my;
     for (int sub = 0; sub < prm.g; ++sub) {
-      if constexpr (PREC == kMixed) hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec);
+      if constexpr (PREC == kMixed) hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec, 0, nblk);
       else hidden_phase64(jb, tb, g, src, h, P, step, sub, []() { __syncthreads(); });
       __syncthreads();
-      if constexpr (PREC == kMixed) visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec);
+      if constexpr (PREC == kMixed) visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec, 0, nblk);
       else visible_phase64(jb, tb, g, h, vp, P, step, sub, []() { __syncthreads(); });
       __syncthreads();
       src = vp;
     }
     FreeSum fs;
-    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp);
-    else fs = free_phase64(jb, tb.f64, g, vp);
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp, 0, nblk);
+    else fs = free_phase64(jb, tb.f64, g, vp, 0, N);
     reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
     if (KIND == kKitaev)
@@ -316,12 +319,12 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         Grp g2 = g;
         g2.active = g.active && ch.flag_rec;
         FreeSum f1;
-        free_energy64(jb, g2, vp, &f1);
+        free_energy64(jb, g2, vp, 0, N, &f1);
         reduce_free<kFP64, false>(f1, g2, scratch);
         Grp g3 = g2;
         g3.active = g2.active && ch.Fb != 0.0;
         FreeSum f2;
-        free_energy64(jb, g3, h, &f2);
+        free_energy64(jb, g3, h, 0, N, &f2);
         reduce_free<kFP64, false>(f2, g3, scratch);
         if (g2.active && g.r == 0) {
           ch.Fp = free_value<kFP64>(jb.vb, f1);
@@ -489,7 +492,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     }
     // FP64 free energy of the final lattices, then everything back to the job
     FreeSum fs;
-    free_energy64(jb, g, my + ch.cur * P, &fs);
+    free_energy64(jb, g, my + ch.cur * P, 0, N, &fs);
     reduce_free<kFP64, false>(fs, g, scratch);
     if (g.active) {
       const uint32_t* v = my + ch.cur * P;
@@ -563,17 +566,17 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
       if (prm.correct) ch.logu = PREC == kFP64 ? log_u64(step) : (double)log_u32(accept_word(step));
     }
     for (int sub = 0; sub < prm.g; ++sub) {
-      if constexpr (PREC == kMixed) hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec);
+      if constexpr (PREC == kMixed) hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec, 0, nblk);
       else hidden_phase64(jb, tb, g, src, h, P, step, sub, loop_sync);
       loop_sync();
-      if constexpr (PREC == kMixed) visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec);
+      if constexpr (PREC == kMixed) visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec, 0, nblk);
       else visible_phase64(jb, tb, g, h, vp, P, step, sub, loop_sync);
       loop_sync();
       src = vp;
     }
     FreeSum fs;
-    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp);
-    else fs = free_phase64(jb, tb.f64, g, vp);
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp, 0, nblk);
+    else fs = free_phase64(jb, tb.f64, g, vp, 0, N);
     loop_reduce(fs, g, std::integral_constant<int, PREC>());
     double kr[4] = {0.0, 0.0, 0.0, 0.0};
     if (KIND == kKitaev) {
@@ -637,9 +640,9 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         Grp g3 = g2;
         g3.active = g2.active && ch.Fb != 0.0;
         double f1[3], f2[3];
-        free_sum_df<KC ? KC : kMaxK>(jb, g2, vp, f1);
+        free_sum_df<KC ? KC : kMaxK>(jb, g2, vp, 0, N, f1);
         grp_reduce<3>(f1, g2, scratch);
-        free_sum_df<KC ? KC : kMaxK>(jb, g3, v, f2);
+        free_sum_df<KC ? KC : kMaxK>(jb, g3, v, 0, N, f2);
         grp_reduce<3>(f2, g3, scratch);
         if (mine) {
           ch.Fp = -jb.vb * f1[2] - f1[0];
@@ -665,12 +668,12 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         Grp g4 = g2;
         g4.active = g2.active && (KIND == kKitaev || ch.flag_rec == 2);
         FreeSum f1;
-        free_energy64(jb, g4, vp, &f1);
+        free_energy64(jb, g4, vp, 0, N, &f1);
         loop_reduce(f1, g4, std::integral_constant<int, kFP64>());
         Grp g3 = g4;
         g3.active = g4.active && ch.Fb != 0.0;
         FreeSum f2;
-        free_energy64(jb, g3, v, &f2);
+        free_energy64(jb, g3, v, 0, N, &f2);
         loop_reduce(f2, g3, std::integral_constant<int, kFP64>());
         // Kitaev: the FP64 eigen-stage of v' (and of v when its log-weight
         // came from the df64 stage), by the group that needs it

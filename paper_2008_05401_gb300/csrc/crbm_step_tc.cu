@@ -505,7 +505,7 @@ static __device__ __noinline__ void mh_redo(const JobDev& jb, ChainSm* chs, doub
     // decision still straddles (3), since the FP32 bound of F(v) alone is
     // often narrow enough
     double f1[3];
-    free_sum_df<4>(jb, g2, pv + c * G::WPC, f1);
+    free_sum_df<4>(jb, g2, pv + c * G::WPC, 0, LT * LT, f1);
     grp_reduce<3>(f1, g2, scratch);
     if (g2.active && g2.r == 0) {
       ch.Fp = -jb.vb * f1[2] - f1[0];
@@ -517,7 +517,7 @@ static __device__ __noinline__ void mh_redo(const JobDev& jb, ChainSm* chs, doub
       Grp g3 = g2;
       g3.active = g2.active && ch.flag_rec == 3;
       double f2[3];
-      free_sum_df<4>(jb, g3, vbits + c * G::WPC, f2);
+      free_sum_df<4>(jb, g3, vbits + c * G::WPC, 0, LT * LT, f2);
       grp_reduce<3>(f2, g3, scratch);
       if (g3.active && g3.r == 0) {
         ch.F = -jb.vb * f2[2] - f2[0];
@@ -530,12 +530,12 @@ static __device__ __noinline__ void mh_redo(const JobDev& jb, ChainSm* chs, doub
     Grp g4 = g2;
     g4.active = g2.active && ch.flag_rec == 2;
     FreeSum f1;
-    free_energy64(jb, g4, pv + c * G::WPC, &f1);
+    free_energy64(jb, g4, pv + c * G::WPC, 0, LT * LT, &f1);
     reduce_free<kFP64, false>(f1, g4, scratch);
     Grp g3 = g4;
     g3.active = g4.active && ch.Fb != 0.0;
     FreeSum f2;
-    free_energy64(jb, g3, vbits + c * G::WPC, &f2);
+    free_energy64(jb, g3, vbits + c * G::WPC, 0, LT * LT, &f2);
     reduce_free<kFP64, false>(f2, g3, scratch);
     if (g4.active && g4.r == 0) {
       ch.Fp = free_value<kFP64>(jb.vb, f1);

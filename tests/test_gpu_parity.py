@@ -111,6 +111,64 @@ def test_many_ising_chains_match_oracle(ctx, L, K, k, n, g):
         job.release()
 
 
+@pytest.mark.parametrize("L,K,k,n,g,correct", [
+    (32, 5, 3, 3, 1, True),      # clusters of 8, four rows per CTA
+    (32, 2, 6, 2, 1, True),      # k - 1 = 5 rows of halo: clusters of 4
+    (32, 2, 7, 30, 2, False),    # clusters of 4, two Gibbs steps, uncorrected
+    (64, 8, 3, 40, 1, True),     # 40 chains: clusters of 2
+    (96, 4, 5, 4, 2, True),      # rows of three words, twelve rows per CTA
+    (96, 1, 1, 19, 1, True),     # one tap: the halo row only counts pairs; all 152 CTAs
+    (224, 4, 3, 2, 1, True),
+    (256, 4, 5, 3, 1, True),
+])
+def test_divided_chains_match_oracle(ctx, L, K, k, n, g, correct):
+    """Mixed-precision chains divided over a cluster's CTAs (few chains at a side
+    or filter shape the tensor-core form does not have): the oracle's lattices,
+    accepts, energies and sums."""
+    from paper_2008_05401_gb300 import ISING, MIXED
+    W, hb, vb = wl.gaussian_crbm(K, k, 0.15, seed=L + 10 * K + k)
+    T = wl.ising_ladder(n, 8)
+    bits0 = wl.pack_bits(wl.random_lattices(n, L, seed=L))
+    S = 4
+    ref = oracle_chains("ising", W, hb, vb, L, T, (1.0,), SEED, n, bits0)
+    worst = run_oracle(ref, S, g=g, correct=correct)
+    mid = ctx.load_model(ISING, W, vb, hb)
+    job = ctx.new_job(mid, ISING, L, T, (1.0,), SEED, 0, bits0, MIXED)
+    job.run(1, g=g, correct=correct, precision=MIXED)
+    job.run(S - 1, g=g, correct=correct, precision=MIXED)
+    _compare(job, ref, worst, S)
+    job.release()
+
+
+def test_divided_chains_in_a_batch_and_a_graph(ctx):
+    """Jobs of several sides (clusters of 8 and 4 in one call), the same jobs in
+    a call with too many chains for clusters, and a replayed graph: one result."""
+    from paper_2008_05401_gb300 import ISING, MIXED
+    W, hb, vb = wl.gaussian_crbm(2, 6, 0.15, seed=4)
+    mid = ctx.load_model(ISING, W, vb, hb)
+
+    def jobs(sizes):
+        return [ctx.new_job(mid, ISING, L, wl.ising_ladder(n, 8), (1.0,), SEED, 100 * i,
+                            wl.pack_bits(wl.random_lattices(n, L, seed=L)), MIXED) for i, (L, n) in enumerate(sizes)]
+    sizes = [(32, 6), (96, 5), (160, 3)]
+    a, b, c = jobs(sizes), jobs(sizes + [(64, 200)]), jobs(sizes)
+    ctx.run_batch(a, 4, precision=MIXED)
+    ctx.run_batch(b, 4, precision=MIXED)
+    gr = ctx.graph(c, 2, precision=MIXED)
+    gr.launch()
+    gr.launch()
+    for x, y, z in zip(a, b, c):
+        sx, ax, _ = x.observables()
+        for other in (y, z):
+            so, ao, _ = other.observables()
+            np.testing.assert_array_equal(other.state()[0], x.state()[0])
+            np.testing.assert_array_equal(ao, ax)
+            np.testing.assert_array_equal(so, sx)
+    gr.destroy()
+    for j in a + b + c:
+        j.release()
+
+
 KITAEV_CASES = [
     # L, K, k, n, correct
     (2, 2, 2, 6, True),
