@@ -173,6 +173,32 @@ __device__ __forceinline__ uint32_t row_window(const uint32_t* __restrict__ bits
   return x & ((1u << w) - 1u);
 }
 
+// Rows of planes whose side is not a multiple of 32 (L <= 31), each repeated
+// with period L over 64 bits: a window of up to 33 - w columns past any start is
+// one shift, where row_window on the packed plane has to cut the row out and
+// repeat it (up to 60 instructions, taken K k times per site of a visible
+// half-step).  Bound by instruction issue; 1024 chains of L = 24, K = 2, k = 5,
+// 20 proposals: 1.26 -> 1.09 ms; 1024 Kitaev chains of L = 6, 8 proposals (with
+// the warps of an idle unit range left out): 2.19 -> 1.92 ms.  (L >= 32 has rows
+// of whole words, whose window is one funnel shift already.)  By the group's
+// threads, from `planes` planes P words apart.
+__device__ __forceinline__ void expand_rows(const uint32_t* plane, int P, uint64_t* ext, int L, int planes, int r,
+                                            int tpc) {
+  if ((L & 31) == 0) return;
+  for (int e = r; e < planes * L; e += tpc) {
+    const int f = e / L, off = (e - f * L) * L;
+    const uint32_t* p = plane + f * P + (off >> 5);
+    uint64_t x = __funnelshift_r(p[0], p[1], off & 31) & ((1u << L) - 1u);
+    for (int s = L; s < 64; s *= 2) x |= x << s;
+    ext[e] = x;
+  }
+}
+// row_window of a plane with (L not a multiple of 32) or without expanded rows.
+__device__ __forceinline__ uint32_t window(const uint32_t* bits, const uint64_t* ext, int L, int r, int c, int w) {
+  if ((L & 31) == 0) return row_window(bits, L, r, c, w);
+  return (uint32_t)(ext[r] >> c) & ((1u << w) - 1u);
+}
+
 __device__ __forceinline__ uint32_t site_bit(const uint32_t* bits, int n) {
   return (bits[n >> 5] >> (n & 31)) & 1u;
 }
@@ -183,7 +209,7 @@ __device__ __forceinline__ uint32_t site_bit(const uint32_t* bits, int n) {
 // (i_t, j_t).  When L % 4 == 0 the 4 sites share a row and one window of
 // k + 3 bits per kernel row serves all of them.  kC > 0 fixes k at compile time.
 template <int kC>
-__device__ __forceinline__ void fwd_codes(const uint32_t* bits, int L, int N, int k, int T, int q,
+__device__ __forceinline__ void fwd_codes(const uint32_t* bits, const uint64_t* ext, int L, int N, int k, int T, int q,
                                           uint32_t (&m)[4][kC ? kC : kMaxk]) {
   constexpr int kU = kC ? kC : kMaxk;
   const uint32_t mk = (1u << k) - 1u;
@@ -194,7 +220,7 @@ __device__ __forceinline__ void fwd_codes(const uint32_t* bits, int L, int N, in
       if (kC || a < k) {
         int r = i + a;
         if (r >= L) r -= L;
-        const uint32_t win = row_window(bits, L, r, j0, k + 3);
+        const uint32_t win = window(bits, ext, L, r, j0, k + 3);
 #pragma unroll
         for (int t = 0; t < 4; ++t) m[t][a] = (uint32_t)(a * T) + ((win >> t) & mk);
       }
@@ -210,7 +236,7 @@ __device__ __forceinline__ void fwd_codes(const uint32_t* bits, int L, int N, in
         if (kC || a < k) {
           int r = i + a;
           if (r >= L) r -= L;
-          m[t][a] = (uint32_t)(a * T) + row_window(bits, L, r, j, k);
+          m[t][a] = (uint32_t)(a * T) + window(bits, ext, L, r, j, k);
         }
       }
     }
@@ -569,7 +595,8 @@ __device__ void hidden_phase64(const JobDev& jb, const Tabs& tb, const Grp& g, c
 // and k at compile time (0: runtime).
 template <int KC, int kC>
 __device__ void hidden_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v,
-                             uint32_t* h, int P, uint32_t step, int sub, unsigned& nrec, int q0, int q1) {
+                             const uint64_t* ext, uint32_t* h, int P, uint32_t step, int sub, unsigned& nrec, int q0,
+                             int q1) {
   constexpr int kU = kC ? kC : kMaxk;
   const int L = jb.L, N = jb.N, K = KC ? KC : jb.K, k = kC ? kC : jb.k, T = tb.T;
   const int iters = (q1 - q0 + g.tpc - 1) / g.tpc;
@@ -577,7 +604,8 @@ __device__ void hidden_phase(const JobDev& jb, const Tabs& tb, const Grp& g, con
     const int q = q0 + g.r + it * g.tpc;
     const bool act = g.active && q < q1;
     uint32_t m[4][kU];
-    fwd_codes<kC>(v, L, N, k, T, act ? q : 0, m);
+    if (!__any_sync(kFull, act)) continue;
+    fwd_codes<kC>(v, ext, L, N, k, T, act ? q : 0, m);
     if (KC == 4) {
       // all four filters per site from the filter-interleaved table
       uint4 w[4];
@@ -675,7 +703,8 @@ __device__ void visible_phase64(const JobDev& jb, const Tabs& tb, const Grp& g, 
 // Mixed form: thread = unit of 4 sites, units q0 .. q1 - 1.
 template <int KC, int kC>
 __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* h,
-                              uint32_t* vp, int P, uint32_t step, int sub, unsigned& nrec, int q0, int q1) {
+                              const uint64_t* ext, uint32_t* vp, int P, uint32_t step, int sub, unsigned& nrec, int q0,
+                              int q1) {
   constexpr int kU = kC ? kC : kMaxk;
   constexpr int KU = KC ? KC : kMaxK;
   const int L = jb.L, N = jb.N, K = KC ? KC : jb.K, k = kC ? kC : jb.k, T = tb.T;
@@ -685,6 +714,7 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
   for (int it = 0; it < iters; ++it) {
     const int q = q0 + g.r + it * g.tpc;
     const bool act = g.active && q < q1;
+    if (!__any_sync(kFull, act)) continue;
     const int qq = act ? q : 0;
     float x32[4];
 #pragma unroll
@@ -698,32 +728,13 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
         if (kC || a < k) {
           const int r = bwd_row(i, a, L);
           // word offsets of this window, shared by the K hidden planes
-          int o0, o1, sh;
           const bool wide = (L & 31) == 0;
-          if (wide) {
-            const int WL = L >> 5, wi = c >> 5;
-            o0 = r * WL + wi;
-            o1 = r * WL + ((wi + 1 == WL) ? 0 : wi + 1);
-            sh = c & 31;
-          } else {
-            const int off = r * L;
-            o0 = off >> 5;
-            o1 = o0 + 1;
-            sh = off & 31;
-          }
+          const int WL = L >> 5, wi = c >> 5, o0 = r * WL + wi, o1 = r * WL + ((wi + 1 == WL) ? 0 : wi + 1);
 #pragma unroll
           for (int f = 0; f < KU; ++f) {
             if (KC || f < K) {
               const uint32_t* pl = h + f * P;
-              uint32_t win;
-              if (wide) {
-                win = __funnelshift_r(pl[o0], pl[o1], sh);
-              } else {
-                const uint32_t row = __funnelshift_r(pl[o0], pl[o1], sh) & ((1u << L) - 1u);
-                uint64_t rr = row;
-                for (int s2 = L; s2 < 64; s2 += L) rr |= (uint64_t)row << s2;
-                win = (uint32_t)(rr >> c);
-              }
+              const uint32_t win = wide ? __funnelshift_r(pl[o0], pl[o1], c & 31) : (uint32_t)(ext[f * L + r] >> c);
               const int base = (f * k + a) * T;
 #pragma unroll
               for (int t = 0; t < 4; ++t) {
@@ -745,7 +756,7 @@ __device__ void visible_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
         for (int a = 0; a < k; ++a) {
           const int r = bwd_row(i, a, L);
           for (int f = 0; f < K; ++f) {
-            const uint32_t code = row_window(h + f * P, L, r, c, k);
+            const uint32_t code = window(h + f * P, ext + f * L, L, r, c, k);
             const int base = (f * k + a) * T;
             x32[t] += tb.bd[base + code];
           }
@@ -830,7 +841,8 @@ __device__ __forceinline__ double free_constant(const JobDev& jb, int tpc) {
 // Mixed form: thread = unit of 4 sites, units q0 .. q1 - 1, FP32 with Kahan
 // compensation.
 template <int KC, int kC>
-__device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v, int q0, int q1) {
+__device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v,
+                              const uint64_t* ext, int q0, int q1) {
   constexpr int kU = kC ? kC : kMaxk;
   const int L = jb.L, N = jb.N, K = KC ? KC : jb.K, k = kC ? kC : jb.k, T = tb.T;
   const int iters = (q1 - q0 + g.tpc - 1) / g.tpc;
@@ -841,7 +853,7 @@ __device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
     const bool act = g.active && q < q1;
     if (!act) continue;
     uint32_t m[4][kU];
-    fwd_codes<kC>(v, L, N, k, T, q, m);
+    fwd_codes<kC>(v, ext, L, N, k, T, q, m);
     if (KC == 4) {
       float sp[4][4];
 #pragma unroll

@@ -13,6 +13,7 @@ size_t smem_bytes(int kind, int prec, int L, int K, int k, int nc, int KC, int n
   b += align16(64 * 8);
   if (kind == kKitaev) b += (size_t)nc * kitaev_work_bytes((int)N);
   b += align16((size_t)nc * (2 + K) * P * 4);
+  if (prec != kFP64 && L % 32 != 0) b += (size_t)nc * (2 + K) * L * 8;      // expanded rows
   return b;
 }
 

@@ -119,6 +119,39 @@ __device__ __forceinline__ unsigned char* mixed_tables(const JobDev& jb, unsigne
   return sp;
 }
 
+// n_gibbs block-Gibbs steps (Eqs. B2, B3) from v into vp through the hidden
+// planes h; xv, xvp, xh: their expanded rows (xv given; xvp left behind).  sync:
+// the group's barrier, also the last thing done.
+template <int PREC, int KC, int kC, class SYNC>
+__device__ __forceinline__ void gibbs_steps(const JobDev& jb, const Tabs& tb, const Grp& g, const uint32_t* v,
+                                            uint32_t* vp, uint32_t* h, const uint64_t* xv, uint64_t* xvp, uint64_t* xh,
+                                            int P, int n_gibbs, uint32_t step, unsigned& nrec, SYNC sync) {
+  const int nblk = (jb.N + 3) >> 2, K = KC ? KC : jb.K;
+  const bool narrow = (jb.L & 31) != 0;
+  for (int sub = 0; sub < n_gibbs; ++sub) {
+    if constexpr (PREC == kMixed) {
+      hidden_phase<KC, kC>(jb, tb, g, v, xv, h, P, step, sub, nrec, 0, nblk);
+      if (narrow) {
+        sync();
+        expand_rows(h, P, xh, jb.L, K, g.r, g.tpc);
+      }
+      sync();
+      visible_phase<KC, kC>(jb, tb, g, h, xh, vp, P, step, sub, nrec, 0, nblk);
+      if (narrow) {
+        sync();
+        expand_rows(vp, P, xvp, jb.L, 1, g.r, g.tpc);
+      }
+      xv = xvp;
+    } else {
+      hidden_phase64(jb, tb, g, v, h, P, step, sub, sync);
+      sync();
+      visible_phase64(jb, tb, g, h, vp, P, step, sub, sync);
+    }
+    sync();
+    v = vp;
+  }
+}
+
 // log pi, e and c_f of a Kitaev lattice in FP64, valid in the group's leader
 // (the open lattices' jobs run in FP64 only).
 template <int PREC, bool MULTI>
@@ -191,6 +224,10 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     eps_st = (double*)kp;
   }
   uint32_t* my = planes + (size_t)g.gl * (2 + K) * P;
+  // mixed: the chain's expanded rows (v, v', the hidden planes; see expand_rows)
+  uint64_t* ex = PREC == kMixed ? (uint64_t*)((unsigned char*)planes + align16((size_t)jb.nc * (2 + K) * P * 4)) +
+                                      (size_t)g.gl * (2 + K) * jb.L
+                                : nullptr;
   ChainSm& ch = cs[g.gl];
 
   for (int i = tid; i < jb.nc * (2 + K) * P; i += NT) planes[i] = 0u;
@@ -228,13 +265,17 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
   }
   __syncthreads();
   unsigned nrec = 0;
+  if (PREC == kMixed) {
+    expand_rows(my, P, ex, jb.L, 1, g.r, g.tpc);
+    __syncthreads();
+  }
 
   if (AUX && prm.mode == 1) {
     // evaluate F (FP64, or in the mixed path FP32 with its certified bound,
     // as after a mixed proposal), log pi and the observables (FP64) of the
     // current lattices
     FreeSum fs;
-    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, my, 0, nblk);
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, my, ex, 0, nblk);
     else fs = free_phase64(jb, tb.f64, g, my, 0, N);
     reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
@@ -267,18 +308,10 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     const uint32_t cycle = (uint32_t)*(volatile unsigned long long*)xj.step;
     uint32_t* vp = my + P;
     uint32_t* h = my + 2 * P;
-    const uint32_t* src = my;
-    for (int sub = 0; sub < prm.g; ++sub) {
-      if constexpr (PREC == kMixed) hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec, 0, nblk);
-      else hidden_phase64(jb, tb, g, src, h, P, step, sub, []() { __syncthreads(); });
-      __syncthreads();
-      if constexpr (PREC == kMixed) visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec, 0, nblk);
-      else visible_phase64(jb, tb, g, h, vp, P, step, sub, []() { __syncthreads(); });
-      __syncthreads();
-      src = vp;
-    }
+    gibbs_steps<PREC, KC, kC>(jb, tb, g, my, vp, h, ex, ex + jb.L, ex + 2 * jb.L, P, prm.g, step, nrec,
+                              []() { __syncthreads(); });
     FreeSum fs;
-    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp, 0, nblk);
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp, ex + jb.L, 0, nblk);
     else fs = free_phase64(jb, tb.f64, g, vp, 0, N);
     reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
@@ -559,23 +592,15 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     uint32_t* v = my + cur * P;
     uint32_t* vp = my + (cur ^ 1) * P;
     uint32_t* h = my + 2 * P;
-    const uint32_t* src = v;
     if (clerk) {
       if (s > 0) settle(step0 + (uint64_t)(s - 1));
       // mixed: in FP32, within 2^-20 (1 + |log u|), a term of the decision's margin
       if (prm.correct) ch.logu = PREC == kFP64 ? log_u64(step) : (double)log_u32(accept_word(step));
     }
-    for (int sub = 0; sub < prm.g; ++sub) {
-      if constexpr (PREC == kMixed) hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec, 0, nblk);
-      else hidden_phase64(jb, tb, g, src, h, P, step, sub, loop_sync);
-      loop_sync();
-      if constexpr (PREC == kMixed) visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec, 0, nblk);
-      else visible_phase64(jb, tb, g, h, vp, P, step, sub, loop_sync);
-      loop_sync();
-      src = vp;
-    }
+    gibbs_steps<PREC, KC, kC>(jb, tb, g, v, vp, h, ex + cur * jb.L, ex + (cur ^ 1) * jb.L, ex + 2 * jb.L, P, prm.g, step,
+                              nrec, loop_sync);
     FreeSum fs;
-    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp, 0, nblk);
+    if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp, ex + (cur ^ 1) * jb.L, 0, nblk);
     else fs = free_phase64(jb, tb.f64, g, vp, 0, N);
     loop_reduce(fs, g, std::integral_constant<int, PREC>());
     double kr[4] = {0.0, 0.0, 0.0, 0.0};

@@ -157,17 +157,17 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_cons
       if (prm.correct) ch.logu = (double)log_u32(accept_word(step));
     }
     for (int sub = 0; sub < prm.g; ++sub) {
-      hidden_phase<KC, kC>(jb, tb, g, src, h, P, step, sub, nrec, q0, q1);
+      hidden_phase<KC, kC>(jb, tb, g, src, nullptr, h, P, step, sub, nrec, q0, q1);
       cl.sync();
       pull(h, K, r0 - halo, prev);
       __syncthreads();
-      visible_phase<KC, kC>(jb, tb, g, h, vp, P, step, sub, nrec, q0, q1);
+      visible_phase<KC, kC>(jb, tb, g, h, nullptr, vp, P, step, sub, nrec, q0, q1);
       cl.sync();
       pull(vp, 1, r1, next);
       __syncthreads();
       src = vp;
     }
-    FreeSum fs = free_phase<KC, kC>(jb, tb, g, vp, q0, q1);
+    FreeSum fs = free_phase<KC, kC>(jb, tb, g, vp, nullptr, q0, q1);
     reduce_free<kMixed, false>(fs, g, scratch);
     const SlabSum all = cluster_sum(cl, {{0.0, 0.0, 0.0}, fs.fx, fs.b, fs.ones, fs.pairs}, slots, turn);
     if (tid == 0) {

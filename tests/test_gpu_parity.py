@@ -111,6 +111,31 @@ def test_many_ising_chains_match_oracle(ctx, L, K, k, n, g):
         job.release()
 
 
+@pytest.mark.parametrize("L,K,k,n,g", [
+    (3, 8, 3, 700, 2),       # a row repeated until it fills 64 bits; the window spans it
+    (7, 3, 7, 200, 1),       # window as wide as the row
+    (20, 4, 7, 40, 2),       # four sites of one row per unit, the widest window
+    (28, 4, 5, 9, 1),
+    (29, 4, 3, 9, 2),        # sites of two rows in a unit
+    (31, 2, 5, 9, 1),        # the longest row
+])
+def test_repeated_rows_match_oracle(ctx, L, K, k, n, g):
+    """Mixed precision at sides that are no multiple of 32, whose windows are
+    taken from rows repeated over 64 bits: the oracle's chains."""
+    from paper_2008_05401_gb300 import ISING, MIXED
+    W, hb, vb = wl.gaussian_crbm(K, k, 0.2, seed=L * 10 + k)
+    T = wl.ising_ladder(n, 8)
+    bits0 = wl.pack_bits(wl.random_lattices(n, L, seed=L))
+    S = 3
+    ref = oracle_chains("ising", W, hb, vb, L, T, (1.0,), SEED, n, bits0)
+    worst = run_oracle(ref, S, g=g)
+    mid = ctx.load_model(ISING, W, vb, hb)
+    job = ctx.new_job(mid, ISING, L, T, (1.0,), SEED, 0, bits0, MIXED)
+    job.run(S, g=g, precision=MIXED)
+    _compare(job, ref, worst, S)
+    job.release()
+
+
 @pytest.mark.parametrize("L,K,k,n,g,correct", [
     (32, 5, 3, 3, 1, True),      # clusters of 8, four rows per CTA
     (32, 2, 6, 2, 1, True),      # k - 1 = 5 rows of halo: clusters of 4
