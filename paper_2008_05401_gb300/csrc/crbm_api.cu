@@ -310,7 +310,7 @@ static int launch_group(crbm_ctx* ctx, std::vector<int> ids, int S, int g, int c
     tiles += kitaev ? (j.n + nc - 1) / nc : j.tiles;
     if (m.edge && prec != kFP64) return fail(ctx, CRBM_EINVAL, "LCRBM models run in CRBM_FP64 only");
     int KC, kC;
-    specialisation(m.K, m.k, KC, kC);
+    specialisation(j.kind, m.K, m.k, KC, kC);
     if (m.edge) {
       KC = kC = 0;                // the class tables are read by the runtime-shape code
       generic = true;
@@ -1335,9 +1335,11 @@ int crbm_tune(crbm_ctx* ctx, int model_id, int L, int precision, int* best_nc, d
   const int N = L * L, nblk = (N + 3) / 4;
   std::vector<int> cand;
   if (m.kind == kIsing) {
+    int KC, kC;
+    specialisation(m.kind, m.K, m.k, KC, kC);
     for (int nc = 1; nc <= kThreads / 8; nc *= 2)
       if ((nc == 1 || (nc / 2) * nblk < 8 * kThreads) &&
-          smem_bytes(m.kind, precision, L, m.K, m.k, nc, m.K == 4 ? 4 : 0) <= 100 * 1024)
+          smem_bytes(m.kind, precision, L, m.K, m.k, nc, KC) <= 100 * 1024)
         cand.push_back(nc);
   } else {
     // group sizes 256 / nc threads (at least a warp); timed alone, a job runs

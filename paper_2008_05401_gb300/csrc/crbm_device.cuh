@@ -64,7 +64,7 @@ struct JobDev {
   const float* bd;
   const float* fh;
   const float* fl;
-  const float4* fd4;            // [k][2^k] filter-interleaved, K <= 4
+  const float4* fd4;            // [k][2^k] filter-interleaved, K <= 4 (Tabs fdi, fhi, fli)
   const float4* fh4;
   const float4* fl4;
   // tensor-core form (Ising, L = 128, 64, 32 or 16, K <= 4, k <= 5; crbm_step_tc.cu):
@@ -460,14 +460,14 @@ __device__ __forceinline__ double block_sum(double x, double* scratch) {
 //             copies of them serve the mixed path's FP64 recomputes)
 //   fd/bd     FP32 roundings of f64/b64 (mixed-path decisions)
 //   fh/fl     hi/lo split of f64 (mixed-path free energy)
-//   fd4/fh4/fl4  the same forward tables with the filter index innermost,
-//             in shared memory replicated 8 times, entry e of copy c at
-//             float4 index 8 e + c; thread t reads copy t % 8 (the pointer
-//             below already includes + t % 8, so entry e is at [e << 3]):
-//             the 8 threads of a quarter-warp hit 8 distinct bank groups
-//             whatever their codes, so a 16-byte table load never conflicts;
-//             (a*T + code)*4 + f, for K <= 4 (zero-padded): one 16-byte load
-//             serves all filters of a site
+//   fdi/fhi/fli  the same forward tables with the filter index innermost
+//             (global: (a*T + code)*4 + f for K <= 4, zero-padded), for K = 4 and,
+//             Ising, K = 2: one 16- or 8-byte load serves all filters of a site.
+//             In shared memory entry e is 32 floats, 32 / K copies of its K
+//             values; thread t reads copy t % (32 / K) (the pointer includes its
+//             offset, so entry e is at [32 e]): the threads one pass of a load
+//             serves (a quarter or a half warp) hit distinct banks whatever
+//             their codes, so it never conflicts
 struct Tabs {
   const double* f64;
   const double* b64;
@@ -475,14 +475,25 @@ struct Tabs {
   const float* bd;
   const float* fh;
   const float* fl;
-  const float4* fd4;
-  const float4* fh4;
-  const float4* fl4;
+  const float *fdi, *fhi, *fli;
   int T;
 };
 
-__device__ __forceinline__ float comp(const float4& v, int f) {
-  return f == 0 ? v.x : (f == 1 ? v.y : (f == 2 ? v.z : v.w));
+// x_f += entry `code` of an interleaved table, all filters in one load.
+template <int KC>
+__device__ __forceinline__ void add_taps(float (&x)[KC], const float* table, uint32_t code) {
+  static_assert(KC == 2 || KC == 4, "one 8- or 16-byte load");
+  if constexpr (KC == 4) {
+    const float4 e = *reinterpret_cast<const float4*>(table + 32 * code);
+    x[0] += e.x;
+    x[1] += e.y;
+    x[2] += e.z;
+    x[3] += e.w;
+  } else {
+    const float2 e = *reinterpret_cast<const float2*>(table + 32 * code);
+    x[0] += e.x;
+    x[1] += e.y;
+  }
 }
 
 // FP64 recomputes of the mixed path (rare; kept out of line so that the FP32
@@ -606,30 +617,24 @@ __device__ void hidden_phase(const JobDev& jb, const Tabs& tb, const Grp& g, con
     uint32_t m[4][kU];
     if (!__any_sync(kFull, act)) continue;
     fwd_codes<kC>(v, ext, L, N, k, T, act ? q : 0, m);
-    if (KC == 4) {
-      // all four filters per site from the filter-interleaved table
-      uint4 w[4];
+    if constexpr (KC != 0) {
+      // all filters per site from the filter-interleaved table
+      uint4 w[KC];
 #pragma unroll
-      for (int f = 0; f < 4; ++f)
-        w[f] = philox4x32_10_rk(make_uint4((uint32_t)q, (uint32_t)(sub * 5 + f), step, g.cid), jb.rk);
-      uint32_t nib[4] = {0u, 0u, 0u, 0u};
+      for (int f = 0; f < KC; ++f)
+        w[f] = philox4x32_10_rk(make_uint4((uint32_t)q, (uint32_t)(sub * (KC + 1) + f), step, g.cid), jb.rk);
+      uint32_t nib[KC] = {};
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        float4 x = make_float4(jb.hb32[0], jb.hb32[1], jb.hb32[2], jb.hb32[3]);
+        float x[KC];
 #pragma unroll
-        for (int a = 0; a < kU; ++a) {
-          if (kC || a < k) {
-            const float4 e = tb.fd4[m[t][a] << 3];
-            x.x += e.x;
-            x.y += e.y;
-            x.z += e.z;
-            x.w += e.w;
-          }
-        }
+        for (int f = 0; f < KC; ++f) x[f] = jb.hb32[f];
+#pragma unroll
+        for (int a = 0; a < kU; ++a) add_taps(x, tb.fdi, m[t][a]);
         const bool site = act && 4 * q + t < N;
 #pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          uint32_t bit = decide32(comp(x, f), pick(w[f], t), jb.c0h, jb.c1);
+        for (int f = 0; f < KC; ++f) {
+          uint32_t bit = decide32(x[f], pick(w[f], t), jb.c0h, jb.c1);
           if (bit == 2u) {
             uint32_t mm[kMaxk];
 #pragma unroll
@@ -641,7 +646,7 @@ __device__ void hidden_phase(const JobDev& jb, const Tabs& tb, const Grp& g, con
         }
       }
 #pragma unroll
-      for (int f = 0; f < 4; ++f) store_nibble(h + f * P, q, nib[f], act);
+      for (int f = 0; f < KC; ++f) store_nibble(h + f * P, q, nib[f], act);
       continue;
     }
     for (int f = 0; f < K; ++f) {
@@ -854,30 +859,31 @@ __device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
     if (!act) continue;
     uint32_t m[4][kU];
     fwd_codes<kC>(v, ext, L, N, k, T, q, m);
-    if (KC == 4) {
-      float sp[4][4];
+    if constexpr (KC != 0) {
+      float sp[4][KC];
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        float4 xh = make_float4(jb.hb_hi[0], jb.hb_hi[1], jb.hb_hi[2], jb.hb_hi[3]);
-        float4 xl = make_float4(jb.hb_lo[0], jb.hb_lo[1], jb.hb_lo[2], jb.hb_lo[3]);
+        float xh[KC], xl[KC];
+#pragma unroll
+        for (int f = 0; f < KC; ++f) {
+          xh[f] = jb.hb_hi[f];
+          xl[f] = jb.hb_lo[f];
+        }
 #pragma unroll
         for (int a = 0; a < kU; ++a) {
-          if (kC || a < k) {
-            const float4 eh = tb.fh4[m[t][a] << 3], el = tb.fl4[m[t][a] << 3];
-            xh.x += eh.x; xh.y += eh.y; xh.z += eh.z; xh.w += eh.w;
-            xl.x += el.x; xl.y += el.y; xl.z += el.z; xl.w += el.w;
-          }
+          add_taps(xh, tb.fhi, m[t][a]);
+          add_taps(xl, tb.fli, m[t][a]);
         }
         const bool site = 4 * q + t < N;
 #pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          const float x = comp(xh, f) + comp(xl, f);
+        for (int f = 0; f < KC; ++f) {
+          const float x = xh[f] + xl[f];
           sp[t][f] = site ? softplus32(x) : 0.0f;
           sabs += site ? fabsf(x) : 0.0f;
         }
       }
 #pragma unroll
-      for (int f = 0; f < 4; ++f) {
+      for (int f = 0; f < KC; ++f) {
         const float us = (sp[0][f] + sp[1][f]) + (sp[2][f] + sp[3][f]);
         ssp += us;
         const float y = us - c32;          // Kahan summation of the unit sums

@@ -8,7 +8,7 @@ size_t smem_bytes(int kind, int prec, int L, int K, int k, int nc, int KC, int n
   const size_t N = (size_t)L * L, P = (N + 31) / 32 + 1, nlut = (size_t)ncls * K * k * ((size_t)1 << k);
   const size_t nq = (size_t)k << k;
   size_t b = (prec == kFP64) ? 0
-             : (KC == 4 ? 3 * align16(nq * 16 * 8) + align16(nlut * 4) : 4 * align16(nlut * 4));
+             : (KC != 0 ? 3 * align16(nq * 16 * 8) + align16(nlut * 4) : 4 * align16(nlut * 4));
   b += align16(nc * sizeof(ChainSm));
   b += align16(64 * 8);
   if (kind == kKitaev) b += (size_t)nc * kitaev_work_bytes((int)N);
@@ -62,11 +62,17 @@ cudaError_t limit_kKitaev_kFP64_256_multi(size_t);
 cudaError_t launch_kKitaev_kMixed_256_multi(int, int, const LaunchParams&, int, size_t, cudaStream_t);
 cudaError_t limit_kKitaev_kMixed_256_multi(size_t);
 
-void specialisation(int K, int k, int& KC, int& kC) {
+// The banks that the configurations use: four or two filters of 3 x 3 or 5 x 5.
+// The runtime variant unrolls for 7 x 7 and 8 filters and reads a table entry per
+// filter (1024 Ising chains of L = 24, K = 2, k = 5, 20 proposals: 1.09 ms with
+// it, 0.49 with their own, bound by instruction issue and the barriers between
+// the half-steps).  A Kitaev proposal is its eigen-stage: two filters there stay
+// with the runtime variant.
+void specialisation(int kind, int K, int k, int& KC, int& kC) {
   KC = 0;
   kC = 0;
-  if (K == 4 && (k == 5 || k == 3)) {
-    KC = 4;
+  if ((K == 4 || (K == 2 && kind == kIsing)) && (k == 5 || k == 3)) {
+    KC = K;
     kC = k;
   }
 }
@@ -85,7 +91,7 @@ int kitaev_group_threads(int N) { return N <= 16 ? 32 : (N <= 64 ? 64 : (N <= 10
 cudaError_t launch_step(int kind, int prec, int K, int k, int nt, const LaunchParams& p, int grid, size_t smem,
                         cudaStream_t st, bool generic, bool multi) {
   int KC, kC;
-  specialisation(K, k, KC, kC);
+  specialisation(kind, K, k, KC, kC);
   if (generic) KC = kC = 0;
   if (multi)
     return prec == kFP64 ? launch_kKitaev_kFP64_256_multi(KC, kC, p, grid, smem, st)

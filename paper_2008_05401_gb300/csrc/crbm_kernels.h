@@ -10,7 +10,7 @@ struct JobDev;
 
 // Compiled specialisation (KC, kC) serving a filter bank of K filters k x k
 // (0 = runtime values).
-void specialisation(int K, int k, int& KC, int& kC);
+void specialisation(int kind, int K, int k, int& KC, int& kC);
 // Dynamic shared memory of one CTA of the fused kernel (ncls kernel classes
 // in the tables: 1 for a CRBM, 2 edge + 1 for an LCRBM).
 size_t smem_bytes(int kind, int prec, int L, int K, int k, int nc, int KC, int ncls = 1);

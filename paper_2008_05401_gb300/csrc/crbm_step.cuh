@@ -88,19 +88,25 @@ __device__ __forceinline__ unsigned char* mixed_tables(const JobDev& jb, unsigne
     sp += align16(bytes);
     return at;
   };
-  if (KC == 4) {
-    float4* t4[3];
-    for (int i = 0; i < 3; ++i) t4[i] = (float4*)take((size_t)nq * 16 * 8);      // 8 bank-interleaved copies
+  if constexpr (KC != 0) {
+    // an entry is 32 / KC copies of its KC filters, 128 bytes: the lanes of a
+    // quarter (KC = 4) or half warp (KC = 2), which one pass serves, read from
+    // copies and so from banks of their own
+    float* ti[3];
+    for (int i = 0; i < 3; ++i) ti[i] = (float*)take((size_t)nq * 128);
     float* bd = (float*)take((size_t)nlut * 4);
     for (int i = tid; i < nlut; i += nt) bd[i] = jb.bd[i];
-    for (int i = tid; i < nq * 8; i += nt) {
-      t4[0][i] = jb.fd4[i >> 3];
-      t4[1][i] = jb.fh4[i >> 3];
-      t4[2][i] = jb.fl4[i >> 3];
+    const float *gd = (const float*)jb.fd4, *gh = (const float*)jb.fh4, *gl = (const float*)jb.fl4;
+    for (int i = tid; i < nq * 32; i += nt) {
+      const int e = (i >> 5) * 4 + (i & (KC - 1));
+      ti[0][i] = gd[e];
+      ti[1][i] = gh[e];
+      ti[2][i] = gl[e];
     }
-    tb.fd4 = t4[0] + (tid & 7);
-    tb.fh4 = t4[1] + (tid & 7);
-    tb.fl4 = t4[2] + (tid & 7);
+    const int copy = KC * (tid & (32 / KC - 1));
+    tb.fdi = ti[0] + copy;
+    tb.fhi = ti[1] + copy;
+    tb.fli = ti[2] + copy;
     tb.bd = bd;
   } else {
     float* t[4];
@@ -181,7 +187,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
   tb.T = T;
   tb.f64 = tb.b64 = nullptr;
   tb.fd = tb.bd = tb.fh = tb.fl = nullptr;
-  tb.fd4 = tb.fh4 = tb.fl4 = nullptr;
+  tb.fdi = tb.fhi = tb.fli = nullptr;
   if constexpr (PREC == kFP64) {
     // read through L1: the FP64 pipe, not the tables, paces the FP64 phases, and
     // an LCRBM's 36 KB of them per CTA left half of the chains waiting for an SM
@@ -797,6 +803,10 @@ cudaError_t launch_nt(int KC, int kC, const LaunchParams& p, int grid, size_t sm
   if constexpr (PREC == kMixed) {
     if (KC == 4 && kC == 5) return launch_inst<KIND, PREC, 4, 5, NT>(p, grid, smem, st);
     if (KC == 4 && kC == 3) return launch_inst<KIND, PREC, 4, 3, NT>(p, grid, smem, st);
+    if constexpr (KIND == kIsing) {
+      if (KC == 2 && kC == 5) return launch_inst<KIND, PREC, 2, 5, NT>(p, grid, smem, st);
+      if (KC == 2 && kC == 3) return launch_inst<KIND, PREC, 2, 3, NT>(p, grid, smem, st);
+    }
   }
   return launch_inst<KIND, PREC, 0, 0, NT>(p, grid, smem, st);
 }
@@ -807,6 +817,10 @@ cudaError_t limit_nt(size_t bytes) {
   if constexpr (PREC == kMixed) {
     if (e == cudaSuccess) e = limit_inst<KIND, PREC, 4, 5, NT>(bytes);
     if (e == cudaSuccess) e = limit_inst<KIND, PREC, 4, 3, NT>(bytes);
+    if constexpr (KIND == kIsing) {
+      if (e == cudaSuccess) e = limit_inst<KIND, PREC, 2, 5, NT>(bytes);
+      if (e == cudaSuccess) e = limit_inst<KIND, PREC, 2, 3, NT>(bytes);
+    }
   }
   return e;
 }

@@ -15,7 +15,7 @@
 // so each takes the same decision and keeps the chain's values itself.
 // Three cluster barriers per proposal of one Gibbs step; the rest is bound by
 // instruction issue like the table kernel (53 % of the slots).  16 chains of
-// L = 256, K = 4 5x5, 40 proposals and the read-back: 2.05 ms (one CTA per chain:
+// L = 256, K = 4 5x5, 40 proposals and the read-back: 1.75 ms (one CTA per chain:
 // 12.5 ms).
 #include <algorithm>
 
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_cons
   tb.T = 1 << jb.k;
   tb.f64 = tb.b64 = nullptr;
   tb.fd = tb.bd = tb.fh = tb.fl = nullptr;
-  tb.fd4 = tb.fh4 = tb.fl4 = nullptr;
+  tb.fdi = tb.fhi = tb.fli = nullptr;
   uint32_t* my = (uint32_t*)mixed_tables<KC>(jb, smem_raw, tb, tid, kSlabThreads);
 
   Grp g;
@@ -279,9 +279,11 @@ cudaError_t launch_inst(const LaunchParams* p, int chains, int CL, size_t smem, 
 
 cudaError_t launch_any(int K, int k, const LaunchParams* p, int chains, int CL, size_t smem, cudaStream_t st, int* fit) {
   int KC, kC;
-  specialisation(K, k, KC, kC);
+  specialisation(kIsing, K, k, KC, kC);
   if (KC == 4 && kC == 5) return launch_inst<4, 5>(p, chains, CL, smem, st, fit);
   if (KC == 4 && kC == 3) return launch_inst<4, 3>(p, chains, CL, smem, st, fit);
+  if (KC == 2 && kC == 5) return launch_inst<2, 5>(p, chains, CL, smem, st, fit);
+  if (KC == 2 && kC == 3) return launch_inst<2, 3>(p, chains, CL, smem, st, fit);
   return launch_inst<0, 0>(p, chains, CL, smem, st, fit);
 }
 
@@ -295,9 +297,9 @@ cudaError_t limit_inst(size_t bytes) {
 
 size_t slab_smem_bytes(int L, int K, int k) {
   int KC, kC;
-  specialisation(K, k, KC, kC);
+  specialisation(kIsing, K, k, KC, kC);
   const size_t P = (size_t)L * L / 32 + 1, nlut = (size_t)K * k << k, nq = (size_t)k << k;
-  return (KC == 4 ? 3 * align16(nq * 16 * 8) + align16(nlut * 4) : 4 * align16(nlut * 4)) + (2 + (size_t)K) * P * 4;
+  return (KC != 0 ? 3 * align16(nq * 16 * 8) + align16(nlut * 4) : 4 * align16(nlut * 4)) + (2 + (size_t)K) * P * 4;
 }
 
 int slab_most(int L, int K, int k, size_t smem_limit) {
@@ -321,6 +323,8 @@ cudaError_t launch_slab(const LaunchParams& p, int chains, int CL, size_t smem, 
 cudaError_t slab_set_smem_limit(size_t bytes) {
   cudaError_t e = limit_inst<4, 5>(bytes);
   if (e == cudaSuccess) e = limit_inst<4, 3>(bytes);
+  if (e == cudaSuccess) e = limit_inst<2, 5>(bytes);
+  if (e == cudaSuccess) e = limit_inst<2, 3>(bytes);
   if (e == cudaSuccess) e = limit_inst<0, 0>(bytes);
   return e;
 }

@@ -143,6 +143,8 @@ def test_repeated_rows_match_oracle(ctx, L, K, k, n, g):
     (64, 8, 3, 40, 1, True),     # 40 chains: clusters of 2
     (96, 4, 5, 4, 2, True),      # rows of three words, twelve rows per CTA
     (96, 1, 1, 19, 1, True),     # one tap: the halo row only counts pairs; all 152 CTAs
+    (96, 2, 5, 3, 1, True),      # two filters from one 8-byte table entry
+    (160, 2, 3, 2, 1, True),
     (224, 4, 3, 2, 1, True),
     (256, 4, 5, 3, 1, True),
 ])
