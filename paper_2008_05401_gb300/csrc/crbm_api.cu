@@ -103,14 +103,35 @@ bool valid_L(int kind, int L) {
   return false;
 }
 
-// Chains per CTA of an Ising job: about two 4-site units per thread, a power
-// of two in [1, 32].  (A Kitaev job's follow from its group size per launch.)
-int chains_per_tile(int kind, int L) {
-  if (kind == kKitaev) return 1;
+// Chains per CTA of an Ising job of n chains (a Kitaev job's follow from its
+// group size per launch): a power of two in [1, 32], at most 16 units of 4 sites
+// a thread.  A proposal of a CTA takes about as long as its units per thread and
+// one more (barriers, reductions and the decision do not grow with its chains),
+// and an SM runs two CTAs side by side, so the choice minimises waves x (units
+// per thread + 1) among those that leave 1.5 CTAs or more for an SM.  40 mixed
+// proposals, K = 2, k = 5, against two units per thread whatever n: 1024 chains of
+// L = 24 822 -> 628 us, 4096 2734 -> 1742; 4096 of L = 12 1062 -> 741, of L = 30
+// 4152 -> 3897; one chain per CTA up to 1.5 chains an SM (100 FP64 proposals of 16
+// chains of L = 8: 8.1 ms in one CTA, 1.15 ms in 16).
+int chains_per_cta(const Model& m, int L, int n, int sms) {
   const int nblk = (L * L + 3) / 4;
-  int nc = 1;
-  while (nc < kThreads / 8 && (nc * 2) * nblk <= 2 * kThreads) nc *= 2;
-  return nc;
+  int KC, kC;
+  specialisation(m.kind, m.K, m.k, KC, kC);
+  int best = 1;
+  long long best_t = 0;
+  for (int nc = 1; nc <= 32; nc *= 2) {
+    const long long tiles = ((long long)n + nc - 1) / nc;
+    if (nc > 1 && (nc * nblk > 16 * kThreads || 2 * tiles < 3LL * sms ||
+                   smem_bytes(m.kind, kMixed, L, m.K, m.k, nc, KC) > 100 * 1024))
+      break;
+    const int tpc = kThreads / nc;
+    const long long t = (tiles + 2 * sms - 1) / (2 * sms) * ((nblk + tpc - 1) / tpc + 1);
+    if (nc == 1 || t < best_t) {
+      best = nc;
+      best_t = t;
+    }
+  }
+  return best;
 }
 
 }  // namespace
@@ -923,10 +944,7 @@ int crbm_init_chains(crbm_ctx* ctx, int model_id, int L, int n_chains, const dou
   j.N = L * L;
   j.Wd = (j.N + 31) / 32;
   j.n = n_chains;
-  j.nc = chains_per_tile(m.kind, L);
-  // few chains: spread them over the SMs (100 FP64 proposals of 16 chains of
-  // L = 8: 8.1 ms in one CTA, 1.15 ms in 16)
-  while (j.nc > 1 && (n_chains + j.nc - 1) / j.nc < ctx->sms) j.nc /= 2;
+  j.nc = m.kind == kIsing ? chains_per_cta(m, L, n_chains, ctx->sms) : 1;
   if (m.kind == kKitaev) j.tpc = kitaev_group_threads(j.N);
   {
     // crbm_tune's choice: chains per CTA (Ising) or the group size (Kitaev)
