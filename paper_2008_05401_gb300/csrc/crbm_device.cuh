@@ -963,6 +963,50 @@ __device__ __forceinline__ int row_split(int m, int nt) {
   return H;
 }
 
+// The same for the FP64 stage, which its pipe's warp instructions pace whatever
+// lanes they fill: of that H and its two next, the one whose warps' steps, with the
+// log2 H additions that join a row, are fewest (35 rows by 64 threads: 70 at H = 1,
+// where the second warp takes 35 for three rows; 55 at H = 4).  Tempering of L = 8,
+// six cycles of 2 x 1024 chains: 7.2 ms without it, 6.9 with.
+__device__ __forceinline__ int row_lanes64(int m, int nt) {
+  int H = row_split(min(m, nt), nt), best = H, cost = 1 << 30;
+  for (int i = 0; i < 3 && H <= 8; ++i, H <<= 1) {
+    const int t = ((m * H + 31) >> 5) * ((m + H - 1) / H + 31 - __clz(H));
+    if (t < cost) {
+      cost = t;
+      best = H;
+    }
+  }
+  return best;
+}
+// Element (c, l) of the rows and columns j1 .. of a packed lower triangle, on
+// either side of its diagonal.  A warp of a matrix-vector product takes one loop
+// over c with it: with a loop along the packed row and one down the packed column,
+// each lane crossing over at its own diagonal, the warp took the longest of both
+// (66 steps for the 35 of the first 32 rows at 35 columns).  Rows start at
+// triangular numbers, distinct mod 16, columns are contiguous: no bank conflicts
+// at one lane per row.  1024 chains of L = 6, mixed, eight proposals 1.92 -> 1.78
+// ms, FP64, four 1.83 -> 1.74; tempering of L = 8 7.8 -> 6.9; 1024 open-boundary
+// chains of L = 8, four proposals 8.7 -> 8.3; 683 mixed chains each of L = 8, 10,
+// 12, three proposals 11.5 -> 11.1.
+template <class T>
+__device__ __forceinline__ T sym_at(const T* A, int j1, int c, int l) {
+  return A[tri(j1 + max(c, l), j1) + min(c, l)];
+}
+// Lane h's share (columns h, h + H, ...) of row l of A22 x; mac(a, x, y): y += a x.
+// (Loops of their own for the columns left and right of the warp's diagonals need
+// no index arithmetic but are four times the code: 2.00 ms for the mixed L = 6.)
+template <class T, class MAC>
+__device__ __forceinline__ void sym_row(const T* A, const T* xs, int j1, int m, int l, int h, int H, T& y0, T& y1,
+                                        MAC mac) {
+  int c = h;
+  for (; c + H < m; c += 2 * H) {
+    mac(sym_at(A, j1, c, l), xs[c], y0);
+    mac(sym_at(A, j1, c + H, l), xs[c + H], y1);
+  }
+  if (c < m) mac(sym_at(A, j1, c, l), xs[c], y0);
+}
+
 // Thread tid of nt visiting a packed triangle of R rows (row r: columns
 // 0..r) with stride nt: rows p and R-1-p side by side form folded row p,
 // R+1 long, so the thread's next element is a fixed step away in the folded
@@ -1305,8 +1349,8 @@ __device__ __forceinline__ void thermal_add(double eps, double beta, double& lp,
 // (before: two counts, then Newton steps of five operations until one confirms
 // the last), one Gershgorin interval in FP32 (before: a serial FP64 loop of one
 // thread), and clusters found by the whole warp.  1024 chains of L = 6, four
-// proposals: 1.81 ms (3.74); six tempering cycles of 1024 + 1024 chains of L = 8,
-// four Gibbs steps each: 7.7 ms (15.0).
+// proposals: 1.74 ms (3.74); six tempering cycles of 1024 + 1024 chains of L = 8,
+// four Gibbs steps each: 6.9 ms (15.0).
 template <bool MULTI>
 __device__ inline void kitaev_logpi64(const Grp& g, const uint32_t* v, int L, const double* J, double beta,
                                const KitaevWork& wk, double (&res)[3], double* eps_out = nullptr) {
@@ -1404,37 +1448,20 @@ __device__ inline void kitaev_logpi64(const Grp& g, const uint32_t* v, int L, co
       }
     }
     double q = 0.0;
-    for (int l0 = 0; l0 < m;) {
-      const int H = row_split(min(m - l0, nt), nt), h = lane & (H - 1);
-      const int l = l0 + warp * (32 / H) + lane / H;
-      double y0 = 0.0, y1 = 0.0;
-      if (l < m) {
-        const double* row = A + tri(j1 + l, j1);
-        int c = h;
-        for (; c + H <= l; c += 2 * H) {
-          y0 = fma(row[c], xs[c], y0);
-          y1 = fma(row[c + H], xs[c + H], y1);
-        }
-        if (c <= l) {
-          y0 = fma(row[c], xs[c], y0);
-          c += H;
-        }
-        for (; c + H < m; c += 2 * H) {
-          y1 = fma(A[tri(j1 + c, j1) + l], xs[c], y1);
-          y0 = fma(A[tri(j1 + c + H, j1) + l], xs[c + H], y0);
-        }
-        if (c < m) y1 = fma(A[tri(j1 + c, j1) + l], xs[c], y1);
-      }
-      double y = y0 + y1;
+    const int H = row_lanes64(m, nt), h = lane & (H - 1);
+    for (int lf = warp * (32 / H); lf < m; lf += nt / H) {
+      const int lr = lf + lane / H, l = min(lr, m - 1);
+      double y = 0.0, y1 = 0.0;
+      sym_row(A, xs, j1, m, l, h, H, y, y1, [](double a, double x, double& t) { t = fma(a, x, t); });
+      y += y1;
       for (int o = 1; o < H; o <<= 1) y += __shfl_xor_sync(kFull, y, o);
-      if (l < m && h == 0) {
+      if (lr < m && h == 0) {
         uw[l].y = y;
         if (l == 0) scA[3] = y;
         q = fma(xs[l], y, q);
       }
-      l0 += nt / H;
     }
-    if (warp * 32 < m * row_split(min(m, nt), nt) || m > nt) {
+    if (warp * (32 / H) < m) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(kFull, q, o);
     }

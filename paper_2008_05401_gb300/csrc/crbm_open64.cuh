@@ -287,38 +287,31 @@ static __device__ __noinline__ void kitaev_logpi64_open(const Grp& g, const uint
     // of a warp per row (H = 1, 2, 4, .. while H m still fits the group), lane
     // h of a row taking the columns c = h mod H -- the row part c <= l
     // (contiguous), then the column part c > l -- alternately into two
-    // accumulators, the H lanes' sums then added by a butterfly
+    // accumulators, the H lanes' sums then added by a butterfly.  One loop for
+    // both parts (see sym_at): ea, eb take turns, and a lane whose column part
+    // starts out of turn exchanges them there, so that every sum keeps its order
     const int H = row_split(m, nt), h = lane & (H - 1);
     double part = 0.0;
     for (int l0 = 0; l0 < m; l0 += nt / H) {
-      const int l = l0 + warp * (32 / H) + lane / H;
-      double e0 = 0.0, e1 = 0.0;
-      if (l < m) {
-        const double* row = A + tri(j1 + l, j1);
-        int c = h;
-        if (c == 0) {
-          e0 = row[0] * u0;
-          c = H;
+      const int l = l0 + warp * (32 / H) + lane / H, lc = min(l, m - 1);
+      double e = 0.0;
+      if (l0 + warp * (32 / H) < m) {
+        int c = h == 0 ? H : h;
+        // ea: the odd accumulator of the row part, which its first term goes to
+        double ea = 0.0, eb = h == 0 ? A[tri(j1 + lc, j1)] * u0 : 0.0;
+        const int turns = lc >= c ? (lc - c) / H + 1 : 0;       // of the row part
+        const int cross = (turns & 1) ? -1 : c + turns * H;     // (an even turn, so ea's)
+        for (; c < m; c += 2 * H) {
+          if (c == cross) {
+            const double t = ea;
+            ea = eb;
+            eb = t;
+          }
+          ea = fma(sym_at(A, j1, c, lc), A[tri(j1 + c, j)], ea);
+          if (c + H < m) eb = fma(sym_at(A, j1, c + H, lc), A[tri(j1 + c + H, j)], eb);
         }
-        for (; c + H <= l; c += 2 * H) {
-          e1 = fma(row[c], A[tri(j1 + c, j)], e1);
-          e0 = fma(row[c + H], A[tri(j1 + c + H, j)], e0);
-        }
-        if (c <= l) {
-          e1 = fma(row[c], A[tri(j1 + c, j)], e1);
-          c += H;
-        }
-        for (; c + H < m; c += 2 * H) {
-          const int b1 = tri(j1 + c, 0), b2 = tri(j1 + c + H, 0);
-          e0 = fma(A[b1 + j1 + l], A[b1 + j], e0);
-          e1 = fma(A[b2 + j1 + l], A[b2 + j], e1);
-        }
-        if (c < m) {
-          const int b1 = tri(j1 + c, 0);
-          e0 = fma(A[b1 + j1 + l], A[b1 + j], e0);
-        }
+        e = ea + eb;
       }
-      double e = e0 + e1;
       for (int o = 1; o < H; o <<= 1) e += __shfl_xor_sync(kFull, e, o);
       if (l < m && h == 0) {
         const double p = tau * e, ul = l == 0 ? u0 : A[tri(j1 + l, j)];
