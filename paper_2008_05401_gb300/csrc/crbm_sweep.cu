@@ -17,9 +17,9 @@
 // FP64 observables of each sweep, one sweep behind, so that no sweep waits on
 // the FP64 pipe.  What bounds it is the issue of the Philox rounds (about 60
 // of some 80 instructions per four sites).
-// 512 chains of 64 x 64, 100 sweeps with the FP64 F of the last and the read-back:
-// 0.68 ms (one site at a time, FP64
-// comparison, Philox per colour, counts by a pass over the sites: 4.32 ms).
+// 512 chains of 64 x 64, 100 sweeps with the FP64 F of the last and the
+// read-back: 0.52 ms (one site at a time, FP64 comparison, Philox per colour,
+// counts by a pass over the sites: 4.32 ms).
 #include <algorithm>
 
 #include "crbm_device.cuh"

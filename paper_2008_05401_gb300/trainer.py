@@ -1,7 +1,7 @@
 """The paper's CRBM trainer (Sec. II, App. A, Algorithm 1) driven from the host.
 
 Every arithmetic step runs in the CUDA library: the epochs of minibatch ADAM
-steps (``crbm_train_epochs``, one CTA per problem), the physical samples
+steps (``crbm_train_epochs``, a cluster of CTAs per problem), the physical samples
 (local-update Metropolis sweeps, ``crbm_local_run``), the buffer of RBM
 samples (uncorrected Gibbs proposals, ``crbm_run`` with correct = 0) and their
 targets (FP64 log pi of the job).  This module only moves lattices, targets
