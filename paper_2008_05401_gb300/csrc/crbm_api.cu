@@ -34,6 +34,7 @@ struct Model {
   float hb32[kMaxK] = {}, hb_hi[kMaxK] = {}, hb_lo[kMaxK] = {};
   float vb32 = 0.f;
   float c0h = 0.f, c0v = 0.f, c1 = 0.f, csp = 0.f, cdf = 0.f;
+  double sp_site = 0.0;      // a site's softplus terms of all filters are at most this
   // tensor-core form (Ising, K <= 4, k <= 5): filter-digit operand images
   uint4* d_tc = nullptr;
   size_t tc_bytes = 0;
@@ -202,6 +203,16 @@ static Job* get_job(crbm_ctx* ctx, int id) {
   return &ctx->jobs[id];
 }
 
+// Exponent e of the mixed path's free-energy sums over a lattice of N sites, kept
+// as integers in units of 2^-e: their sum stays below 2^61 (the FP32 terms' own
+// roundings included).  Beyond e = -100 the FP32 sums are infinite and so is the
+// bound that sends the decision to FP64.
+static int fx_exponent(const Model& m, int N) {
+  const double most = (double)N * m.sp_site;
+  if (!(most < 0x1p160)) return -100;
+  return std::min(59, 60 - std::ilogb(std::fmax(most, 1.0)));
+}
+
 static JobDev make_jobdev(const crbm_ctx* ctx, const Job& j) {
   const Model& m = ctx->models[j.model];
   JobDev d;
@@ -232,6 +243,9 @@ static JobDev make_jobdev(const crbm_ctx* ctx, const Job& j) {
   d.c1 = m.c1;
   d.csp = m.csp;
   d.cdf = m.cdf;
+  const int fx = fx_exponent(m, j.N);
+  d.fx_scale = std::ldexp(1.0f, fx);
+  d.fx_unit = std::ldexp(1.0, -fx);
   d.f64 = m.d_f64;
   d.b64 = m.d_f64 + m.nlut;
   if (m.d_f32) {                 // an LCRBM has FP64 tables only
@@ -721,6 +735,7 @@ static int build_model(crbm_ctx* ctx, Model& m, int kind, int K, int k, const do
         bwd[((size_t)f * k + a) * T + w] = fwd[((size_t)f * k + a) * T + rev];
       }
   // S_h, S_v: largest possible |partial sum| of a hidden / visible pre-activation
+  m.sp_site = 0.0;
   double sh = 0.0, sv = std::fabs(v_bias);
   for (int f = 0; f < K; ++f) {
     double sf = std::fabs(h_bias[f]);
@@ -731,6 +746,7 @@ static int build_model(crbm_ctx* ctx, Model& m, int kind, int K, int k, const do
       sv += mx;
     }
     sh = std::fmax(sh, sf);
+    m.sp_site += sf + 1.0;        // softplus(x) <= |x| + ln 2
   }
   // hi/lo split for the FP32 free energy: hi on a 2^-gbits grid such that every
   // partial sum of hi terms is exact in FP32; lo = the FP32-rounded remainder.

@@ -58,6 +58,8 @@ struct JobDev {
   float hb32[kMaxK], hb_hi[kMaxK], hb_lo[kMaxK];
   float c0h, c0v, c1, csp;      // FP32 error-bound constants (see host code)
   float cdf;                    // per unit: |hi/lo-table pre-activation - FP64 path's|
+  float fx_scale;               // 2^e: units of the mixed path's free-energy sums (FreeSum::fx) in 1
+  double fx_unit;               // 2^-e
   const double* f64;            // [K][k][2^k] row-sum tables, see struct Tabs
   const double* b64;
   const float* fd;
@@ -383,9 +385,11 @@ __device__ __forceinline__ void grp_sync(const Grp& g) {
 }
 
 // Sums of a free-energy pass: F's softplus sum -- FP64 (s), or for the FP32
-// pass the thread's sum as an integer in units of 2^-32 (fx: exact additions
-// off the FP64 pipe, each thread's conversion within 2^-33) with the data part
-// of its error bound (b) -- and the lattice counts.
+// pass the thread's sum as an integer in units of jb.fx_unit (fx: exact additions
+// off the FP64 pipe, each thread's conversion within half a unit) with the data
+// part of its error bound (b) -- and the lattice counts.  The unit is the power
+// of two that leaves the largest sum the filters allow below 2^61 (fx_exponent):
+// a fixed one would wrap for large filters, or round small sums.
 struct FreeSum {
   double s;
   long long fx;
@@ -436,9 +440,9 @@ __device__ __forceinline__ void reduce_free(FreeSum& x, const Grp& g, double* sc
 
 // F (Eq. 13) from the group's sums.
 template <int PREC>
-__device__ __forceinline__ double free_value(double vb, const FreeSum& x) {
-  if (PREC == kFP64) return -vb * (double)x.ones - x.s;
-  return fma((double)x.fx, -0x1p-32, -vb * (double)x.ones);
+__device__ __forceinline__ double free_value(const JobDev& jb, const FreeSum& x) {
+  if (PREC == kFP64) return -jb.vb * (double)x.ones - x.s;
+  return fma((double)x.fx, -jb.fx_unit, -jb.vb * (double)x.ones);
 }
 
 // Deterministic block-wide sum, result returned to every thread.
@@ -840,7 +844,7 @@ __device__ __forceinline__ double free_bound(const FreeSum& x, double cst, doubl
 }
 // Per unit the special-function and table errors, per thread the fixed-point conversion.
 __device__ __forceinline__ double free_constant(const JobDev& jb, int tpc) {
-  return (double)jb.K * (double)jb.N * (1.5 * 0x1p-23 + (double)jb.csp) + (double)tpc * 0x1p-33;
+  return (double)jb.K * (double)jb.N * (1.5 * 0x1p-23 + (double)jb.csp) + (double)tpc * (0.5 * jb.fx_unit);
 }
 
 // Mixed form: thread = unit of 4 sites, units q0 .. q1 - 1, FP32 with Kahan
@@ -943,7 +947,7 @@ __device__ FreeSum free_phase(const JobDev& jb, const Tabs& tb, const Grp& g, co
   }
   FreeSum out;
   out.s = 0.0;
-  out.fx = __float2ll_rn(s32 * 0x1p32f);
+  out.fx = __float2ll_rn(s32 * jb.fx_scale);
   // x rounding + ex2 argument: 2^-23 |x|; pairwise, Kahan and final add: 6 2^-24 sp
   // (free_bound's factor covers the FP32 accumulation of these two sums themselves)
   out.b = sabs * 0x1p-23f + ssp * (6.0f * 0x1p-24f);

@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     if (KIND == kKitaev)
       fp64_spectrum<PREC, MULTI>(jb, g, my, g.active ? ch.beta : 1.0, wk, kr, g.active ? jb.eps + (size_t)g.c * N : nullptr);
     if (g.active && g.r == 0) {
-      const double F = free_value<PREC>(jb.vb, fs);
+      const double F = free_value<PREC>(jb, fs);
       const double E = KIND == kIsing ? ising_energy(jb, fs.pairs) : kr[1];
       double ot[kNobs];
       observables<KIND>(jb, E, kr[2], fs.ones, fs.pairs, ot);
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     if (g.active)
       for (int w = g.r; w < jb.Wd; w += g.tpc) h[w] = xj.bits[(size_t)g.c * jb.Wd + w];
     if (g.active && g.r == 0) {
-      ch.Fp = free_value<PREC>(jb.vb, fs);
+      ch.Fp = free_value<PREC>(jb, fs);
       ch.Bp = PREC == kMixed ? free_bound(fs, free_constant(jb, g.tpc), ch.Fp) : 0.0;
       ch.Ep = KIND == kIsing ? ising_energy(jb, fs.pairs) : kr[1];
       ch.lpp = KIND == kIsing ? -ch.beta * ch.Ep : kr[0];
@@ -366,10 +366,10 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         free_energy64(jb, g3, h, 0, N, &f2);
         reduce_free<kFP64, false>(f2, g3, scratch);
         if (g2.active && g.r == 0) {
-          ch.Fp = free_value<kFP64>(jb.vb, f1);
+          ch.Fp = free_value<kFP64>(jb, f1);
           ch.Bp = 0.0;
           if (g3.active) {
-            ch.F = free_value<kFP64>(jb.vb, f2);
+            ch.F = free_value<kFP64>(jb, f2);
             ch.Fb = 0.0;
           }
           const double loga = (ch.lpp - ch.lp) + (ch.Fp - ch.F);
@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
       const uint32_t* v = my + ch.cur * P;
       for (int w = g.r; w < jb.Wd; w += g.tpc) jb.bits[(size_t)g.c * jb.Wd + w] = v[w];
       if (g.r == 0) {
-        jb.F[g.c] = free_value<kFP64>(jb.vb, fs);
+        jb.F[g.c] = free_value<kFP64>(jb, fs);
         jb.Fb[g.c] = 0.0;
         jb.Lb[g.c] = ch.lpb;
         jb.logpi[g.c] = ch.lp;
@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     if (g.active && g.r == 0) {
       const double E = KIND == kIsing ? ising_energy(jb, fs.pairs) : kr[1];
       const double lpp = KIND == kIsing ? -ch.beta * E : kr[0];
-      const double Fp = free_value<PREC>(jb.vb, fs);
+      const double Fp = free_value<PREC>(jb, fs);
       ch.Ep = E;
       ch.lpp = lpp;
       ch.cfp = kr[2];
@@ -715,10 +715,10 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
           if (redo_v) fp64_spectrum<PREC, MULTI>(jb, g, v, ch.beta, wk, k0v, nullptr);
         }
         if (g4.active && g.r == 0) {
-          ch.Fp = free_value<kFP64>(jb.vb, f1);
+          ch.Fp = free_value<kFP64>(jb, f1);
           ch.Bp = 0.0;
           if (g3.active) {
-            ch.F = free_value<kFP64>(jb.vb, f2);
+            ch.F = free_value<kFP64>(jb, f2);
             ch.Fb = 0.0;
           }
           if (KIND == kKitaev) {

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_cons
       fs.b = all.b;
       fs.ones = all.ones;
       fs.pairs = all.pairs;
-      const double E = ising_energy(jb, fs.pairs), lpp = -ch.beta * E, Fp = free_value<kMixed>(jb.vb, fs);
+      const double E = ising_energy(jb, fs.pairs), lpp = -ch.beta * E, Fp = free_value<kMixed>(jb, fs);
       ch.Ep = E;
       ch.lpp = lpp;
       ch.onesp = fs.ones;

@@ -538,10 +538,10 @@ static __device__ __noinline__ void mh_redo(const JobDev& jb, ChainSm* chs, doub
     free_energy64(jb, g3, vbits + c * G::WPC, 0, LT * LT, &f2);
     reduce_free<kFP64, false>(f2, g3, scratch);
     if (g4.active && g4.r == 0) {
-      ch.Fp = free_value<kFP64>(jb.vb, f1);
+      ch.Fp = free_value<kFP64>(jb, f1);
       ch.Bp = 0.0;
       if (g3.active) {
-        ch.F = free_value<kFP64>(jb.vb, f2);
+        ch.F = free_value<kFP64>(jb, f2);
         ch.Fb = 0.0;
       }
       const double logr = (ch.lpp - ch.lp) + (ch.Fp - ch.F);

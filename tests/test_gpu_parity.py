@@ -196,6 +196,36 @@ def test_divided_chains_in_a_batch_and_a_graph(ctx):
         j.release()
 
 
+@pytest.mark.parametrize("model,L,K,k,n,hb", [
+    ("ising", 24, 2, 5, 40, 2e6),     # softplus sum 2.3e9, just past 2^31
+    ("ising", 5, 3, 2, 40, 1e9),
+    ("ising", 96, 2, 5, 12, 3e6),     # divided over clusters
+    ("ising", 64, 8, 3, 12, 1e8),
+    ("ising", 24, 2, 5, 40, -2e6),    # silent units: the sum vanishes
+    ("kitaev", 4, 2, 3, 24, 2e8),
+])
+def test_large_free_energies_keep_the_decisions(ctx, model, L, K, k, n, hb):
+    """Filters whose free energy passes any fixed range of the mixed path's sums:
+    its decisions are the FP64 path's whatever the size of F.  Weak filters and
+    temperatures of the lattice's side keep F and log pi of two lattices within a
+    few units, so that proposals are accepted and rejected."""
+    from paper_2008_05401_gb300 import FP64, ISING, KITAEV, MIXED
+    W, _, vb = wl.gaussian_crbm(K, k, 1.0 / (L * k), seed=L * 10 + K)
+    kind, J = (ISING, (1.0,)) if model == "ising" else (KITAEV, (1.0, 1.0, 1.0))
+    T = L * (wl.ising_ladder(n, 8) if model == "ising" else wl.kitaev_ladder(n, 8))
+    bits0 = wl.pack_bits(wl.random_lattices(n, L, seed=L))
+    mid = ctx.load_model(kind, W, vb, np.full(K, hb))
+    S, got = 3, []
+    for prec in (FP64, MIXED):
+        job = ctx.new_job(mid, kind, L, T, J, SEED, 0, bits0, prec)
+        job.run(S, precision=prec)
+        got.append((job.state()[0], job.observables()[1]))
+        job.release()
+    assert 0 < got[0][1].sum() < n * S
+    np.testing.assert_array_equal(got[1][0], got[0][0])
+    np.testing.assert_array_equal(got[1][1], got[0][1])
+
+
 KITAEV_CASES = [
     # L, K, k, n, correct
     (2, 2, 2, 6, True),
