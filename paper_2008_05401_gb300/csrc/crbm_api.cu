@@ -374,10 +374,12 @@ static int launch_group(crbm_ctx* ctx, std::vector<int> ids, int S, int g, int c
 // Whether the proposals of job j run on the tensor-core form: a property of
 // the job alone (kind, precision, lattice, filter bank), so that its results
 // are the same alone or batched.
+// That kernel adds the softplus terms in units of 2^-32, so it takes the jobs
+// whose sum is sure to stay below 2^30; larger filters run on the table kernel.
 static bool on_tc(const crbm_ctx* ctx, const Job& j, int prec, int mode) {
   const Model& m = ctx->models[j.model];
   return ctx->use_tc && ctx->tc_ok && (mode == 0 || mode == 1) && m.d_tc && !m.edge &&
-         tc_supported(j.kind, prec, j.L, m.K, m.k);
+         tc_supported(j.kind, prec, j.L, m.K, m.k) && (double)j.N * m.sp_site < 0x1p30;
 }
 
 // One persistent launch of the tensor-core kernel for the given jobs (any of
