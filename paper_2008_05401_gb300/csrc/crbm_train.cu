@@ -4,8 +4,7 @@
 //   d loss/d theta = (2/M) sum_i (diff_i - C) [ sum_ij sigma(a^f_ij) v_(i+a)(j+b),
 //                                               sum_ij v_ij,  sum_ij sigma(a^f_ij) ]
 // (the W, v_bias, h_bias components; sum_i (diff_i - C) = 0 removes C's own
-// dependence on theta), then ADAM (Kingma & Ba 2014).  Everything is FP64; the
-// sums of sigma run in 64-bit fixed point with FP64's spacing below 2.
+// dependence on theta), then ADAM (Kingma & Ba 2014).  Everything is FP64.
 //
 // One cluster of CTAs per training problem (the paper trains one CRBM per
 // temperature): minibatch steps depend on each other through the parameters,
@@ -21,12 +20,13 @@
 // pipe for about 64 cycles on GB300) and the serial chain of a step.  Hence:
 //   - the sum of log(1 + e^-|x|) of a warp's units is the log of their product
 //     (each factor in (1, 2]): one multiplication per unit instead of a log1p;
-//   - sigma goes to shared memory as round(2^52 sigma), and the gradient's
-//     sums over sites are exact integer additions off the FP64 pipe;
+//   - the gradient's sums over sites are exact 128-bit fixed-point additions of
+//     the FP64 sigma(a) off the FP64 pipe (WideSum), in FP64 for samples with a
+//     unit below their range;
 //   - the bias corrections 1 / (1 - b^t) are taken for 32 steps at a time, one
 //     step per lane (a pow per thread and step was a third of the epoch);
 //   - the next minibatch's samples and targets are fetched during a step.
-// K = 2 5x5, L = 8, 10^4 samples, batch 20: 24 problems 9.0 ms per epoch
+// K = 2 5x5, L = 8, 10^4 samples, batch 20: 24 problems 9.6 ms per epoch
 // (one 512-thread CTA per problem, log1p and pow per unit and thread, FP64
 // gradient sums: 69.3 ms).
 #include <algorithm>
@@ -109,19 +109,45 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src) {
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
+// Exact sum of up to 1024 FP64 values in [kWideMin, 1]: 128-bit fixed point in
+// units of 2^-116, so every bit of every value counts whatever the others' size.
+// About 20 integer instructions an addition, where an FP64 one holds the pipe for
+// 64 cycles (epoch of 24 problems, K = 2 5x5, L = 8: 9.6 ms, 12.0 with FP64 sums).
+constexpr int kWideMinHi = (1023 - 63) << 20;      // high word of 2^-63
+struct WideSum {
+  uint32_t w0 = 0u, w1 = 0u, w2 = 0u, w3 = 0u;
+  // adds x where mask is all ones, nothing where it is 0
+  __device__ __forceinline__ void add(double x, uint32_t mask) {
+    // the 53-bit mantissa, 64 zero bits below it, shifted down by 0 <= sh <= 63
+    const uint32_t xh = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x) & mask;
+    const uint32_t sh = 1023u - (xh >> 20), hi = ((xh & 0xFFFFFu) | 0x100000u) & mask;
+    const bool far = sh >= 32u;
+    const uint32_t t3 = far ? 0u : hi, t2 = far ? hi : lo, t1 = far ? lo : 0u;
+    asm("{\nadd.cc.u32 %0, %0, %4;\naddc.cc.u32 %1, %1, %5;\naddc.cc.u32 %2, %2, %6;\naddc.u32 %3, %3, %7;\n}\n"
+        : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3)
+        : "r"(__funnelshift_r(0u, t1, sh)), "r"(__funnelshift_r(t1, t2, sh)), "r"(__funnelshift_r(t2, t3, sh)),
+          "r"(__funnelshift_r(t3, 0u, sh)));
+  }
+  __device__ __forceinline__ double value() const {
+    const double hi = (double)(((unsigned long long)w3 << 32) | w2), lo = (double)(((unsigned long long)w1 << 32) | w0);
+    return fma(hi, 0x1p-52, lo * 0x1p-116);
+  }
+};
+
 // Warps per sample of unit_pass for ns samples, and the hidden units (a
 // multiple of 32) each takes of the sample's K N.
 __device__ __forceinline__ int segments(int ns) { return ns >= kTrainWarps ? 1 : kTrainWarps / ns; }
 
 // Hidden units of samples [i0, i1): SEG warps per sample, lanes over its
-// units (f, site).  sig[(i - i0) K N + unit] = round(2^52 sigma(a)) of the
+// units (f, site).  sig[(i - i0) K N + unit] = sigma(a) of the
 // samples below i0 + cap; with WANT_F also, per (sample, segment), the sum of
 // max(a, 0) in spos and the product of 1 + e^-|a| in sprod (softplus a =
 // max(a, 0) + log(1 + e^-|a|)).  A product of up to 960 factors of at most 2
-// cannot overflow; longer segments take their lanes' logs first.
+// cannot overflow; longer segments take their lanes' logs first.  Bit i of tiny:
+// sample i holds a sigma below kWideMin.
 template <bool WANT_F>
 __device__ void unit_pass(const uint32_t* vb, int Wd, const double* tab, const double* hbias, int K, int k, int T,
-                          int L, int i0, int i1, int cap, unsigned long long* sig, double* spos, double* sprod) {
+                          int L, int i0, int i1, int cap, double* sig, double* spos, double* sprod, unsigned* tiny) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = L * L, U = K * N;
   const int SEG = segments(i1 - i0), span = ((U + SEG - 1) / SEG + 31) & ~31;
   for (int task = warp; task < (i1 - i0) * SEG; task += kTrainWarps) {
@@ -129,6 +155,7 @@ __device__ void unit_pass(const uint32_t* vb, int Wd, const double* tab, const d
     const uint32_t* v = vb + i * Wd;
     const bool keep = i - i0 < cap;
     double pos = 0.0, prod = 1.0;
+    bool small = false;
     for (int u = u0 + lane; u < u1; u += 32) {
       const int f = u / N, s = u - f * N, si = s / L, sj = s - si * L;
       double x = hbias[f];
@@ -138,15 +165,16 @@ __device__ void unit_pass(const uint32_t* vb, int Wd, const double* tab, const d
       }
       const double e = exp(-fabs(x)), d = 1.0 + e;
       if (keep) {
-        // 1 + sigma in [1, 2]: the FP64 addition rounds sigma to a multiple of 2^-52
-        const double y = 1.0 + (x >= 0.0 ? 1.0 : e) / d;
-        sig[(size_t)(i - i0) * U + u] = (unsigned long long)(__double_as_longlong(y) - __double_as_longlong(1.0));
+        const double y = (x >= 0.0 ? 1.0 : e) / d;
+        sig[(size_t)(i - i0) * U + u] = y;
+        small = small || __double2hiint(y) < kWideMinHi;
       }
       if (WANT_F) {
         pos += fmax(x, 0.0);
         prod *= d;
       }
     }
+    if (__any_sync(kFull, small) && lane == 0) atomicOr(tiny + (i >> 5), 1u << (i & 31));
     if (WANT_F) {
       if (span > 960) {
         pos += log(prod);
@@ -171,6 +199,28 @@ __device__ __forceinline__ int count_ones(const uint32_t* v, int Wd) {
   return c;
 }
 
+// Sum of sp[si L + j] over the sites of rows si = s0, s0 + step, .. whose bit j of
+// row(si) is set.
+template <class ROW>
+__device__ __forceinline__ double site_sum(const double* sp, int L, int s0, int step, bool exact, ROW row) {
+  WideSum wide;
+  double sum = 0.0;
+  for (int si = s0; si < L; si += step) {
+    const double* x = sp + si * L;
+    const uint32_t win = row(si);
+    if (exact) {
+#pragma unroll 8
+      for (int j = 0; j < L; ++j) wide.add(x[j], 0u - ((win >> j) & 1u));
+    } else {
+      double part = 0.0;
+      for (int j = 0; j < L; ++j)
+        if ((win >> j) & 1u) part += x[j];
+      sum += part;
+    }
+  }
+  return exact ? wide.value() : sum;
+}
+
 __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __grid_constant__ TrainParams p) {
   cg::cluster_group cl = cg::this_cluster();
   const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -181,6 +231,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __g
   const int M = p.batch, per = p.per, cap = sig_capacity(K, N);
 
   extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned tiny[kMaxBatch / 32];
   const TrainLayout y = train_layout(K, k, L, M, per);
   double* th = (double*)(smem + y.th);
   double* am = (double*)(smem + y.am);
@@ -194,7 +245,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __g
   double* sprod = (double*)(smem + y.sprod);
   double* rbc = (double*)(smem + y.rbc);
   double* part = (double*)(smem + y.part);
-  unsigned long long* sig = (unsigned long long*)(smem + y.sig);
+  double* sig = (double*)(smem + y.sig);
   int* ord = (int*)(smem + y.ord);
   uint32_t* bits = (uint32_t*)(smem + y.bits);
 
@@ -238,6 +289,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __g
     // the next minibatch's data and the order of the one after it (waited for at the step's end)
     if (b + 1 < nb) fetch(b + 1);
     if (b + 2 < nb) fetch_order(b + 2);
+    if (tid < kMaxBatch / 32) tiny[tid] = 0u;
     // (1) row-sum tables of the current filters (bits summed in increasing b)
     for (int e = tid; e < nlut; e += kTrainThreads) {
       const int code = e % T, fa = e / T;
@@ -255,7 +307,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __g
     const double vbias = th[nW];
     const double* hbias = th + nW + 1;
     // (2) F of this CTA's samples (and the hidden probabilities of the first chunk)
-    if (ns > 0) unit_pass<true>(vb, Wd, tab, hbias, K, k, T, L, 0, ns, cap, sig, spos, sprod);
+    if (ns > 0) unit_pass<true>(vb, Wd, tab, hbias, K, k, T, L, 0, ns, cap, sig, spos, sprod, tiny);
     __syncthreads();
     if (warp == 0) {
       const int SEG = ns > 0 ? segments(ns) : 1;
@@ -298,52 +350,45 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __g
     }
     __syncthreads();
     // (3) this CTA's gradient sums, chunks of samples whose probabilities are
-    // in shared memory: thread (parameter, sample group), sites as integers,
-    // then cw_i times the sum in FP64; the groups' partials added in order
-    const int SG = max(1, min(ns, kTrainThreads / P));
-    const int pp = tid % P, sg = tid / P;
+    // in shared memory: thread (parameter, sample group, every RS-th row), sites
+    // exactly or, where one is too small for that, row by row in FP64, then cw_i
+    // times the sum; the groups' partials added in order
+    const int SG = max(1, min(ns, kTrainThreads / P)), RS = min(L, kTrainThreads / P / SG), groups = SG * RS;
+    const int pp = tid % P, grp = tid / P, sg = grp % SG, row0 = grp / SG;
     double acc = 0.0;
     for (int i0 = 0; i0 < ns; i0 += cap) {
       const int i1 = min(ns, i0 + cap);
       if (i0 > 0) {
         // the first pass kept the probabilities of the first chunk only: recompute this one
         __syncthreads();
-        unit_pass<false>(vb, Wd, tab, hbias, K, k, T, L, i0, i1, cap, sig, nullptr, nullptr);
+        unit_pass<false>(vb, Wd, tab, hbias, K, k, T, L, i0, i1, cap, sig, nullptr, nullptr, tiny);
         __syncthreads();
       }
-      if (sg < SG) {
+      if (grp < groups) {
         for (int i = i0 + sg; i < i1; i += SG) {
           const uint32_t* v = vb + i * Wd;
-          const unsigned long long* sp = sig + (size_t)(i - i0) * U;
-          unsigned long long sum = 0ull;
-          if (pp < nW) {
-            const int f = pp / (k * k), ab = pp - f * k * k, a = ab / k, bb = ab - a * k;
-            sp += f * N;
-            for (int si = 0; si < L; ++si) {
-              // bit j of the window: v at (si + a, j + bb), periodic
-              const int r = si + a < L ? si + a : si + a - L;
-              const uint32_t lo = row_window(v, L, r, bb, L < 16 ? L : 16);
-              const uint32_t hi = L > 16 ? row_window(v, L, r, bb + 16 < L ? bb + 16 : bb + 16 - L, L - 16) : 0u;
-              const uint32_t win = lo | (hi << 16);
-#pragma unroll 8
-              for (int j = 0; j < L; ++j)
-                if ((win >> j) & 1u) sum += sp[si * L + j];
-            }
-          } else if (pp == nW) {
-            sum = (unsigned long long)count_ones(v, Wd) << 52;
-          } else {
-            sp += (pp - nW - 1) * N;
-            for (int s = 0; s < N; ++s) sum += sp[s];
+          const bool exact = ((tiny[i >> 5] >> (i & 31)) & 1u) == 0u;
+          if (pp == nW) {
+            if (row0 == 0) acc = fma(cw[i], (double)count_ones(v, Wd), acc);
+            continue;
           }
-          acc = fma(cw[i], (double)sum, acc);           // sum in units of 2^-52
+          // W^f_ab: the sites whose v at (si + a, j + b), periodic, is set; h_bias^f: all
+          const bool tap = pp < nW;
+          const int f = tap ? pp / (k * k) : pp - nW - 1, ab = tap ? pp - f * k * k : 0, a = ab / k, bb = ab - a * k;
+          acc = fma(cw[i], site_sum(sig + (size_t)(i - i0) * U + f * N, L, row0, RS, exact, [&](int si) {
+            const int r = si + a < L ? si + a : si + a - L;
+            const uint32_t lo = row_window(v, L, r, bb, L < 16 ? L : 16);
+            const uint32_t hi = L > 16 ? row_window(v, L, r, bb + 16 < L ? bb + 16 : bb + 16 - L, L - 16) : 0u;
+            return tap ? lo | (hi << 16) : ~0u;
+          }), acc);
         }
       }
     }
-    if (sg < SG) part[sg * P + pp] = acc * 0x1p-52;
+    if (grp < groups) part[grp * P + pp] = acc;
     __syncthreads();
     for (int i = tid; i < P; i += kTrainThreads) {
       double s = 0.0;
-      for (int g = 0; g < SG; ++g) s += part[g * P + i];
+      for (int g = 0; g < groups; ++g) s += part[g * P + i];
       gr[i] = s;
     }
     cl.sync();

@@ -166,6 +166,34 @@ def test_cluster_split_matches_oracle(ctx, n_problems, K, k, L, n, batch):
         assert int(probs[i].t.item()) == st.t == steps
 
 
+@pytest.mark.parametrize("L,k,hb", [(8, 3, (0.0, -25.0)), (8, 3, (0.0, -40.0)), (17, 2, (0.5, -60.0))])
+def test_silent_filters_keep_their_gradient(ctx, L, k, hb):
+    """A filter whose units are all but off has a gradient of its own (small)
+    size, which ADAM's normalisation restores.  One minibatch from zero moments:
+    m / (1 - b1) is the gradient (2/M) sum_i d_i S_i, d_i = t_i - F_i - C, S_i >= 0
+    a sum of at most N sigmas.  FP64 leaves d_i within 1e-12 (|t_i| + |F_i|) and
+    S_i within 1e-12 of itself (a few hundred units of 2^-53 each)."""
+    import torch
+    from oracle import train
+    from paper_2008_05401_gb300 import trainer
+    n, K = 20, len(hb)
+    v = wl.random_lattices(n, L, seed=L)
+    rng = np.random.default_rng(5)
+    t = rng.normal(0.0, 3.0, n)
+    th0 = np.concatenate([rng.normal(0.0, 0.3, K * k * k), [0.1], hb])
+    prob = trainer.Problem.new(ctx, K, k, L, th0)
+    losses = trainer.train_epochs(ctx, [prob], [torch.tensor(wl.pack_bits(v).view(np.int32), device="cuda:0")],
+                                  [torch.tensor(t, device="cuda:0")], [torch.arange(n, dtype=torch.int32, device="cuda:0")], n)
+    F, G = train.free_energy_grad(v, th0, K, k)
+    d = t - F - (t - F).mean()
+    off = 1e-12 * (np.abs(t) + np.abs(F))
+    off += off.mean()
+    tol = (2.0 / n) * ((off + 1e-12 * np.abs(d))[:, None] * np.abs(G)).sum(0)
+    g = -(2.0 / n) * (d[:, None] * G).sum(0)
+    assert np.all(np.abs(prob.m.cpu().numpy() / (1.0 - 0.9) - g) <= tol + 1e-13 * np.abs(g))
+    assert abs(losses[0].item() - (d * d).mean()) <= 2.0 * (np.abs(d) * off).mean() + 1e-13 * (d * d).mean()
+
+
 def test_train_rejects_bad_shapes(ctx):
     import torch
     from paper_2008_05401_gb300 import CrbmError, trainer
