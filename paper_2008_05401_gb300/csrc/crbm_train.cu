@@ -18,15 +18,15 @@
 //
 // What bounds it: the FP64 pipe (a warp instruction holds its sub-partition's
 // pipe for about 64 cycles on GB300) and the serial chain of a step.  Hence:
-//   - the sum of log(1 + e^-|x|) of a warp's units is the log of their product
-//     (each factor in (1, 2]): one multiplication per unit instead of a log1p;
+//   - the sum of log(1 + e^-|x|) of a warp's units is the log of their product:
+//     two operations per unit (join_log1p) instead of a log1p;
 //   - the gradient's sums over sites are exact 128-bit fixed-point additions of
 //     the FP64 sigma(a) off the FP64 pipe (WideSum), in FP64 for samples with a
 //     unit below their range;
 //   - the bias corrections 1 / (1 - b^t) are taken for 32 steps at a time, one
 //     step per lane (a pow per thread and step was a third of the epoch);
 //   - the next minibatch's samples and targets are fetched during a step.
-// K = 2 5x5, L = 8, 10^4 samples, batch 20: 24 problems 9.6 ms per epoch
+// K = 2 5x5, L = 8, 10^4 samples, batch 20: 24 problems 9.8 ms per epoch
 // (one 512-thread CTA per problem, log1p and pow per unit and thread, FP64
 // gradient sums: 69.3 ms).
 #include <algorithm>
@@ -140,21 +140,24 @@ __device__ __forceinline__ int segments(int ns) { return ns >= kTrainWarps ? 1 :
 
 // Hidden units of samples [i0, i1): SEG warps per sample, lanes over its
 // units (f, site).  sig[(i - i0) K N + unit] = sigma(a) of the
-// samples below i0 + cap; with WANT_F also, per (sample, segment), the sum of
-// max(a, 0) in spos and the product of 1 + e^-|a| in sprod (softplus a =
-// max(a, 0) + log(1 + e^-|a|)).  A product of up to 960 factors of at most 2
-// cannot overflow; longer segments take their lanes' logs first.  Bit i of tiny:
-// sample i holds a sigma below kWideMin.
+// samples below i0 + cap; with WANT_F also, per (sample, segment), softplus a =
+// log(1 + e^a) as a product of the factors, less 1, in sprod, or, where a is above
+// the bound that keeps the product below e^700, as a in spos and the factor
+// 1 + e^-a (spos is rarely needed, and so is its sum over the lanes).  Segments
+// longer than 960 units take their lanes' logs first.  Bit i of tiny: sample i
+// holds a sigma below kWideMin.
 template <bool WANT_F>
 __device__ void unit_pass(const uint32_t* vb, int Wd, const double* tab, const double* hbias, int K, int k, int T,
                           int L, int i0, int i1, int cap, double* sig, double* spos, double* sprod, unsigned* tiny) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = L * L, U = K * N;
   const int SEG = segments(i1 - i0), span = ((U + SEG - 1) / SEG + 31) & ~31;
+  // n factors of at most 1 + e^top < 2 e^top
+  const double top = (double)(__fdividef(700.0f, (float)(span > 960 ? span / 32 : span)) - 0.7f);
   for (int task = warp; task < (i1 - i0) * SEG; task += kTrainWarps) {
     const int i = i0 + task / SEG, u0 = (task % SEG) * span, u1 = min(U, u0 + span);
     const uint32_t* v = vb + i * Wd;
     const bool keep = i - i0 < cap;
-    double pos = 0.0, prod = 1.0;
+    double pos = 0.0, prod = 0.0;
     bool small = false;
     for (int u = u0 + lane; u < u1; u += 32) {
       const int f = u / N, s = u - f * N, si = s / L, sj = s - si * L;
@@ -163,28 +166,27 @@ __device__ void unit_pass(const uint32_t* vb, int Wd, const double* tab, const d
         const int r = si + a < L ? si + a : si + a - L;
         x += tab[(f * k + a) * T + (int)row_window(v, L, r, sj, k)];
       }
-      const double e = exp(-fabs(x)), d = 1.0 + e;
+      const bool up = x <= top;
+      const double e = exp(up ? x : -x), d = 1.0 + e;
       if (keep) {
-        const double y = (x >= 0.0 ? 1.0 : e) / d;
+        const double y = (up ? e : 1.0) / d;
         sig[(size_t)(i - i0) * U + u] = y;
         small = small || __double2hiint(y) < kWideMinHi;
       }
       if (WANT_F) {
-        pos += fmax(x, 0.0);
-        prod *= d;
+        if (!up) pos += x;
+        prod = join_log1p(prod, e);
       }
     }
     if (__any_sync(kFull, small) && lane == 0) atomicOr(tiny + (i >> 5), 1u << (i & 31));
     if (WANT_F) {
       if (span > 960) {
-        pos += log(prod);
-        prod = 1.0;
+        pos += log_joined(prod);
+        prod = 0.0;
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        pos += __shfl_xor_sync(kFull, pos, o);
-        prod *= __shfl_xor_sync(kFull, prod, o);
-      }
+      for (int o = 16; o > 0; o >>= 1) prod = join_log1p(prod, __shfl_xor_sync(kFull, prod, o));
+      if (__any_sync(kFull, pos != 0.0)) pos = warp_sum64(pos);
       if (lane == 0) {
         spos[task] = pos;
         sprod[task] = prod;
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_epoch_kernel(const __g
     __syncthreads();
     if (warp == 0) {
       const int SEG = ns > 0 ? segments(ns) : 1;
-      for (int e = lane; e < ns * SEG; e += 32) spos[e] += log(sprod[e]);
+      for (int e = lane; e < ns * SEG; e += 32) spos[e] += log_joined(sprod[e]);
       __syncwarp();
       for (int i = lane; i < ns; i += 32) {
         double sp = 0.0;

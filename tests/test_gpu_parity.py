@@ -228,6 +228,24 @@ def test_large_free_energies_keep_the_decisions(ctx, model, L, K, k, n, hb):
     np.testing.assert_array_equal(got[1][1], got[0][1])
 
 
+@pytest.mark.parametrize("L,n,hb", [(8, 16, -25.0), (8, 16, -40.0), (24, 4, -60.0), (256, 1, -38.0), (3, 700, -300.0)])
+def test_silent_units_keep_their_free_energy(ctx, L, n, hb):
+    """F of a model whose units are all but off is the small sum of their softplus
+    terms, to FP64's relative rounding (a few units of 2^-53 per term and
+    addition), in an evaluation and at a run's end."""
+    from oracle import crbm
+    from paper_2008_05401_gb300 import FP64, ISING
+    W, _, _ = wl.gaussian_crbm(2, 3, 0.3, seed=L)
+    bits0 = wl.pack_bits(wl.random_lattices(n, L, seed=L))
+    mid = ctx.load_model(ISING, W, 0.0, np.full(2, hb))
+    job = ctx.new_job(mid, ISING, L, wl.ising_ladder(n, 8), (1.0,), SEED, 0, bits0, FP64)
+    for S in (0, 2):
+        job.run(S, precision=FP64)
+        F = crbm.free_energy(wl.unpack_bits(job.state()[0], L), W, np.full(2, hb), 0.0)
+        np.testing.assert_allclose(job.energies()[1], F, rtol=1e-12, atol=0.0)
+    job.release()
+
+
 KITAEV_CASES = [
     # L, K, k, n, correct
     (2, 2, 2, 6, True),

@@ -166,8 +166,12 @@ def test_cluster_split_matches_oracle(ctx, n_problems, K, k, L, n, batch):
         assert int(probs[i].t.item()) == st.t == steps
 
 
-@pytest.mark.parametrize("L,k,hb", [(8, 3, (0.0, -25.0)), (8, 3, (0.0, -40.0)), (17, 2, (0.5, -60.0))])
-def test_silent_filters_keep_their_gradient(ctx, L, k, hb):
+@pytest.mark.parametrize("L,k,hb,vb,spread", [(8, 3, (0.0, -25.0), 0.1, 3.0), (8, 3, (0.0, -40.0), 0.1, 3.0),
+                                                 (17, 2, (0.5, -60.0), 0.1, 3.0),
+                                                 (8, 3, (25.0, -40.0), 0.1, 3.0), (17, 2, (60.0, 1.0), 0.1, 3.0),
+                                                 (8, 3, (-30.0, -35.0), 0.0, 0.0),     # F itself that small
+                                                 (31, 2, (-30.0, -38.0), 0.0, 0.0)])
+def test_silent_filters_keep_their_gradient(ctx, L, k, hb, vb, spread):
     """A filter whose units are all but off has a gradient of its own (small)
     size, which ADAM's normalisation restores.  One minibatch from zero moments:
     m / (1 - b1) is the gradient (2/M) sum_i d_i S_i, d_i = t_i - F_i - C, S_i >= 0
@@ -179,8 +183,8 @@ def test_silent_filters_keep_their_gradient(ctx, L, k, hb):
     n, K = 20, len(hb)
     v = wl.random_lattices(n, L, seed=L)
     rng = np.random.default_rng(5)
-    t = rng.normal(0.0, 3.0, n)
-    th0 = np.concatenate([rng.normal(0.0, 0.3, K * k * k), [0.1], hb])
+    t = rng.normal(0.0, spread, n)
+    th0 = np.concatenate([rng.normal(0.0, 0.3, K * k * k), [vb], hb])
     prob = trainer.Problem.new(ctx, K, k, L, th0)
     losses = trainer.train_epochs(ctx, [prob], [torch.tensor(wl.pack_bits(v).view(np.int32), device="cuda:0")],
                                   [torch.tensor(t, device="cuda:0")], [torch.arange(n, dtype=torch.int32, device="cuda:0")], n)
