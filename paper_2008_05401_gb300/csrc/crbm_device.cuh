@@ -804,18 +804,17 @@ __device__ __forceinline__ double log_joined(double p) {
   return log(u) + (p < 1.0 ? p - (u - 1.0) : 0.0);
 }
 
-// FP64 form: thread (filter, site), sites n0 .. n1 - 1; the log(1 + e^-|x|) of a
+// FP64 form: thread (filter, site); the log(1 + e^-|x|) of a
 // thread's units are the log of their product (factors in (1, 2], the log taken at
 // least every 512), kept less 1.
-__device__ inline FreeSum free_phase64(const JobDev& jb, const double* f64, const Grp& g, const uint32_t* v, int n0,
-                                       int n1) {
-  const int L = jb.L, K = jb.K, k = jb.k, T = 1 << k;
+__device__ inline FreeSum free_phase64(const JobDev& jb, const double* f64, const Grp& g, const uint32_t* v) {
+  const int L = jb.L, N = jb.N, K = jb.K, k = jb.k, T = 1 << k;
   FreeSum out = {0.0, 0ll, 0.0f, 0, 0};
   if (!g.active) return out;
   double prod = 0.0;
   int held = 0;
-  for (int e = g.r; e < K * (n1 - n0); e += g.tpc) {
-    const int f = e / (n1 - n0), n = n0 + e - f * (n1 - n0), i = n / L, j = n - i * L;
+  for (int e = g.r; e < K * N; e += g.tpc) {
+    const int f = e / N, n = e - f * N, i = n / L, j = n - i * L;
     double x = jb.hb[f];
     if (jb.lc_edge) {
       x = lc_preact64(jb, f64, f, v, n, k, T);
@@ -834,7 +833,7 @@ __device__ inline FreeSum free_phase64(const JobDev& jb, const double* f64, cons
     }
   }
   if (held) out.s += log_joined(prod);
-  for (int n = n0 + g.r; n < n1; n += g.tpc) {
+  for (int n = g.r; n < N; n += g.tpc) {
     const int i = n / L, j = n - i * L, jr = j + 1 == L ? 0 : j + 1;
     const uint32_t b0 = site_bit(v, n);
     out.ones += (int)b0;

@@ -51,9 +51,8 @@ __host__ __device__ inline size_t kitaev_work_bytes(int N) {
 }
 
 // The mixed path's FP64 free energy (rare), out of line to spare registers.
-static __device__ __noinline__ void free_energy64(const JobDev& jb, const Grp& g, const uint32_t* v, int n0, int n1,
-                                                  FreeSum* out) {
-  *out = free_phase64(jb, jb.f64, g, v, n0, n1);
+static __device__ __noinline__ void free_energy64(const JobDev& jb, const Grp& g, const uint32_t* v, FreeSum* out) {
+  *out = free_phase64(jb, jb.f64, g, v);
 }
 
 // Observables of a lattice: Ising from E and the number of ones; Kitaev from
@@ -282,7 +281,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     // current lattices
     FreeSum fs;
     if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, my, ex, 0, nblk);
-    else fs = free_phase64(jb, tb.f64, g, my, 0, N);
+    else fs = free_phase64(jb, tb.f64, g, my);
     reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
     if (KIND == kKitaev)
@@ -318,7 +317,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
                               []() { __syncthreads(); });
     FreeSum fs;
     if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp, ex + jb.L, 0, nblk);
-    else fs = free_phase64(jb, tb.f64, g, vp, 0, N);
+    else fs = free_phase64(jb, tb.f64, g, vp);
     reduce_free<PREC, false>(fs, g, scratch);
     double kr[3] = {0.0, 0.0, 0.0};
     if (KIND == kKitaev)
@@ -358,12 +357,12 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         Grp g2 = g;
         g2.active = g.active && ch.flag_rec;
         FreeSum f1;
-        free_energy64(jb, g2, vp, 0, N, &f1);
+        free_energy64(jb, g2, vp, &f1);
         reduce_free<kFP64, false>(f1, g2, scratch);
         Grp g3 = g2;
         g3.active = g2.active && ch.Fb != 0.0;
         FreeSum f2;
-        free_energy64(jb, g3, h, 0, N, &f2);
+        free_energy64(jb, g3, h, &f2);
         reduce_free<kFP64, false>(f2, g3, scratch);
         if (g2.active && g.r == 0) {
           ch.Fp = free_value<kFP64>(jb, f1);
@@ -531,7 +530,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
     }
     // FP64 free energy of the final lattices, then everything back to the job
     FreeSum fs;
-    free_energy64(jb, g, my + ch.cur * P, 0, N, &fs);
+    free_energy64(jb, g, my + ch.cur * P, &fs);
     reduce_free<kFP64, false>(fs, g, scratch);
     if (g.active) {
       const uint32_t* v = my + ch.cur * P;
@@ -607,7 +606,7 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
                               nrec, loop_sync);
     FreeSum fs;
     if constexpr (PREC == kMixed) fs = free_phase<KC, kC>(jb, tb, g, vp, ex + (cur ^ 1) * jb.L, 0, nblk);
-    else fs = free_phase64(jb, tb.f64, g, vp, 0, N);
+    else fs = free_phase64(jb, tb.f64, g, vp);
     loop_reduce(fs, g, std::integral_constant<int, PREC>());
     double kr[4] = {0.0, 0.0, 0.0, 0.0};
     if (KIND == kKitaev) {
@@ -699,12 +698,12 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         Grp g4 = g2;
         g4.active = g2.active && (KIND == kKitaev || ch.flag_rec == 2);
         FreeSum f1;
-        free_energy64(jb, g4, vp, 0, N, &f1);
+        free_energy64(jb, g4, vp, &f1);
         loop_reduce(f1, g4, std::integral_constant<int, kFP64>());
         Grp g3 = g4;
         g3.active = g4.active && ch.Fb != 0.0;
         FreeSum f2;
-        free_energy64(jb, g3, v, 0, N, &f2);
+        free_energy64(jb, g3, v, &f2);
         loop_reduce(f2, g3, std::integral_constant<int, kFP64>());
         // Kitaev: the FP64 eigen-stage of v' (and of v when its log-weight
         // came from the df64 stage), by the group that needs it

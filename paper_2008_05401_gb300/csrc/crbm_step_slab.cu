@@ -197,19 +197,30 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_cons
     }
     // every CTA holds the same values, so the cluster takes these branches together
     if (__syncthreads_or(tid == 0 && ch.flag_rec)) {
-      auto level = [&](bool df64, const uint32_t* lattice) {
+      // df64 softplus: the CTAs' rows, summed over the cluster; FP64: the whole
+      // lattice in every CTA, by the FP64 path's threads in its order, so that the
+      // decision is that path's to the last bit (rare)
+      auto level = [&](bool df64, uint32_t* lattice) {
         SlabSum mine = {{0.0, 0.0, 0.0}, 0ll, 0.0f, 0, 0};
         if (df64) {
           free_sum_df<KC ? KC : kMaxK>(jb, g, lattice, n0, n1, mine.d);
           grp_reduce<3>(mine.d, g, scratch);
-        } else {
-          FreeSum f;
-          free_energy64(jb, g, lattice, n0, n1, &f);
-          reduce_free<kFP64, false>(f, g, scratch);
-          mine.d[0] = f.s;
-          mine.d[2] = (double)f.ones;
+          return cluster_sum(cl, mine, slots, turn);
         }
-        return cluster_sum(cl, mine, slots, turn);
+        for (int w = tid; w < Wd; w += kSlabThreads) {
+          const int owner = ((w / WL + 1) * CL - 1) / L;
+          if (owner != rank) lattice[w] = cl.map_shared_rank(lattice, owner)[w];
+        }
+        __syncthreads();
+        Grp g64 = g;
+        g64.tpc = kThreads / jb.nc;
+        g64.active = tid < g64.tpc;
+        FreeSum f;
+        free_energy64(jb, g64, lattice, &f);
+        reduce_free<kFP64, false>(f, g64, scratch);
+        mine.d[0] = f.s;
+        mine.d[2] = (double)f.ones;
+        return mine;
       };
       const bool redo_v = ch.Fb != 0.0;
       // second level: df64 softplus; then, inside its bound too, the FP64 path's own

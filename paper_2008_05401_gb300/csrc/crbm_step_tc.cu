@@ -530,12 +530,12 @@ static __device__ __noinline__ void mh_redo(const JobDev& jb, ChainSm* chs, doub
     Grp g4 = g2;
     g4.active = g2.active && ch.flag_rec == 2;
     FreeSum f1;
-    free_energy64(jb, g4, pv + c * G::WPC, 0, LT * LT, &f1);
+    free_energy64(jb, g4, pv + c * G::WPC, &f1);
     reduce_free<kFP64, false>(f1, g4, scratch);
     Grp g3 = g4;
     g3.active = g4.active && ch.Fb != 0.0;
     FreeSum f2;
-    free_energy64(jb, g3, vbits + c * G::WPC, 0, LT * LT, &f2);
+    free_energy64(jb, g3, vbits + c * G::WPC, &f2);
     reduce_free<kFP64, false>(f2, g3, scratch);
     if (g4.active && g4.r == 0) {
       ch.Fp = free_value<kFP64>(jb, f1);

@@ -205,6 +205,10 @@ def test_divided_chains_in_a_batch_and_a_graph(ctx):
     ("kitaev", 4, 2, 3, 24, 2e8),
     ("ising", 16, 4, 5, 40, 3e6),     # a side and shape of the tensor-core form
     ("ising", 128, 2, 3, 12, 1e5),
+    # F's own FP64 rounding of the size of the decisions: the same order of its sums too
+    ("ising", 24, 2, 5, 40, 1e12),
+    ("ising", 96, 2, 5, 12, 1e12),
+    ("ising", 64, 8, 3, 40, 1e12),
 ])
 def test_large_free_energies_keep_the_decisions(ctx, model, L, K, k, n, hb):
     """Filters whose free energy passes any fixed range of the mixed path's sums:
