@@ -24,6 +24,7 @@ namespace crbm {
 namespace {
 
 constexpr int kTauThreads = 256;
+constexpr int kTauStatic = 4096;                   // of a CTA's shared memory, for the static arrays
 
 constexpr int kLagTile = 16;                       // lags of a warp
 constexpr int kLagGroups = 2;                      // lag tiles of a round
@@ -151,6 +152,13 @@ static __device__ __align__(256) unsigned char g_tau_scratch[kMaxNoAllocSeries *
 
 }  // namespace
 
+// The kernel's limit is the process's, so it is set once to the most that any
+// call takes (with a context's creation), not by each call to its own size:
+// another thread's call between that and the launch would lower it.
+cudaError_t tau_set_smem_limit(size_t optin) {
+  return cudaFuncSetAttribute(tau_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)optin - kTauStatic);
+}
+
 static cudaError_t launch_tau_kernel(const double* x, int n_series, long long n, double c, double* tau, long long* w,
                                      cudaStream_t st) {
   // a series that does not fit the shared memory of a CTA is read from global memory
@@ -159,12 +167,10 @@ static cudaError_t launch_tau_kernel(const double* x, int n_series, long long n,
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   const long long bytes = (n + kLagTile) * 8;
-  if (bytes > optin - 4096) {
+  if (bytes > optin - kTauStatic) {
     tau_kernel<false><<<n_series, kTauThreads, 0, st>>>(x, n_series, n, c, tau, w);
     return cudaGetLastError();
   }
-  e = cudaFuncSetAttribute(tau_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
   tau_kernel<true><<<n_series, kTauThreads, (size_t)bytes, st>>>(x, n_series, n, c, tau, w);
   return cudaGetLastError();
 }

@@ -556,6 +556,8 @@ int crbm_create(crbm_ctx** out, int device, size_t hbm_budget_bytes) {
     ctx->smem_optin = (size_t)optin;
     e = set_smem_limits((size_t)optin);
     if (e == cudaSuccess) e = slab_set_smem_limit((size_t)optin);
+    if (e == cudaSuccess) e = tau_set_smem_limit((size_t)optin);
+    if (e == cudaSuccess) e = train_set_smem_limit((size_t)optin);
     if (e == cudaSuccess && (size_t)optin >= tc_smem_bytes(128, 4, 5)) {
       e = tc_set_smem_limit();
       ctx->tc_ok = e == cudaSuccess;

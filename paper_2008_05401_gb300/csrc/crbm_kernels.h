@@ -67,6 +67,7 @@ cudaError_t launch_ising_sweeps(const JobDev& j, int S, bool add, cudaStream_t s
 // [n][n_series] device array (crbm_analysis.cu); tau and w are device arrays.
 cudaError_t launch_tau(const double* x, int n_series, long long n, double c, double* tau, long long* w,
                        cudaStream_t st);
+cudaError_t tau_set_smem_limit(size_t optin);
 // The same into a fixed device scratch array (no device allocation), results
 // copied to the host arrays; returns after the copies.  n_series must not
 // exceed CRBM_AUTOCORR_NOALLOC_MAX_SERIES.
@@ -78,6 +79,7 @@ cudaError_t launch_tau_noalloc(const double* x, int n_series, long long n, doubl
 #include "crbm.h"
 namespace crbm {
 size_t train_smem_bytes(const crbm_train_problem& q, int batch);
+cudaError_t train_set_smem_limit(size_t optin);
 // Measured FP32 / FP64 FMA throughput of `device` (crbm_analysis.cu).
 cudaError_t probe_fma_peaks(int device, double* fp32_tflops, double* fp64_tflops, cudaStream_t st);
 cudaError_t launch_train(const crbm_train_problem* pr, int n, int batch, double lr, double b1, double b2,

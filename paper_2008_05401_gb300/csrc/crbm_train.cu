@@ -439,6 +439,12 @@ size_t train_smem_bytes(const crbm_train_problem& q, int batch) {
   return (size_t)train_layout(q.K, q.k, q.L, batch, batch).total;
 }
 
+// Once for the process (with a context's creation): a limit set by each call would
+// be lowered by another thread's call between that and the launch.
+cudaError_t train_set_smem_limit(size_t optin) {
+  return cudaFuncSetAttribute(train_epoch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)optin - 1024);
+}
+
 cudaError_t launch_train(const crbm_train_problem* pr, int n, int batch, double lr, double b1, double b2,
                          double eps, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
@@ -455,8 +461,6 @@ cudaError_t launch_train(const crbm_train_problem* pr, int n, int batch, double 
     p.pr[i] = pr[i];
     smem = std::max(smem, (size_t)train_layout(pr[i].K, pr[i].k, pr[i].L, batch, p.per).total);
   }
-  cudaError_t e = cudaFuncSetAttribute(train_epoch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(n * CL));
   cfg.blockDim = dim3(kTrainThreads);

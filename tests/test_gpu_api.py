@@ -375,3 +375,56 @@ def test_autotuned_tile_shape_keeps_parity(ctx):
         np.testing.assert_array_equal(job.state()[0], wl.pack_bits(ref.v))
         np.testing.assert_array_equal(job.observables()[1], ref.accepts)
     job.release()
+
+
+def _side_by_side(calls, rounds):
+    """Each of `calls` repeated `rounds` times in a thread of its own; their exceptions."""
+    import threading
+    errors = []
+
+    def work(fn):
+        try:
+            for _ in range(rounds):
+                fn()
+        except Exception as e:          # the assertion is the caller's
+            errors.append(e)
+    threads = [threading.Thread(target=work, args=(fn,)) for fn in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    return errors
+
+
+def test_threads_with_contexts_of_their_own():
+    """Two host threads, a context and a stream each: series (and training
+    problems) that need much and little shared memory side by side."""
+    import ctypes
+
+    import torch
+    from paper_2008_05401_gb300 import Context, binding, trainer
+    ctxs = [gpu_ctx(), Context(0)]
+    streams = [torch.cuda.Stream() for _ in ctxs]
+    series = [torch.randn(n, 1, dtype=torch.float64, device="cuda:0") for n in (20000, 50)]
+    want = [c.autocorr(x) for c, x in zip(ctxs, series)]
+    # problems without samples, many to a call: launches back to back
+    probs = [trainer.Problem.new(c, 4, 3, L, wl.init_train_params(4, 3, seed=L)) for c, L in zip(ctxs, (31, 4))]
+    many = 4096
+    descs = [(binding.TrainProblem * many)(*[binding.TrainProblem(
+        p.K, p.k, p.L, 0, None, None, None, p.theta.data_ptr(), p.m.data_ptr(), p.v.data_ptr(), p.t.data_ptr(), None)] * many)
+        for p in probs]
+
+    def train(i):
+        rc = binding.load().crbm_train_epochs(ctxs[i].h, many, ctypes.cast(descs[i], ctypes.c_void_p), 4, 1e-3, 0.9, 0.999,
+                                              1e-8, ctypes.c_void_p(streams[i].cuda_stream))
+        assert rc == 0, binding.crbm_last_error(ctxs[i].h)
+    torch.cuda.synchronize()
+    assert _side_by_side([lambda i=i: ctxs[i].autocorr(series[i], stream=streams[i]) for i in (0, 1)], 1000) == []
+    assert _side_by_side([lambda i=i: train(i) for i in (0, 1)], 300) == []
+    torch.cuda.synchronize()
+    for c, x, (tau, win), st in zip(ctxs, series, want, streams):
+        got = c.autocorr(x, stream=st)
+        np.testing.assert_array_equal(got[0], tau)
+        np.testing.assert_array_equal(got[1], win)
+    for c in ctxs:
+        c.close()
