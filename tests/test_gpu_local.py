@@ -198,3 +198,22 @@ def test_autocorr_rounds_match_oracle(ctx, n, cols, rho):
     t_ref, w_ref = autocorr.tau_int_columns(x)
     np.testing.assert_array_equal(win, w_ref)
     np.testing.assert_allclose(tau, t_ref, rtol=1e-9)
+
+
+@pytest.mark.parametrize("n", [40, 2500, 30721])
+def test_autocorr_short_and_long_windows_match_oracle(ctx, n):
+    """Windows that close in each round of 4, 4, 8, 16 and 32 lags (independent
+    steps to tau about 20), in shared memory and in chunks of a longer series, one
+    of them of a single step; tolerance as above."""
+    import torch
+    from oracle import autocorr
+    rho = np.array([0.0, 0.2, 0.45, 0.7, 0.8, 0.95])
+    x = np.random.default_rng(n).normal(size=(n, len(rho)))
+    for t in range(1, n):
+        x[t] += rho * x[t - 1]
+    tau, win = ctx.autocorr(torch.tensor(x, device="cuda:0"))
+    t_ref, w_ref = autocorr.tau_int_columns(x)
+    np.testing.assert_array_equal(win, w_ref)
+    np.testing.assert_allclose(tau, t_ref, rtol=1e-9)
+    if n > 100:
+        assert win[0] <= 4 < win[2] <= 8 < win[3] <= 16 < win[4] <= 32 < win[5]
