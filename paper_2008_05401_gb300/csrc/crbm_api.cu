@@ -47,7 +47,8 @@ struct Layout {
 
 struct Job {
   bool live = false;
-  int model = -1, kind = 0, L = 0, N = 0, Wd = 0, n = 0, nc = 1, tiles = 0;
+  int model = -1, kind = 0, L = 0, N = 0, Wd = 0, n = 0;
+  int nc[2] = {1, 1};   // Ising: chains per CTA, by precision (crbm_precision)
   int tpc = 0;   // Kitaev: threads of each chain's group (chains per CTA follow per launch)
   double J[3] = {1.0, 1.0, 1.0};
   uint64_t seed = 0, cid_base = 0, step = 0;
@@ -104,30 +105,41 @@ bool valid_L(int kind, int L) {
   return false;
 }
 
-// Chains per CTA of an Ising job of n chains (a Kitaev job's follow from its
-// group size per launch): a power of two in [1, 32], at most 16 units of 4 sites
-// a thread.  A proposal of a CTA takes about as long as its units per thread and
-// one more (barriers, reductions and the decision do not grow with its chains),
-// and an SM runs two CTAs side by side, so the choice minimises waves x (units
-// per thread + 1) among those that leave 1.5 CTAs or more for an SM.  40 mixed
-// proposals, K = 2, k = 5, against two units per thread whatever n: 1024 chains of
-// L = 24 822 -> 628 us, 4096 2734 -> 1742; 4096 of L = 12 1062 -> 741, of L = 30
-// 4152 -> 3897; one chain per CTA up to 1.5 chains an SM (100 FP64 proposals of 16
-// chains of L = 8: 8.1 ms in one CTA, 1.15 ms in 16).
-int chains_per_cta(const Model& m, int L, int n, int sms) {
+// Chains per CTA of an Ising job of n chains in a precision (a Kitaev job's follow
+// from its group size per launch): a power of two in [1, 32], at most 16 units of
+// 4 sites a thread.
+//   FP64: a proposal of a CTA takes about as long as its units per thread and one
+// more (barriers, reductions and the decision do not grow with its chains), and an
+// SM runs two CTAs side by side: the choice minimises waves x (units per thread +
+// 1) among those that leave 1.5 CTAs or more for an SM, the FP64 pipe's share of
+// them all (100 proposals of 16 chains of L = 8: 8.1 ms in one CTA, 1.15 ms in 16).
+//   Mixed: an SM takes its CTAs two at a time, and each pair its longest of a CTA's
+// chain of half-steps (u + 1/2 units) and the issue of both (0.08 units a warp and
+// unit, 0.16 a CTA).  Over L = 2 .. 30, 60 to 4000 chains and seven banks (913
+// cases) within 0.5 % of the best power of two on average, where the FP64 rule was
+// 17 % and up to 1.9 times off: 1300 chains of L = 5, K = 3, k = 3, 37 us a proposal
+// with it, 20 with this (and with two units a thread whatever n; 1024 chains of
+// L = 24, K = 2, k = 5: 31 then, 20 with either rule).
+int chains_per_cta(const Model& m, int prec, int L, int n, int sms) {
   const int nblk = (L * L + 3) / 4;
   int KC, kC;
   specialisation(m.kind, m.K, m.k, KC, kC);
   int best = 1;
-  long long best_t = 0;
+  double best_t = 0.0;
   for (int nc = 1; nc <= 32; nc *= 2) {
-    const long long tiles = ((long long)n + nc - 1) / nc;
-    if (nc > 1 && (nc * nblk > 16 * kThreads || 2 * tiles < 3LL * sms ||
+    const int tiles = (n + nc - 1) / nc, tpc = kThreads / nc, u = (nblk + tpc - 1) / tpc;
+    if (nc > 1 && (nc * nblk > 16 * kThreads || (prec == kFP64 && 2LL * tiles < 3LL * sms) ||
                    smem_bytes(m.kind, kMixed, L, m.K, m.k, nc, KC) > 100 * 1024))
       break;
-    const int tpc = kThreads / nc;
-    const long long t = (tiles + 2 * sms - 1) / (2 * sms) * ((nblk + tpc - 1) / tpc + 1);
-    if (nc == 1 || t < best_t) {
+    double t;
+    if (prec == kFP64) {
+      t = (double)((tiles + 2 * sms - 1) / (2 * sms)) * (u + 1);
+    } else {
+      const int warps = tpc >= 32 ? nc * ((std::min(nblk, tpc) + 31) / 32) : kThreads / 32, deep = (tiles + sms - 1) / sms;
+      const double alone = u + 0.5, issue = 0.08 * warps * u + 0.16;
+      t = (deep / 2) * std::max(alone, 2.0 * issue) + (deep % 2) * std::max(alone, issue);
+    }
+    if (nc == 1 || t < 0.999 * best_t) {
       best = nc;
       best_t = t;
     }
@@ -225,7 +237,7 @@ static JobDev make_jobdev(const crbm_ctx* ctx, const Job& j) {
   d.K = m.K;
   d.k = m.k;
   d.n_chains = j.n;
-  d.nc = j.nc;
+  d.nc64 = j.nc[kFP64];
   d.vb = m.vb;
   d.lc_edge = m.edge;
   d.ncls = m.ncls;
@@ -297,9 +309,9 @@ static JobDev make_jobdev(const crbm_ctx* ctx, const Job& j) {
 
 // Launch the fused kernel for a set of jobs (same kind and filter shape);
 // mode 1 = evaluate.  The threads of a chain's group (Ising: the job's chains
-// per 256-thread CTA; Kitaev: the job's group size) -- and so its per-chain
-// reduction order and every bit of its results -- depend only on the job, so
-// it gives the same results alone or batched.  A Kitaev launch takes CTAs of
+// per 256-thread CTA in that precision; Kitaev: the job's group size) -- and so its
+// per-chain reduction order and every bit of its results -- depend only on the job,
+// so it gives the same results alone or batched.  A Kitaev launch takes CTAs of
 // the largest group size among its jobs, each job as many chains per CTA as
 // its groups fill: small matrices alone run in small CTAs, a batch of mixed
 // sizes in one launch.  The jobs' tiles are laid out by decreasing lattice
@@ -340,9 +352,9 @@ static int launch_group(crbm_ctx* ctx, std::vector<int> ids, int S, int g, int c
     kind = j.kind;
     p.tile_begin[i] = tiles;
     p.job[i] = make_jobdev(ctx, j);
-    const int nc = kitaev ? nt / j.tpc : j.nc;
+    const int nc = kitaev ? nt / j.tpc : j.nc[prec];
     p.job[i].nc = nc;
-    tiles += kitaev ? (j.n + nc - 1) / nc : j.tiles;
+    tiles += (j.n + nc - 1) / nc;
     if (m.edge && prec != kFP64) return fail(ctx, CRBM_EINVAL, "LCRBM models run in CRBM_FP64 only");
     int KC, kC;
     specialisation(j.kind, m.K, m.k, KC, kC);
@@ -964,14 +976,16 @@ int crbm_init_chains(crbm_ctx* ctx, int model_id, int L, int n_chains, const dou
   j.N = L * L;
   j.Wd = (j.N + 31) / 32;
   j.n = n_chains;
-  j.nc = m.kind == kIsing ? chains_per_cta(m, L, n_chains, ctx->sms) : 1;
   if (m.kind == kKitaev) j.tpc = kitaev_group_threads(j.N);
+  else for (int prec : {kFP64, kMixed}) j.nc[prec] = chains_per_cta(m, prec, L, n_chains, ctx->sms);
   {
     // crbm_tune's choice: chains per CTA (Ising) or the group size (Kitaev)
     const auto it = ctx->tuned.find(std::make_tuple(m.kind, L, m.K, m.k));
-    if (it != ctx->tuned.end()) (m.kind == kKitaev ? j.tpc : j.nc) = it->second;
+    if (it != ctx->tuned.end()) {
+      if (m.kind == kKitaev) j.tpc = it->second;
+      else j.nc[kFP64] = j.nc[kMixed] = it->second;
+    }
   }
-  j.tiles = (n_chains + j.nc - 1) / j.nc;
   if (m.kind == kIsing) {
     j.J[0] = n_chains > 0 ? J[0] : 1.0;
   } else if (n_chains > 0) {
@@ -1415,14 +1429,8 @@ int crbm_tune(crbm_ctx* ctx, int model_id, int L, int precision, int* best_nc, d
   float best_t = 1e30f;
   for (int nc : cand) {
     Job& jj = ctx->jobs[id];
-    if (m.kind == kKitaev) {
-      jj.tpc = kThreads / nc;
-      jj.nc = 1;
-      jj.tiles = n_chains;
-    } else {
-      jj.nc = nc;
-      jj.tiles = (n_chains + nc - 1) / nc;
-    }
+    if (m.kind == kKitaev) jj.tpc = kThreads / nc;
+    else jj.nc[kFP64] = jj.nc[kMixed] = nc;
     if ((rc = launch_jobs(ctx, {id}, 0, 1, 1, kFP64, 1, ctx->own))) break;        // F, log pi of the state
     if ((rc = launch_jobs(ctx, {id}, 2, 1, 1, precision, 0, ctx->own))) break;    // warm-up
     cudaEventRecord(e0, ctx->own);

@@ -48,6 +48,7 @@ enum DevErr : int { kErrNone = 0, kErrConfig = 1, kErrTimeout = 2 };
 // parameters.  Pointers into the job's caller-owned device memory.
 struct JobDev {
   int kind, L, N, Wd, P, K, k, n_chains, nc;
+  int nc64;                     // chains per CTA of the FP64 path (Ising)
   int lc_edge;                  // > 0: LCRBM with lc_edge unshared kernels per side; lattice open along j
   int ncls;                     // kernel classes in the tables: 2 lc_edge + 1, or 1
   int nhex;                     // Kitaev hexagons: N, or L (L-1) with open columns

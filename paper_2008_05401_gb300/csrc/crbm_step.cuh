@@ -55,6 +55,40 @@ static __device__ __noinline__ void free_energy64(const JobDev& jb, const Grp& g
   *out = free_phase64(jb, jb.f64, g, v);
 }
 
+// F of a lattice by the threads of an FP64-path CTA and in their order of sums,
+// valid in thread 0.  Every thread of the CTA (256 or more) calls.
+static __device__ __noinline__ double path64_free(const JobDev& jb, const Grp& g, const uint32_t* v, double* scratch) {
+  Grp q = g;
+  q.r = (int)threadIdx.x;
+  q.tpc = kThreads / jb.nc64;
+  q.active = q.r < q.tpc;
+  FreeSum f = free_phase64(jb, jb.f64, q, v);
+  reduce_free<kFP64, false>(f, q, scratch);
+  return free_value<kFP64>(jb, f);
+}
+// An Ising CTA's chains with flag_rec == flag, one after the other (rare): F of
+// their proposals prop(i) as the FP64 path has it, and of the current lattices
+// cur(i) whose F carries a bound.  Ends with a barrier.
+template <class PROP, class CUR>
+__device__ __forceinline__ void ising_redo64(const JobDev& jb, const Grp& g, ChainSm* cs, int flag, double* scratch,
+                                             PROP prop, CUR cur) {
+  for (int i = 0; i < jb.nc; ++i) {
+    const bool redo = cs[i].Fb != 0.0;
+    if (cs[i].flag_rec != flag) continue;
+    const double Fp = path64_free(jb, g, prop(i), scratch), F = redo ? path64_free(jb, g, cur(i), scratch) : 0.0;
+    __syncthreads();                // every thread has read the chain's flags
+    if (threadIdx.x == 0) {
+      cs[i].Fp = Fp;
+      cs[i].Bp = 0.0;
+      if (redo) {
+        cs[i].F = F;
+        cs[i].Fb = 0.0;
+      }
+    }
+  }
+  __syncthreads();
+}
+
 // Observables of a lattice: Ising from E and the number of ones; Kitaev from
 // (e, c_f) of its spectrum and its count of hexagons with flux -1.
 template <int KIND>
@@ -356,21 +390,28 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         // FP64 free energies of y' and (when only its FP32 value is known) of x
         Grp g2 = g;
         g2.active = g.active && ch.flag_rec;
-        FreeSum f1;
-        free_energy64(jb, g2, vp, &f1);
-        reduce_free<kFP64, false>(f1, g2, scratch);
-        Grp g3 = g2;
-        g3.active = g2.active && ch.Fb != 0.0;
-        FreeSum f2;
-        free_energy64(jb, g3, h, &f2);
-        reduce_free<kFP64, false>(f2, g3, scratch);
-        if (g2.active && g.r == 0) {
-          ch.Fp = free_value<kFP64>(jb, f1);
-          ch.Bp = 0.0;
-          if (g3.active) {
-            ch.F = free_value<kFP64>(jb, f2);
-            ch.Fb = 0.0;
+        if constexpr (KIND == kIsing) {
+          ising_redo64(jb, g, cs, 1, scratch, [&](int i) { return planes + (size_t)i * (2 + K) * P + (vp - my); },
+                       [&](int i) { return planes + (size_t)i * (2 + K) * P + (h - my); });
+        } else {
+          FreeSum f1;
+          free_energy64(jb, g2, vp, &f1);
+          reduce_free<kFP64, false>(f1, g2, scratch);
+          Grp g3 = g2;
+          g3.active = g2.active && ch.Fb != 0.0;
+          FreeSum f2;
+          free_energy64(jb, g3, h, &f2);
+          reduce_free<kFP64, false>(f2, g3, scratch);
+          if (g2.active && g.r == 0) {
+            ch.Fp = free_value<kFP64>(jb, f1);
+            ch.Bp = 0.0;
+            if (g3.active) {
+              ch.F = free_value<kFP64>(jb, f2);
+              ch.Fb = 0.0;
+            }
           }
+        }
+        if (g2.active && g.r == 0) {
           const double loga = (ch.lpp - ch.lp) + (ch.Fp - ch.F);
           const uint4 w = philox4x32_10_rk(
               make_uint4(0u, kTagSwap, cycle, (uint32_t)(xj.cid_base + (uint64_t)g.c)), xj.rk);
@@ -695,32 +736,32 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
         // the FP64 path's free energies of v' (and of v when only its FP32
         // value is known), computed by the same code and reduction order
         // (tables from global memory: the mixed kernel keeps only FP32 ones)
-        Grp g4 = g2;
-        g4.active = g2.active && (KIND == kKitaev || ch.flag_rec == 2);
-        FreeSum f1;
-        free_energy64(jb, g4, vp, &f1);
-        loop_reduce(f1, g4, std::integral_constant<int, kFP64>());
-        Grp g3 = g4;
-        g3.active = g4.active && ch.Fb != 0.0;
-        FreeSum f2;
-        free_energy64(jb, g3, v, &f2);
-        loop_reduce(f2, g3, std::integral_constant<int, kFP64>());
-        // Kitaev: the FP64 eigen-stage of v' (and of v when its log-weight
-        // came from the df64 stage), by the group that needs it
-        double k1v[3] = {0.0, 0.0, 0.0}, k0v[3] = {0.0, 0.0, 0.0};
-        const bool redo_v = ch.lpb != 0.0;
-        if (KIND == kKitaev) {
+        if constexpr (KIND == kIsing) {
+          ising_redo64(jb, g, cs, 2, scratch,
+                       [&](int i) { return planes + (size_t)i * (2 + K) * P + (cs[i].cur ^ 1) * P; },
+                       [&](int i) { return planes + (size_t)i * (2 + K) * P + cs[i].cur * P; });
+        } else {
+          FreeSum f1;
+          free_energy64(jb, g2, vp, &f1);
+          loop_reduce(f1, g2, std::integral_constant<int, kFP64>());
+          Grp g3 = g2;
+          g3.active = g2.active && ch.Fb != 0.0;
+          FreeSum f2;
+          free_energy64(jb, g3, v, &f2);
+          loop_reduce(f2, g3, std::integral_constant<int, kFP64>());
+          // the FP64 eigen-stage of v' (and of v when its log-weight came from
+          // the df64 stage), by the group that needs it
+          double k1v[3] = {0.0, 0.0, 0.0}, k0v[3] = {0.0, 0.0, 0.0};
+          const bool redo_v = ch.lpb != 0.0;
           fp64_spectrum<PREC, MULTI>(jb, g, vp, ch.beta, wk, k1v, nullptr);
           if (redo_v) fp64_spectrum<PREC, MULTI>(jb, g, v, ch.beta, wk, k0v, nullptr);
-        }
-        if (g4.active && g.r == 0) {
-          ch.Fp = free_value<kFP64>(jb, f1);
-          ch.Bp = 0.0;
-          if (g3.active) {
-            ch.F = free_value<kFP64>(jb, f2);
-            ch.Fb = 0.0;
-          }
-          if (KIND == kKitaev) {
+          if (mine) {
+            ch.Fp = free_value<kFP64>(jb, f1);
+            ch.Bp = 0.0;
+            if (g3.active) {
+              ch.F = free_value<kFP64>(jb, f2);
+              ch.Fb = 0.0;
+            }
             ch.lpp = k1v[0];
             ch.lppb = 0.0;
             ch.Ep = k1v[1];
@@ -729,10 +770,11 @@ __global__ void __launch_bounds__(NT, CRBM_MIN_BLOCKS * 256 / NT) crbm_step_kern
               ch.lp = k0v[0];
               ch.lpb = 0.0;
             }
+            ch.rec_mh += 1ull;      // Ising: counted at the df64 level
           }
-          ch.flag_acc = log_u64(step) < (ch.lpp - ch.lp) + (ch.Fp - ch.F);
-          if (KIND == kKitaev) ch.rec_mh += 1ull;   // Ising: counted at the df64 level
         }
+        if (mine && (KIND == kKitaev || ch.flag_rec == 2))
+          ch.flag_acc = log_u64(step) < (ch.lpp - ch.lp) + (ch.Fp - ch.F);
       }
       if (mine && ch.flag_acc) ch.cur ^= 1;
       loop_sync();

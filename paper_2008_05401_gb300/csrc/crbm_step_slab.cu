@@ -212,14 +212,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_cons
           if (owner != rank) lattice[w] = cl.map_shared_rank(lattice, owner)[w];
         }
         __syncthreads();
-        Grp g64 = g;
-        g64.tpc = kThreads / jb.nc;
-        g64.active = tid < g64.tpc;
-        FreeSum f;
-        free_energy64(jb, g64, lattice, &f);
-        reduce_free<kFP64, false>(f, g64, scratch);
-        mine.d[0] = f.s;
-        mine.d[2] = (double)f.ones;
+        mine.d[0] = -path64_free(jb, g, lattice, scratch);       // F = -v_bias d[2] - d[0]
         return mine;
       };
       const bool redo_v = ch.Fb != 0.0;

@@ -209,6 +209,8 @@ def test_divided_chains_in_a_batch_and_a_graph(ctx):
     ("ising", 24, 2, 5, 40, 1e12),
     ("ising", 96, 2, 5, 12, 1e12),
     ("ising", 64, 8, 3, 40, 1e12),
+    ("ising", 5, 3, 3, 1300, 1e12),   # other chains per CTA in FP64 than in mixed precision
+    ("ising", 2, 8, 2, 701, 1e12),
 ])
 def test_large_free_energies_keep_the_decisions(ctx, model, L, K, k, n, hb):
     """Filters whose free energy passes any fixed range of the mixed path's sums:

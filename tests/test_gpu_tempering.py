@@ -162,6 +162,28 @@ def test_pt_after_proposals_reevaluates(ctx):
     jy.release()
 
 
+@pytest.mark.parametrize("L,K,k,n,hb", [(5, 3, 3, 1300, 1e12), (24, 2, 5, 40, 1e12), (8, 2, 3, 60, 3e7)])
+def test_pt_swaps_of_large_free_energies_are_the_fp64_path_s(ctx, L, K, k, n, hb):
+    """F past any fixed range of the mixed path's sums, and of an FP64 rounding as
+    large as the swaps' log ratios: the mixed swaps are those of the FP64 path,
+    whose CTAs hold other numbers of chains."""
+    from paper_2008_05401_gb300 import FP64, ISING, MIXED
+    W, _, vb = wl.gaussian_crbm(K, k, 1.0 / (L * k), seed=L * 10 + K)
+    mid = ctx.load_model(ISING, W, vb, np.full(K, hb))
+    T = L * wl.ising_ladder(n, 8)
+    got = []
+    for prec in (FP64, MIXED):
+        jx, jy = (ctx.new_job(mid, ISING, L, T, (1.0,), SEED_X + i, i * n, wl.pack_bits(wl.random_lattices(n, L, seed=L + i)),
+                              prec) for i in (0, 1))
+        ctx.pt_run(jx, jy, 3, precision=prec)
+        got.append((jx.state()[0], jy.state()[0], jx.observables()[1]))
+        jx.release()
+        jy.release()
+    assert got[0][2].sum() > 0
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
+
+
 def test_pt_rejects_mismatched_jobs(ctx):
     import paper_2008_05401_gb300 as P
     from paper_2008_05401_gb300 import CrbmError
