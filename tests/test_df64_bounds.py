@@ -206,3 +206,53 @@ def test_df_sqrt_and_reciprocal_bound():
         e = fma(-a[1], y, fma(-a[0], y, Fr(1)))
         q = fast_two_sum(y, mul(y, e))
         assert abs(val(q) * val(a) - 1) <= Fr(1, 2 ** 44)
+
+
+def df_neg(a):
+    return (-a[0], -a[1])
+
+
+def df_sqrt_fast(a, y):
+    """The device's square root from y near a^-1/2, and its value before the last correction."""
+    half = mul(Fr(1, 2), y)
+    h = mul(a[0], y)
+    h = fma(fma(-h, h, a[0]), half, h)
+    q = fast_two_sum(h, mul(add(fma(-h, h, a[0]), a[1]), half))
+    return fast_two_sum(q[0], fma(df_fma(df_neg(q), q, a)[0], half, q[1])), q
+
+
+def df_rcp_fast(a, y):
+    """The device's reciprocal from y near 1 / a, and its value before the last correction."""
+    y = fma(y, fma(-a[0], y, Fr(1)), y)
+    q = fast_two_sum(y, mul(y, fma(-a[1], y, fma(-a[0], y, Fr(1)))))
+    return fast_two_sum(q[0], fma(df_fma(df_neg(a), q, (Fr(1), Fr(0)))[0], y, q[1])), q
+
+
+def test_df_sqrt_and_reciprocal_reach_the_spacing():
+    """With the last correction, from approximations within 2^-22: the high parts
+    of its residual cancel exactly (Sterbenz); its three FP32 operations have values
+    below 2, 3 and 4 2^-24 of the operand and round by 2^-24 of that, and the product
+    of low parts is dropped: 10 2^-48 (6 2^-48 for the reciprocal, whose 1 has no low
+    part).  The square root is off by half of it, and the correction's addition rounds
+    by 2^-48: 6 2^-48 and 7 2^-48 relative.  That the correction is one: on average
+    the values before it are further off, those with it taken the wrong way further still."""
+    rng = random.Random(72)
+    bound = {"sqrt": Fr(6, 2 ** 48), "rcp": Fr(7, 2 ** 48)}
+    mean = {}
+    for n in range(N_CASES):
+        a = rand_df(rng, scale=2.0)
+        if val(a) <= 0:
+            a = df_neg(a)
+        if a[0] == 0:
+            continue
+        off = 1 + Fr(1, 2 ** 22) * Fr(1 if n % 3 == 0 else -1 if n % 3 == 1 else rng.uniform(-1.0, 1.0))
+        for name, (x, q), err in (
+                ("sqrt", df_sqrt_fast(a, f32(Fr(float(a[0]) ** -0.5) * off)), lambda v: (val(v) ** 2 / val(a) - 1) / 2),
+                ("rcp", df_rcp_fast(a, f32(1 / a[0] * off)), lambda v: val(v) * val(a) - 1)):
+            assert abs(err(x)) <= bound[name]
+            wrong = (q[0], q[1] - (val(x) - val(q)))
+            sums = mean.setdefault(name, [0.0, 0.0, 0.0])
+            for i, v in enumerate((x, q, wrong)):
+                sums[i] += abs(float(err(v))) / N_CASES
+    for name, (done, before, wrong) in mean.items():
+        assert done < 0.8 * before and wrong > 1.2 * before, (name, done, before, wrong)
