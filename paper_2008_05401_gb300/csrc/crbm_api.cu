@@ -507,9 +507,9 @@ static int launch_jobs(crbm_ctx* ctx, const std::vector<int>& ids, int S, int g,
   const int slab = partner ? 0 : slab_size(ctx, ids, prec, mode);
   auto part_of = [&](const Job& j) {
     if (slab > 0) return -2;
-    return !partner && on_tc(ctx, j, prec, mode) ? -1 : threads_for(j.kind, j.N);
+    return !partner && on_tc(ctx, j, prec, mode) ? -1 : kThreads;
   };
-  for (int nt : {-2, -1, 256}) {
+  for (int nt : {-2, -1, kThreads}) {
     std::vector<int> part;
     for (int id : ids)
       if (ctx->jobs[id].n > 0 && part_of(ctx->jobs[id]) == nt) part.push_back(id);

@@ -310,11 +310,7 @@ __device__ __forceinline__ void decide32_split(float x, uint32_t w, float c0, fl
   amb = fabsf(d) > delta ? 0u : 1u;
 }
 
-// log(1 + e^x) without overflow.
-__device__ __forceinline__ double softplus64(double x) {
-  return fmax(x, 0.0) + log1p(exp(-fabs(x)));
-}
-// FP32: max(x, 0) + ln 2 * log2(1 + 2^(-|x| log2 e)).
+// log(1 + e^x) in FP32 without overflow: max(x, 0) + ln 2 * log2(1 + 2^(-|x| log2 e)).
 __device__ __forceinline__ float softplus32(float x) {
   const float e = ex2_approx(fabsf(x) * -1.4426950408889634f);
   return fmaxf(x, 0.0f) + 0.69314718055994531f * lg2_approx(1.0f + e);

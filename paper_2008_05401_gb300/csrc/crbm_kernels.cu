@@ -81,8 +81,7 @@ void specialisation(int kind, int K, int k, int& KC, int& kC) {
 // group of its own (kitaev_group_threads or its tuned size); a launch of
 // Kitaev jobs takes CTAs of the largest group size among them, so jobs of
 // every lattice side share one launch, several small chains per CTA.
-int threads_for(int, int) { return 256; }
-
+//
 // Threads of a Kitaev chain's group, measured on the Kitaev workloads when
 // they were CTA sizes: 32 up to 16 cells, 64 up to 64, 128 up to 100 and 256
 // above (the reduction's per-column barriers cost less in small groups).
