@@ -127,15 +127,17 @@ int chains_per_cta(const Model& m, int prec, int L, int n, int sms) {
   int best = 1;
   double best_t = 0.0;
   for (int nc = 1; nc <= 32; nc *= 2) {
-    const int tiles = (n + nc - 1) / nc, tpc = kThreads / nc, u = (nblk + tpc - 1) / tpc;
-    if (nc > 1 && (nc * nblk > 16 * kThreads || (prec == kFP64 && 2LL * tiles < 3LL * sms) ||
+    const long long tiles = ((long long)n + nc - 1) / nc;
+    const int tpc = kThreads / nc, u = (nblk + tpc - 1) / tpc;
+    if (nc > 1 && (nc * nblk > 16 * kThreads || (prec == kFP64 && 2 * tiles < 3LL * sms) ||
                    smem_bytes(m.kind, kMixed, L, m.K, m.k, nc, KC) > 100 * 1024))
       break;
     double t;
     if (prec == kFP64) {
       t = (double)((tiles + 2 * sms - 1) / (2 * sms)) * (u + 1);
     } else {
-      const int warps = tpc >= 32 ? nc * ((std::min(nblk, tpc) + 31) / 32) : kThreads / 32, deep = (tiles + sms - 1) / sms;
+      const int warps = tpc >= 32 ? nc * ((std::min(nblk, tpc) + 31) / 32) : kThreads / 32;
+      const long long deep = (tiles + sms - 1) / sms;
       const double alone = u + 0.5, issue = 0.08 * warps * u + 0.16;
       t = (deep / 2) * std::max(alone, 2.0 * issue) + (deep % 2) * std::max(alone, issue);
     }

@@ -1319,10 +1319,11 @@ __device__ __forceinline__ void group_thermal(double& lp, double& en, double& cf
 
 // Couplings scaled by a power of two so that the largest lies in [1, 2) (exact,
 // undone at the end): FP32 helpers then never run out of exponents.  M's
-// entries are the 2 J.
+// entries are the 2 J.  (Subnormal J: the least normal exponent, whose inverse
+// times 2 is finite.)
 __device__ __forceinline__ int coupling_exponent(const double* J) {
   const double m = fmax(fabs(J[0]), fmax(fabs(J[1]), fabs(J[2])));
-  return m > 0.0 ? ((__double2hiint(m) >> 20) & 0x7ff) - 1023 : 0;
+  return m > 0.0 ? max((__double2hiint(m) >> 20) & 0x7ff, 1) - 1023 : 0;
 }
 
 // One single-fermion level's share of log pi, e and c_f (Sec. IV):

@@ -313,6 +313,26 @@ def test_kitaev_degenerate_couplings_match_oracle(ctx, L, J):
         job.release()
 
 
+@pytest.mark.parametrize("scale", [1e-310, 1e-160, 1e-40])
+def test_kitaev_tiny_couplings_match_oracle(ctx, scale):
+    """Couplings far below the temperatures, down to subnormal numbers: every
+    level's share of log pi is log 2 to rounding, in both precisions."""
+    from paper_2008_05401_gb300 import FP64, KITAEV, MIXED
+    W, hb, vb = wl.gaussian_crbm(2, 3, 0.05, seed=3)
+    n, S, L, J = 12, 2, 4, (3 * scale, scale, 2 * scale)
+    T = wl.kitaev_ladder(n, 12)
+    bits0 = wl.pack_bits(wl.random_lattices(n, L, seed=L))
+    ref = oracle_chains("kitaev", W, hb, vb, L, T, J, SEED, n, bits0)
+    worst = run_oracle(ref, S)
+    mid = ctx.load_model(KITAEV, W, vb, hb)
+    for prec in (FP64, MIXED):
+        job = ctx.new_job(mid, KITAEV, L, T, J, SEED, 0, bits0, prec)
+        job.run(S, precision=prec)
+        np.testing.assert_allclose(job.energies()[0], L * L * np.log(2.0), rtol=1e-12)
+        _compare(job, ref, worst, S)
+        job.release()
+
+
 def test_random_init_matches_oracle(ctx):
     """init = 0 draws the lattices from the stream's init tag on the device."""
     from oracle import chain
