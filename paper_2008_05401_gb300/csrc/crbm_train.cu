@@ -20,13 +20,13 @@
 // pipe for about 64 cycles on GB300) and the serial chain of a step.  Hence:
 //   - the sum of log(1 + e^-|x|) of a warp's units is the log of their product:
 //     two operations per unit (join_log1p) instead of a log1p;
-//   - the gradient's sums over sites are exact 128-bit fixed-point additions of
+//   - the gradient's sums over sites are exact 96-bit fixed-point additions of
 //     the FP64 sigma(a) off the FP64 pipe (WideSum), in FP64 for samples with a
 //     unit below their range;
 //   - the bias corrections 1 / (1 - b^t) are taken for 32 steps at a time, one
 //     step per lane (a pow per thread and step was a third of the epoch);
 //   - the next minibatch's samples and targets are fetched during a step.
-// K = 2 5x5, L = 8, 10^4 samples, batch 20: 24 problems 9.8 ms per epoch
+// K = 2 5x5, L = 8, 10^4 samples, batch 20: 24 problems 9.4 ms per epoch
 // (one 512-thread CTA per problem, log1p and pow per unit and thread, FP64
 // gradient sums: 69.3 ms).
 #include <algorithm>
@@ -109,28 +109,24 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src) {
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Exact sum of up to 1024 FP64 values in [kWideMin, 1]: 128-bit fixed point in
-// units of 2^-116, so every bit of every value counts whatever the others' size.
-// About 20 integer instructions an addition, where an FP64 one holds the pipe for
-// 64 cycles (epoch of 24 problems, K = 2 5x5, L = 8: 9.6 ms, 12.0 with FP64 sums).
-constexpr int kWideMinHi = (1023 - 63) << 20;      // high word of 2^-63
+// Exact sum of up to 1024 FP64 values in [kWideMin, 1]: 96-bit fixed point in
+// units of 2^-84, so every bit of every value counts whatever the others' size.  Ten
+// integer instructions an addition, where an FP64 one holds the pipe for 64 cycles
+// (epoch of 24 problems, K = 2 5x5, L = 8: 9.4 ms, about 12 with FP64 sums).
+constexpr int kWideMinHi = (1023 - 31) << 20;      // high word of 2^-31
 struct WideSum {
-  uint32_t w0 = 0u, w1 = 0u, w2 = 0u, w3 = 0u;
-  // adds x where mask is all ones, nothing where it is 0
-  __device__ __forceinline__ void add(double x, uint32_t mask) {
-    // the 53-bit mantissa, 64 zero bits below it, shifted down by 0 <= sh <= 63
-    const uint32_t xh = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x) & mask;
-    const uint32_t sh = 1023u - (xh >> 20), hi = ((xh & 0xFFFFFu) | 0x100000u) & mask;
-    const bool far = sh >= 32u;
-    const uint32_t t3 = far ? 0u : hi, t2 = far ? hi : lo, t1 = far ? lo : 0u;
-    asm("{\nadd.cc.u32 %0, %0, %4;\naddc.cc.u32 %1, %1, %5;\naddc.cc.u32 %2, %2, %6;\naddc.u32 %3, %3, %7;\n}\n"
-        : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3)
-        : "r"(__funnelshift_r(0u, t1, sh)), "r"(__funnelshift_r(t1, t2, sh)), "r"(__funnelshift_r(t2, t3, sh)),
-          "r"(__funnelshift_r(t3, 0u, sh)));
+  uint32_t w1 = 0u, w2 = 0u, w3 = 0u;
+  // adds x if on != 0
+  __device__ __forceinline__ void add(double x, uint32_t on) {
+    // the 53-bit mantissa, 32 zero bits below it, shifted down by 0 <= sh <= 31
+    const uint32_t xh = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t sh = 1023u - (xh >> 20), hi = (xh & 0xFFFFFu) | 0x100000u;
+    asm("{\n.reg .pred p;\nsetp.ne.u32 p, %6, 0;\n@p add.cc.u32 %0, %0, %3;\n@p addc.cc.u32 %1, %1, %4;\n@p addc.u32 %2, %2, %5;\n}\n"
+        : "+r"(w1), "+r"(w2), "+r"(w3)
+        : "r"(__funnelshift_r(0u, lo, sh)), "r"(__funnelshift_r(lo, hi, sh)), "r"(hi >> (sh & 31u)), "r"(on));
   }
   __device__ __forceinline__ double value() const {
-    const double hi = (double)(((unsigned long long)w3 << 32) | w2), lo = (double)(((unsigned long long)w1 << 32) | w0);
-    return fma(hi, 0x1p-52, lo * 0x1p-116);
+    return fma((double)(((unsigned long long)w3 << 32) | w2), 0x1p-52, (double)w1 * 0x1p-84);
   }
 };
 
@@ -212,7 +208,7 @@ __device__ __forceinline__ double site_sum(const double* sp, int L, int s0, int 
     const uint32_t win = row(si);
     if (exact) {
 #pragma unroll 8
-      for (int j = 0; j < L; ++j) wide.add(x[j], 0u - ((win >> j) & 1u));
+      for (int j = 0; j < L; ++j) wide.add(x[j], win & (1u << j));
     } else {
       double part = 0.0;
       for (int j = 0; j < L; ++j)

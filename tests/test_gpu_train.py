@@ -167,6 +167,7 @@ def test_cluster_split_matches_oracle(ctx, n_problems, K, k, L, n, batch):
 
 
 @pytest.mark.parametrize("L,k,hb,vb,spread", [(8, 3, (0.0, -25.0), 0.1, 3.0), (8, 3, (0.0, -40.0), 0.1, 3.0),
+                                                 (8, 3, (0.0, -20.0), 0.1, 3.0), (16, 3, (0.0, -21.5), 0.1, 3.0),   # on either side of 2^-31
                                                  (17, 2, (0.5, -60.0), 0.1, 3.0),
                                                  (8, 3, (25.0, -40.0), 0.1, 3.0), (17, 2, (60.0, 1.0), 0.1, 3.0),
                                                  (8, 3, (-30.0, -35.0), 0.0, 0.0),     # F itself that small
