@@ -62,6 +62,19 @@ __device__ __forceinline__ SlabSum cluster_sum(cg::cluster_group& cl, SlabSum mi
   return x;
 }
 
+// F of a lattice whose rows the cluster's CTAs hold, as the FP64 path has it, by
+// every CTA on its own copy (out of line: rare).
+__device__ __noinline__ double whole_free64(const JobDev& jb, const Grp& g, uint32_t* lattice, double* scratch) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank(), WL = jb.L >> 5;
+  for (int w = threadIdx.x; w < jb.Wd; w += kSlabThreads) {
+    const int owner = ((w / WL + 1) * CL - 1) / jb.L;
+    if (owner != rank) lattice[w] = cl.map_shared_rank(lattice, owner)[w];
+  }
+  __syncthreads();
+  return path64_free(jb, g, lattice, scratch);
+}
+
 template <int KC, int kC>
 __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_constant__ LaunchParams prm) {
   cg::cluster_group cl = cg::this_cluster();
@@ -207,12 +220,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_cons
           grp_reduce<3>(mine.d, g, scratch);
           return cluster_sum(cl, mine, slots, turn);
         }
-        for (int w = tid; w < Wd; w += kSlabThreads) {
-          const int owner = ((w / WL + 1) * CL - 1) / L;
-          if (owner != rank) lattice[w] = cl.map_shared_rank(lattice, owner)[w];
-        }
-        __syncthreads();
-        mine.d[0] = -path64_free(jb, g, lattice, scratch);       // F = -v_bias d[2] - d[0]
+        mine.d[0] = -whole_free64(jb, g, lattice, scratch);      // F = -v_bias d[2] - d[0]
         return mine;
       };
       const bool redo_v = ch.Fb != 0.0;
