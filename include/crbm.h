@@ -62,9 +62,13 @@ typedef enum { CRBM_ISING = 0, CRBM_KITAEV = 1 } crbm_model_kind;
 
 /* CRBM_FP64: every pre-activation, probability, free energy and decision in
  * FP64.  CRBM_MIXED: FP32 pre-activations (hi/lo split filters), FP32
- * sigmoid/softplus with FP64 accumulation; every Bernoulli or accept/reject
- * decision that lies within the FP32 error bound of its threshold is redone
- * with the FP64 code, so the chain takes exactly the FP64 path's decisions. */
+ * sigmoid/softplus whose per-thread sums are added as integers; every Bernoulli
+ * or accept/reject decision that lies within the FP32 error bound of its
+ * threshold is redone with the FP64 code, so the chain takes exactly the FP64
+ * path's decisions.  A chain's FP64 sums are taken by its threads, whose number
+ * depends on the job (side, chain count, filters, the device's SMs, crbm_tune):
+ * the same lattice in a job of another chain count has the same F to FP64
+ * rounding, not always to the last bit. */
 typedef enum { CRBM_FP64 = 0, CRBM_MIXED = 1 } crbm_precision;
 
 /* Per-chain observable sums (crbm_read_observables), CRBM_NOBS per chain:
@@ -109,7 +113,9 @@ CRBM_API int crbm_load_model(crbm_ctx* ctx, int kind, int K, int k, const double
  * unit (f, i, j) of class c to visible unit ((i+a) mod L, j+b).  Hidden biases
  * (K) and the visible bias are shared.  Jobs of this model simulate the
  * open-boundary Kitaev model (vison density over the L (L-1) hexagons that do
- * not cross the cut) and run in CRBM_FP64 only.
+ * not cross the cut) and run in CRBM_FP64 only.  Known limit: where edge modes
+ * form pairs closer than FP32 separates, log pi and e of a lattice can be off by
+ * up to 1e-5 of their size (the periodic model's spectra are certified).
  * Errors: CRBM_EINVAL (kind not Kitaev, edge outside [1, 6],
  * (2 edge + 1) K k 2^k > 4096), CRBM_ECUDA. */
 CRBM_API int crbm_load_lcrbm(crbm_ctx* ctx, int kind, int K, int k, int edge, const double* W, double v_bias,

@@ -12,7 +12,7 @@
 // quarter of the series, a register accumulator per lag, so that the FP64
 // additions that bring a round's sums together are 16 for each 16 n / 128
 // multiply-adds of a warp instead of a block sum per lag.  1024 series of
-// 2000 steps, W about 140: 1.05 ms with the copies (one lag at a time: 6.5 ms).
+// 2000 steps, W about 140: 1.03 ms with the copies (one lag at a time: 6.5 ms).
 #include <mutex>
 
 #include "crbm.h"

@@ -112,7 +112,7 @@ bool valid_L(int kind, int L) {
 // more (barriers, reductions and the decision do not grow with its chains), and an
 // SM runs two CTAs side by side: the choice minimises waves x (units per thread +
 // 1) among those that leave 1.5 CTAs or more for an SM, the FP64 pipe's share of
-// them all (100 proposals of 16 chains of L = 8: 8.1 ms in one CTA, 1.15 ms in 16).
+// them all (100 proposals of 16 chains of L = 8: 8.1 ms in one CTA, 1.17 ms in 16).
 //   Mixed: an SM takes its CTAs two at a time, and each pair its longest of a CTA's
 // chain of half-steps (u + 1/2 units) and the issue of both (0.08 units a warp and
 // unit, 0.16 a CTA).  Over L = 2 .. 30, 60 to 4000 chains and seven banks (913

@@ -8,8 +8,9 @@
 // in single lattices.  Chains are continued and compared by these values, so
 // the arithmetic of this stage -- its operations, their order, the sums over the
 // group -- is kept to the bit; kitaev_logpi64 (periodic lattices), whose
-// eigenvalues are certified, has no such error and takes two thirds of the
-// time, but gives other values on these lattices.
+// eigenvalues are certified, has no such error and would take less time (four
+// proposals of 1024 chains of L = 8: 4.7 ms instead of 8.3), but gives other
+// values on these lattices: the right ones.
 #pragma once
 #include "crbm_device.cuh"
 

@@ -14,9 +14,9 @@
 // the phase writing them.  The CTAs' sums are added in rank order by every CTA,
 // so each takes the same decision and keeps the chain's values itself.
 // Three cluster barriers per proposal of one Gibbs step; the rest is bound by
-// instruction issue like the table kernel (53 % of the slots).  16 chains of
-// L = 256, K = 4 5x5, 40 proposals and the read-back: 1.75 ms (one CTA per chain:
-// 12.5 ms).
+// instruction issue like the table kernel (59 % of the slots).  16 chains of
+// L = 256, K = 4 5x5, 40 proposals and the read-back, in clusters of six: 1.74 ms
+// (one CTA per chain: 12.5 ms).
 #include <algorithm>
 
 #include <cooperative_groups.h>
